@@ -257,6 +257,18 @@ int normpre_newton_schulz(const normpre_config* cfg, int batch, int64_t rows, in
                           const void* X, void* T, void* stream);
 
 /*
+ * The same in a workspace of the caller's, without allocating: device memory
+ * of at least the size that normpre_newton_schulz_workspace reports (16-byte
+ * aligned, contents undefined before and after), used by this call alone until
+ * it returns (it synchronizes `stream` too).
+ * Errors: as normpre_newton_schulz, and ARG for a workspace that is too small.
+ */
+int normpre_newton_schulz_workspace(const normpre_config* cfg, int batch, int64_t rows, int64_t cols,
+                                    int64_t* bytes);
+int normpre_newton_schulz_ws(const normpre_config* cfg, int batch, int64_t rows, int64_t cols, const void* X, void* T,
+                             void* workspace, int64_t workspace_bytes, void* stream);
+
+/*
  * The Gaussian sketch matrix of one matrix and step (Algorithm 2, "sample
  * Omega"), computed by the kernel the NormPre-L step uses, with the random
  * stream it draws from written out for checking:

@@ -181,13 +181,25 @@ struct NSGroupBuf {
   size_t elem = 2;              // element size of X, A, B
 };
 
+// Buffers of a plan that allocates nothing (the stand-alone call).
+struct NSExternal {
+  void* ws = nullptr;           // NSPlan::workspace_bytes() of device memory
+  int steps = 0;
+  void* x_in = nullptr;         // optional: the caller's X as X[0] / T as X[out_index(steps)],
+  void* x_out = nullptr;        // for matrices without padding
+};
+constexpr int kNsCopyCtas = 512;  // most CTAs per matrix of the load / store passes
+
 class NSPlan {
  public:
   NSPlan() = default;
   ~NSPlan();
   // Allocates the buffers of every group and prepares launch descriptors.
   // bf16 = true: tcgen05 tensor-core path; false: fp32 SIMT path.
-  cudaError_t init(bool bf16, const std::vector<NSGroupSpec>& groups, std::string* err);
+  // With ext, of one group: in the caller's workspace instead.
+  cudaError_t init(bool bf16, const std::vector<NSGroupSpec>& groups, std::string* err,
+                   const NSExternal* ext = nullptr);
+  static size_t workspace_bytes(bool bf16, const NSGroupSpec& spec);
   // q iterations of X <- aX + (b A + c A^2) X on X[0] of groups
   // [g0, g0 + cnt) (cnt < 0: every group from g0) -- with cnt = 1, of its
   // matrices [m0, m1) (m1 < 0: to the last) -- with X[0] scaled by inscale[]
@@ -201,8 +213,11 @@ class NSPlan {
   cudaError_t scale_from_count(const int* count, const int* const* group_mat_ids, float eps,
                                cudaStream_t s, ProfileHook* prof = nullptr, int g0 = 0, int cnt = -1,
                                int m0 = 0, int m1 = -1);
-  // Computes inscale[] = 1/(||X0||_F + eps) directly from X[0].
-  cudaError_t scale_from_norm(float eps, cudaStream_t s);
+  // Stand-alone call (one group): X [batch][rows][cols] into X[0] (padded)
+  // and inscale[] = 1/(||X||_F + eps), with part [batch][kNsCopyCtas] for the
+  // partial sums; and the result of `steps` iterations into T.
+  cudaError_t load(const void* X, double* part, float eps, cudaStream_t s);
+  cudaError_t store(void* T, int steps, cudaStream_t s);
   static int out_index(int steps) { return (steps % 2 == 1) ? 1 : 2; }
   std::vector<NSGroupBuf>& groups() { return groups_; }
   bool bf16() const { return bf16_; }

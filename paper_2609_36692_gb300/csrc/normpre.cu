@@ -894,44 +894,95 @@ int normpre_read(normpre_handle* h, int mat, int what, void* dst, int64_t capaci
   return NORMPRE_OK;
 }
 
-int normpre_newton_schulz(const normpre_config* cfg, int batch, int64_t rows, int64_t cols, const void* X, void* T,
-                          void* stream) {
-  if (!cfg || !X || !T) return fail(nullptr, NORMPRE_ERR_ARG, "null argument");
+namespace {
+
+// Arguments of the stand-alone Newton-Schulz calls (X and T null: sizes only).
+int check_ns(const normpre_config* cfg, int batch, int64_t rows, int64_t cols) {
   if (batch < 1) return fail(nullptr, NORMPRE_ERR_ARG, "batch must be >= 1");
   if (rows < 1 || cols < 1 || rows > 65536 || cols > 65536) return fail(nullptr, NORMPRE_ERR_SHAPE, "dimensions must be in [1, 65536]");
   if (cfg->ns_steps < 1 || cfg->ns_steps > 100) return fail(nullptr, NORMPRE_ERR_ARG, "ns_steps must be in [1, 100]");
   if (cfg->precision != NORMPRE_PREC_BF16 && cfg->precision != NORMPRE_PREC_F32) return fail(nullptr, NORMPRE_ERR_ARG, "bad precision");
-  if (!aligned16(X) || !aligned16(T)) return fail(nullptr, NORMPRE_ERR_ALIGN, "X and T must be 16-byte aligned");
+  return NORMPRE_OK;
+}
+// Workspace: the status word, the partial sums of ||X||^2, the plan's buffers.
+constexpr size_t kNsFlagBytes = 256;
+size_t ns_part_bytes(int batch) { return static_cast<size_t>(batch) * kNsCopyCtas * sizeof(double); }
+
+int newton_schulz_impl(const normpre_config* cfg, int batch, int64_t rows, int64_t cols, const void* X, void* T,
+                       void* ws, void* stream) {
   const bool bf = cfg->precision == NORMPRE_PREC_BF16;
-  const size_t el = bf ? 2 : 4;
+  const NSGroupSpec spec{batch, rows, cols};
   cudaStream_t s = static_cast<cudaStream_t>(stream);
+  NSExternal ext;
+  int* flags = static_cast<int*>(ws);
+  double* part = reinterpret_cast<double*>(static_cast<char*>(ws) + kNsFlagBytes);
+  ext.ws = reinterpret_cast<char*>(part) + ns_part_bytes(batch);
+  ext.steps = cfg->ns_steps;
+  // Matrices that fill their padded buffers are read and written where they
+  // are, unless the result overlaps the input, which every iteration's first
+  // product still reads
+  const int64_t fill = bf ? 256 : 64;
+  const size_t bytes = static_cast<size_t>(batch) * rows * cols * (bf ? 2 : 4);
+  const uintptr_t x0 = reinterpret_cast<uintptr_t>(X), t0 = reinterpret_cast<uintptr_t>(T);
+  if (rows % fill == 0 && cols % fill == 0 && (x0 + bytes <= t0 || t0 + bytes <= x0)) {
+    ext.x_in = const_cast<void*>(X);
+    ext.x_out = T;
+  }
   NSPlan plan;
   std::string msg;
-  cudaError_t e = plan.init(bf, {NSGroupSpec{batch, rows, cols}}, &msg);
+  cudaError_t e = plan.init(bf, {spec}, &msg, &ext);
   if (e) return fail(nullptr, NORMPRE_ERR_CUDA, "Newton-Schulz plan: " + (msg.empty() ? std::string(cudaGetErrorString(e)) : msg));
-  int* flags = nullptr;
-  if ((e = cudaMalloc(&flags, sizeof(int)))) return cuda_fail(nullptr, e, "cudaMalloc");
-  cudaMemsetAsync(flags, 0, sizeof(int), s);
-  NSGroupBuf& g = plan.groups()[0];
-  const int64_t xs = g.rows_pad * g.cols_pad;
-  for (int b = 0; b < batch && !e; ++b)
-    e = cudaMemcpy2DAsync(static_cast<char*>(g.X[0]) + b * xs * el, g.cols_pad * el,
-                          static_cast<const char*>(X) + b * rows * cols * el, cols * el, cols * el, rows,
-                          cudaMemcpyDeviceToDevice, s);
-  if (!e) e = plan.scale_from_norm(cfg->ns_eps, s);
-  if (!e) e = plan.run(cfg->ns_steps, cfg->ns_coef, s, flags);
-  const int oi = NSPlan::out_index(cfg->ns_steps);
-  for (int b = 0; b < batch && !e; ++b)
-    e = cudaMemcpy2DAsync(static_cast<char*>(T) + b * rows * cols * el, cols * el,
-                          static_cast<char*>(g.X[oi]) + b * xs * el, g.cols_pad * el, cols * el, rows,
-                          cudaMemcpyDeviceToDevice, s);
-  if (!e) e = cudaStreamSynchronize(s);
   int hf = 0;
-  if (!e) e = cudaMemcpy(&hf, flags, sizeof(int), cudaMemcpyDeviceToHost);
-  cudaFree(flags);
+  e = cudaMemsetAsync(flags, 0, sizeof(int), s);
+  if (!e) e = plan.load(X, part, cfg->ns_eps, s);
+  if (!e) e = plan.run(cfg->ns_steps, cfg->ns_coef, s, flags);
+  if (!e) e = plan.store(T, cfg->ns_steps, s);
+  if (!e) e = cudaMemcpyAsync(&hf, flags, sizeof(int), cudaMemcpyDeviceToHost, s);
+  // whatever was launched ends before the workspace goes
+  const cudaError_t es = cudaStreamSynchronize(s);
+  if (!e) e = es;
   if (e) return cuda_fail(nullptr, e, "Newton-Schulz");
   if (hf & kFlagTimeout) return fail(nullptr, NORMPRE_ERR_TIMEOUT, "a bounded device wait gave up");
   return NORMPRE_OK;
+}
+
+}  // namespace
+
+int normpre_newton_schulz_workspace(const normpre_config* cfg, int batch, int64_t rows, int64_t cols,
+                                    int64_t* bytes) {
+  if (!cfg || !bytes) return fail(nullptr, NORMPRE_ERR_ARG, "null argument");
+  const int rc = check_ns(cfg, batch, rows, cols);
+  if (rc) return rc;
+  *bytes = static_cast<int64_t>(kNsFlagBytes + ns_part_bytes(batch) +
+                                NSPlan::workspace_bytes(cfg->precision == NORMPRE_PREC_BF16, {batch, rows, cols}));
+  return NORMPRE_OK;
+}
+
+int normpre_newton_schulz_ws(const normpre_config* cfg, int batch, int64_t rows, int64_t cols, const void* X, void* T,
+                             void* workspace, int64_t workspace_bytes, void* stream) {
+  if (!cfg || !X || !T || !workspace) return fail(nullptr, NORMPRE_ERR_ARG, "null argument");
+  int64_t need = 0;
+  const int rc = normpre_newton_schulz_workspace(cfg, batch, rows, cols, &need);
+  if (rc) return rc;
+  if (!aligned16(X) || !aligned16(T) || !aligned16(workspace))
+    return fail(nullptr, NORMPRE_ERR_ALIGN, "X, T and the workspace must be 16-byte aligned");
+  if (workspace_bytes < need) return fail(nullptr, NORMPRE_ERR_ARG, "workspace too small");
+  return newton_schulz_impl(cfg, batch, rows, cols, X, T, workspace, stream);
+}
+
+int normpre_newton_schulz(const normpre_config* cfg, int batch, int64_t rows, int64_t cols, const void* X, void* T,
+                          void* stream) {
+  if (!cfg || !X || !T) return fail(nullptr, NORMPRE_ERR_ARG, "null argument");
+  int64_t need = 0;
+  const int rc0 = normpre_newton_schulz_workspace(cfg, batch, rows, cols, &need);
+  if (rc0) return rc0;
+  if (!aligned16(X) || !aligned16(T)) return fail(nullptr, NORMPRE_ERR_ALIGN, "X and T must be 16-byte aligned");
+  void* ws = nullptr;
+  const cudaError_t e = cudaMalloc(&ws, static_cast<size_t>(need));
+  if (e) return cuda_fail(nullptr, e, "cudaMalloc");
+  const int rc = newton_schulz_impl(cfg, batch, rows, cols, X, T, ws, stream);
+  cudaFree(ws);
+  return rc;
 }
 
 }  // extern "C"

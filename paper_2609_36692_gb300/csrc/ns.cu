@@ -30,7 +30,9 @@
 #include <cudaTypedefs.h>
 
 #include <algorithm>
+#include <atomic>
 #include <cstring>
+#include <type_traits>
 
 #include "common.cuh"
 #include "internal.h"
@@ -637,17 +639,115 @@ __global__ void k_scale_from_count(const ScaleArgs a) {
   }
 }
 
-template <typename T>
-__global__ void k_scale_from_norm(const T* X, int64_t per, float* inscale, float eps) {
-  __shared__ double red[32];
-  const T* x = X + static_cast<int64_t>(blockIdx.x) * per;
-  double s = 0;
-  for (int64_t i = threadIdx.x; i < per; i += blockDim.x) {
-    const double v = to_f32(x[i]);
-    s += v * v;
+// ---------------------------------------------------------------------------
+// Stand-alone Newton-Schulz input and output (normpre_newton_schulz).
+//
+// k_ns_load: X [rows][cols] -> the padded first buffer (zeros past rows and
+// cols), or nothing when `dst` is null (the products then read X itself), and
+// per CTA the sum of squares of its rows.  Bound by HBM (X read, X written);
+// the sums run in fp32 pairs with error-free additions (TwoSum, and the
+// product's own error for fp32 X; x * x of a bf16 x is exact), about 2^-46
+// relative, because fp64 runs at 1/64 of the fp32 rate here: one 512-thread
+// CTA per matrix summing in fp64 took 2256 us on 4 x 1024 x 4096.  Where a
+// square could overflow or vanish in fp32 the CTA sums its rows in fp64.
+// ---------------------------------------------------------------------------
+struct PairSum {
+  float s = 0.f, e = 0.f;
+  __device__ __forceinline__ void add_square(float x, bool exact) {
+    const float p = __fmul_rn(x, x);
+    const float t = __fadd_rn(s, p);
+    const float bb = __fadd_rn(t, -s);
+    float err = __fadd_rn(__fadd_rn(s, -__fadd_rn(t, -bb)), __fadd_rn(p, -bb));
+    if (!exact) err = __fadd_rn(err, __fmaf_rn(x, x, -p));
+    e = __fadd_rn(e, err);
+    s = t;
   }
+};
+
+struct NsCopyArgs {
+  const void* src;              // load: X; store: T's buffer
+  void* dst;
+  int rows, cols;               // the matrices as the caller holds them, contiguous
+  int rows_pad, cols_pad;       // the padded buffer
+  int rows_per_cta;             // rows of the padded buffer (load) or of the matrix (store)
+  double* part;                 // load: [batch][gridDim.y] sums of squares
+};
+// One CTA per (matrix, row chunk).
+template <typename T, bool VEC>
+__global__ void __launch_bounds__(256) k_ns_load(const __grid_constant__ NsCopyArgs a) {
+  __shared__ double red[32];
+  __shared__ float redf[32];
+  constexpr int E = VEC ? 8 : 1;
+  const int b = blockIdx.x;
+  const T* x = static_cast<const T*>(a.src) + static_cast<int64_t>(b) * a.rows * a.cols;
+  T* y = a.dst ? static_cast<T*>(a.dst) + static_cast<int64_t>(b) * a.rows_pad * a.cols_pad : nullptr;
+  const int r0 = blockIdx.y * a.rows_per_cta;
+  const int r1 = min(r0 + a.rows_per_cta, y ? a.rows_pad : a.rows);
+  const int cpr = (y ? a.cols_pad : a.cols) / E;    // pieces per row
+  const int total = r1 > r0 ? (r1 - r0) * cpr : 0;
+  PairSum ps[2];
+  float top = 0.f;
+#pragma unroll 2
+  for (int i = threadIdx.x; i < total; i += blockDim.x) {
+    const int r = r0 + i / cpr, c = (i % cpr) * E;
+    float v[E];
+#pragma unroll
+    for (int e = 0; e < E; ++e) v[e] = 0.f;
+    if (r < a.rows && c < a.cols) {
+      if constexpr (VEC) load8(x + static_cast<int64_t>(r) * a.cols + c, v);
+      else v[0] = to_f32(x[static_cast<int64_t>(r) * a.cols + c]);
+    }
+    if (y) {
+      if constexpr (VEC) store8(y + static_cast<int64_t>(r) * a.cols_pad + c, v);
+      else y[static_cast<int64_t>(r) * a.cols_pad + c] = from_f32<T>(v[0]);
+    }
+#pragma unroll
+    for (int e = 0; e < E; ++e) {
+      ps[e & 1].add_square(v[e], std::is_same<T, bf16>::value);
+      top = fmaxf(top, fabsf(v[e]));
+    }
+  }
+  double s = (static_cast<double>(ps[0].s) + ps[1].s) + (static_cast<double>(ps[0].e) + ps[1].e);
   s = block_sum(s, red);
-  if (threadIdx.x == 0) inscale[blockIdx.x] = static_cast<float>(1.0 / (sqrt(s) + static_cast<double>(eps)));
+  top = warp_max(top);
+  if ((threadIdx.x & 31) == 0) redf[threadIdx.x >> 5] = top;
+  __syncthreads();
+  for (int w = 0; w < static_cast<int>(blockDim.x >> 5); ++w) top = fmaxf(top, redf[w]);
+  if (!(top < 1e18f && top > 1e-15f) || !isfinite(s)) {
+    double d = 0;
+    for (int i = threadIdx.x; i < total; i += blockDim.x) {
+      const int r = r0 + i / cpr, c = (i % cpr) * E;
+      if (r >= a.rows || c >= a.cols) continue;
+      for (int e = 0; e < E; ++e) {
+        const double v = to_f32(x[static_cast<int64_t>(r) * a.cols + c + e]);
+        d += v * v;
+      }
+    }
+    s = block_sum(d, red);
+  }
+  if (threadIdx.x == 0) a.part[static_cast<int64_t>(b) * gridDim.y + blockIdx.y] = s;
+}
+
+// T's padded buffer -> the caller's [rows][cols]
+template <typename T, bool VEC>
+__global__ void __launch_bounds__(256) k_ns_store(const __grid_constant__ NsCopyArgs a) {
+  constexpr int E = VEC ? 8 : 1;
+  const int b = blockIdx.x;
+  const T* x = static_cast<const T*>(a.src) + static_cast<int64_t>(b) * a.rows_pad * a.cols_pad;
+  T* y = static_cast<T*>(a.dst) + static_cast<int64_t>(b) * a.rows * a.cols;
+  const int r0 = blockIdx.y * a.rows_per_cta, r1 = min(r0 + a.rows_per_cta, a.rows);
+  const int cpr = a.cols / E, total = r1 > r0 ? (r1 - r0) * cpr : 0;
+#pragma unroll 2
+  for (int i = threadIdx.x; i < total; i += blockDim.x) {
+    const int r = r0 + i / cpr, c = (i % cpr) * E;
+    if constexpr (VEC) {
+      float v[8];
+      load8(x + static_cast<int64_t>(r) * a.cols_pad + c, v);
+      store8(y + static_cast<int64_t>(r) * a.cols + c, v);
+    } else {
+      y[static_cast<int64_t>(r) * a.cols + c] = x[static_cast<int64_t>(r) * a.cols_pad + c];
+    }
+  }
 }
 
 // ---------------------------------------------------------------------------
@@ -673,6 +773,26 @@ static void pair_config(cudaLaunchConfig_t* cfg, cudaLaunchAttribute* attr, int 
   cfg->numAttrs = 1;
 }
 
+// How many two-CTA clusters of the GEMM fit at once (a GPC with an odd number
+// of usable SMs leaves one of them out); the persistent grid stays within it.
+// A property of the device, looked up once per device.
+static cudaError_t max_active_pairs(int* out, int num_sms) {
+  static std::atomic<int> known[64];
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  if (dev >= 0 && dev < 64 && known[dev].load() > 0) {
+    *out = known[dev].load() - 1;
+    return cudaSuccess;
+  }
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute attr[1];
+  pair_config(&cfg, attr, 2 * std::max(1, num_sms / 2), nullptr);
+  e = cudaOccupancyMaxActiveClusters(out, k_ns_gemm_tc<true>, &cfg);
+  if (e == cudaSuccess && dev >= 0 && dev < 64) known[dev].store(*out + 1);
+  return e;
+}
+
 NSPlan::~NSPlan() { release(); }
 
 void NSPlan::release() {
@@ -694,41 +814,72 @@ static bool make_map(CUtensorMap* m, void* base, int64_t rows, int64_t cols, int
   return driver_encode_tiled(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, base, dims, strides, box, err);
 }
 
-cudaError_t NSPlan::init(bool bf16, const std::vector<NSGroupSpec>& specs, std::string* err) {
+// Tile sizes and padded dimensions of one shape group.
+static NSGroupBuf ns_geometry(bool bf16, const NSGroupSpec& sp) {
+  const int64_t tile_m = bf16 ? 128 : 64;
+  NSGroupBuf g;
+  g.spec = sp;
+  g.tall = sp.rows > sp.cols;
+  g.s = std::min(sp.rows, sp.cols);
+  g.big = std::max(sp.rows, sp.cols);
+  g.elem = bf16 ? 2 : 4;
+  if (bf16) {
+    g.s_pad = round_up(g.s, 128);
+    g.bn_s = (g.s_pad % 256 == 0) ? 256 : 128;
+    // 256: the update of a tall matrix then has an even number of 128-row
+    // tiles and can run on two-CTA clusters
+    g.big_pad = round_up(g.big, 256);
+    g.bn_big = g.tall ? g.bn_s : 256;
+  } else {
+    g.s_pad = round_up(g.s, tile_m);
+    g.big_pad = round_up(g.big, tile_m);
+    g.bn_s = g.bn_big = 64;
+  }
+  g.rows_pad = g.tall ? g.big_pad : g.s_pad;
+  g.cols_pad = g.tall ? g.s_pad : g.big_pad;
+  return g;
+}
+
+namespace {
+struct NsBytes {
+  size_t x, a, scale;
+  explicit NsBytes(const NSGroupBuf& g)
+      : x(round_up(static_cast<int64_t>(g.spec.batch) * g.rows_pad * g.cols_pad * g.elem, 1024)),
+        a(round_up(static_cast<int64_t>(g.spec.batch) * g.s_pad * g.s_pad * g.elem, 1024)),
+        scale(round_up(static_cast<int64_t>(g.spec.batch) * sizeof(float), 1024)) {}
+};
+}  // namespace
+
+size_t NSPlan::workspace_bytes(bool bf16, const NSGroupSpec& spec) {
+  const NsBytes n(ns_geometry(bf16, spec));
+  return 1024 + 3 * n.x + 2 * n.a + n.scale;
+}
+
+cudaError_t NSPlan::init(bool bf16, const std::vector<NSGroupSpec>& specs, std::string* err, const NSExternal* ext) {
   release();
   bf16_ = bf16;
   num_sms_ = device_sm_count();
-  if (static_cast<int>(specs.size()) > kMaxGroups) {
+  if (static_cast<int>(specs.size()) > kMaxGroups || (ext && specs.size() != 1)) {
     if (err) *err = "too many Newton-Schulz shape groups";
     return cudaErrorInvalidValue;
   }
   const int64_t tile_m = bf16 ? 128 : 64;
   for (const NSGroupSpec& sp : specs) {
-    NSGroupBuf g;
-    g.spec = sp;
-    g.tall = sp.rows > sp.cols;
-    g.s = std::min(sp.rows, sp.cols);
-    g.big = std::max(sp.rows, sp.cols);
-    g.elem = bf16 ? 2 : 4;
-    if (bf16) {
-      g.s_pad = round_up(g.s, 128);
-      g.bn_s = (g.s_pad % 256 == 0) ? 256 : 128;
-      if (g.tall) {
-        // 256: the update of a tall matrix then has an even number of
-        // 128-row tiles and can run on two-CTA clusters
-        g.big_pad = round_up(g.big, 256);
-        g.bn_big = g.bn_s;
-      } else {
-        g.big_pad = round_up(g.big, 256);
-        g.bn_big = 256;
-      }
-    } else {
-      g.s_pad = round_up(g.s, tile_m);
-      g.big_pad = round_up(g.big, tile_m);
-      g.bn_s = g.bn_big = 64;
+    NSGroupBuf g = ns_geometry(bf16, sp);
+    if (ext) {
+      // the caller's workspace, carved; nothing has to be zero in it (load()
+      // writes the padding of X[0], the products write whole padded tiles)
+      const NsBytes n(g);
+      char* p = reinterpret_cast<char*>(round_up(reinterpret_cast<uintptr_t>(ext->ws), 1024));
+      for (int i = 0; i < 3; ++i, p += n.x) g.X[i] = p;
+      g.A = p; p += n.a;
+      g.B = p; p += n.a;
+      g.inscale = reinterpret_cast<float*>(p);
+      if (ext->x_in) g.X[0] = ext->x_in;
+      if (ext->x_out) g.X[out_index(ext->steps)] = ext->x_out;
+      groups_.push_back(g);
+      continue;
     }
-    g.rows_pad = g.tall ? g.big_pad : g.s_pad;
-    g.cols_pad = g.tall ? g.s_pad : g.big_pad;
     const size_t xbytes = static_cast<size_t>(sp.batch) * g.rows_pad * g.cols_pad * g.elem;
     const size_t abytes = static_cast<size_t>(sp.batch) * g.s_pad * g.s_pad * g.elem;
     // tiles of the update GEMM (its epilogue emits the ||T||^2 partials)
@@ -854,13 +1005,8 @@ cudaError_t NSPlan::init(bool bf16, const std::vector<NSGroupSpec>& specs, std::
       e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kTcSmem));
       if (e != cudaSuccess) return e;
     }
-    // how many two-CTA clusters fit at once (a GPC with an odd number of
-    // usable SMs leaves one of them out); the persistent grid stays within it
-    cudaLaunchConfig_t cfg = {};
-    cudaLaunchAttribute attr[1];
-    pair_config(&cfg, attr, 2 * std::max(1, num_sms_ / 2), nullptr);
     int n = 0;
-    e = cudaOccupancyMaxActiveClusters(&n, k_ns_gemm_tc<true>, &cfg);
+    e = max_active_pairs(&n, num_sms_);
     if (e != cudaSuccess) return e;
     max_pairs_ = n;
     if (n < 1) L->mc[0] = L->mc[1] = L->mc[2] = false;
@@ -984,15 +1130,61 @@ cudaError_t NSPlan::scale_from_count(const int* count, const int* const* group_m
   return cudaGetLastError();
 }
 
-cudaError_t NSPlan::scale_from_norm(float eps, cudaStream_t s) {
-  for (NSGroupBuf& g : groups_) {
-    const int64_t per = g.rows_pad * g.cols_pad;
-    if (bf16_) k_scale_from_norm<normpre::bf16><<<g.spec.batch, 512, 0, s>>>(static_cast<const normpre::bf16*>(g.X[0]), per, g.inscale, eps);
-    else k_scale_from_norm<float><<<g.spec.batch, 512, 0, s>>>(static_cast<const float*>(g.X[0]), per, g.inscale, eps);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
+// CTAs per matrix of the load and store passes: eight per SM over the batch,
+// at least four rows each.
+static int copy_ctas(int64_t rows, int batch) {
+  const int64_t want = cdiv(static_cast<int64_t>(device_sm_count()) * 8, batch);
+  return static_cast<int>(std::max<int64_t>(1, std::min(std::min<int64_t>(want, kNsCopyCtas), cdiv(rows, 4))));
+}
+
+cudaError_t NSPlan::load(const void* X, double* part, float eps, cudaStream_t s) {
+  NSGroupBuf& g = groups_[0];
+  const bool direct = g.X[0] == X;
+  NsCopyArgs a;
+  a.src = X;
+  a.dst = direct ? nullptr : g.X[0];
+  a.rows = static_cast<int>(g.spec.rows); a.cols = static_cast<int>(g.spec.cols);
+  a.rows_pad = static_cast<int>(g.rows_pad); a.cols_pad = static_cast<int>(g.cols_pad);
+  a.part = part;
+  const int64_t rows = direct ? g.spec.rows : g.rows_pad;
+  const int n = copy_ctas(rows, g.spec.batch);
+  a.rows_per_cta = static_cast<int>(cdiv(rows, n));
+  const dim3 grid(g.spec.batch, n);
+  const bool vec = g.spec.cols % 8 == 0;
+  if (bf16_) {
+    if (vec) k_ns_load<normpre::bf16, true><<<grid, 256, 0, s>>>(a);
+    else k_ns_load<normpre::bf16, false><<<grid, 256, 0, s>>>(a);
+  } else {
+    if (vec) k_ns_load<float, true><<<grid, 256, 0, s>>>(a);
+    else k_ns_load<float, false><<<grid, 256, 0, s>>>(a);
   }
-  return cudaSuccess;
+  cudaError_t e = cudaGetLastError();
+  if (e != cudaSuccess) return e;
+  return launch_muon_prescale(part, n, n, g.spec.batch, g.inscale, eps, s);
+}
+
+cudaError_t NSPlan::store(void* T, int steps, cudaStream_t s) {
+  NSGroupBuf& g = groups_[0];
+  const void* src = g.X[out_index(steps)];
+  if (src == T) return cudaSuccess;      // the last product wrote it
+  NsCopyArgs a;
+  a.src = src;
+  a.dst = T;
+  a.rows = static_cast<int>(g.spec.rows); a.cols = static_cast<int>(g.spec.cols);
+  a.rows_pad = static_cast<int>(g.rows_pad); a.cols_pad = static_cast<int>(g.cols_pad);
+  a.part = nullptr;
+  const int n = copy_ctas(g.spec.rows, g.spec.batch);
+  a.rows_per_cta = static_cast<int>(cdiv(g.spec.rows, n));
+  const dim3 grid(g.spec.batch, n);
+  const bool vec = g.spec.cols % 8 == 0;
+  if (bf16_) {
+    if (vec) k_ns_store<normpre::bf16, true><<<grid, 256, 0, s>>>(a);
+    else k_ns_store<normpre::bf16, false><<<grid, 256, 0, s>>>(a);
+  } else {
+    if (vec) k_ns_store<float, true><<<grid, 256, 0, s>>>(a);
+    else k_ns_store<float, false><<<grid, 256, 0, s>>>(a);
+  }
+  return cudaGetLastError();
 }
 
 }  // namespace normpre

@@ -90,6 +90,11 @@ def load_library(path: str = LIB_PATH) -> ctypes.CDLL:
     lib.normpre_read.restype = ctypes.c_int
     lib.normpre_newton_schulz.argtypes = [ctypes.POINTER(normpre_config), ctypes.c_int, i64, i64, P, P, P]
     lib.normpre_newton_schulz.restype = ctypes.c_int
+    lib.normpre_newton_schulz_workspace.argtypes = [ctypes.POINTER(normpre_config), ctypes.c_int, i64, i64,
+                                                    ctypes.POINTER(i64)]
+    lib.normpre_newton_schulz_workspace.restype = ctypes.c_int
+    lib.normpre_newton_schulz_ws.argtypes = [ctypes.POINTER(normpre_config), ctypes.c_int, i64, i64, P, P, P, i64, P]
+    lib.normpre_newton_schulz_ws.restype = ctypes.c_int
     lib.normpre_profile.argtypes = [P, ctypes.c_int]
     lib.normpre_profile.restype = ctypes.c_int
     lib.normpre_profile_read.argtypes = [P, ctypes.c_int, ctypes.POINTER(ctypes.c_double),
@@ -181,6 +186,19 @@ def normpre_newton_schulz(cfg: normpre_config, batch: int, rows: int, cols: int,
                           T_ptr: int, stream: int = 0) -> int:
     return _check(load_library().normpre_newton_schulz(ctypes.byref(cfg), int(batch), int(rows),
                                                        int(cols), X_ptr, T_ptr, stream))
+
+
+def normpre_newton_schulz_workspace(cfg: normpre_config, batch: int, rows: int, cols: int) -> int:
+    n = ctypes.c_int64()
+    _check(load_library().normpre_newton_schulz_workspace(ctypes.byref(cfg), int(batch), int(rows), int(cols),
+                                                          ctypes.byref(n)))
+    return n.value
+
+
+def normpre_newton_schulz_ws(cfg: normpre_config, batch: int, rows: int, cols: int, X_ptr: int, T_ptr: int,
+                             ws_ptr: int, ws_bytes: int, stream: int = 0) -> int:
+    return _check(load_library().normpre_newton_schulz_ws(ctypes.byref(cfg), int(batch), int(rows), int(cols),
+                                                          X_ptr, T_ptr, ws_ptr, int(ws_bytes), stream))
 
 
 PROFILE_CLASSES = ["normalize", "ns_gram", "ns_poly", "ns_update", "apply_g", "omega", "contract",

@@ -216,6 +216,10 @@ def newton_schulz(X, **config):
     if x.dtype != want:
         raise TypeError("precision %d needs %s input" % (cfg.precision, want))
     T = torch.empty_like(x)
-    C.normpre_newton_schulz(cfg, x.shape[0], x.shape[1], x.shape[2], x.data_ptr(), T.data_ptr(),
-                            torch.cuda.current_stream().cuda_stream)
+    # the workspace from torch's caching allocator: its memory stays with torch
+    # between calls instead of being mapped and unmapped by each
+    n = C.normpre_newton_schulz_workspace(cfg, *x.shape)
+    ws = torch.empty(n, dtype=torch.uint8, device=x.device)
+    C.normpre_newton_schulz_ws(cfg, *x.shape, x.data_ptr(), T.data_ptr(), ws.data_ptr(), n,
+                               torch.cuda.current_stream().cuda_stream)
     return T if X.dim() == 3 else T[0]
