@@ -46,12 +46,29 @@ __global__ void __launch_bounds__(256) k_apply_g(const __grid_constant__ ApplyLa
       store8(W + static_cast<int64_t>(r) * a.cols + c, w);
     }
   } else {
+    // rows that are not whole 16-byte pieces: a CTA takes runs of 2048
+    // consecutive elements of W, lane next to lane, eight loads of each
+    // operand in flight; (row, column) advance without a division (one 64-bit
+    // division per element took 2 x 2048 x 5461 from 129 us to what HBM needs)
     const int64_t n = a.rows * a.cols;
-    for (int64_t i = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; i < n;
-         i += static_cast<int64_t>(gridDim.x) * blockDim.x) {
-      const int64_t r = i / a.cols, c = i - r * a.cols;
-      const float w = to_f32(W[i]);
-      W[i] = from_f32<TW>(fmaf(cw, w, ct * to_f32(T[r * a.t_ld + c])));
+    const int cols = static_cast<int>(a.cols);
+    const int dr = 256 / cols, dc = 256 - dr * cols;
+    for (int64_t i0 = static_cast<int64_t>(blockIdx.x) * 2048 + threadIdx.x; i0 < n;
+         i0 += static_cast<int64_t>(gridDim.x) * 2048) {
+      int64_t r = i0 / cols;
+      int c = static_cast<int>(i0 - r * cols);
+      float w[8], t[8];
+#pragma unroll
+      for (int e = 0; e < 8; ++e) {
+        const bool ok = i0 + 256 * e < n;
+        w[e] = ok ? to_f32(W[i0 + 256 * e]) : 0.f;
+        t[e] = ok ? to_f32(T[r * a.t_ld + c]) : 0.f;
+        c += dc; r += dr;
+        if (c >= cols) { c -= cols; ++r; }
+      }
+#pragma unroll
+      for (int e = 0; e < 8; ++e)
+        if (i0 + 256 * e < n) W[i0 + 256 * e] = from_f32<TW>(fmaf(cw, w[e], ct * t[e]));
     }
   }
 }
@@ -60,7 +77,7 @@ cudaError_t launch_apply_g(const ApplyLaunch& a, cudaStream_t s) {
   if (a.n <= 0) return cudaSuccess;
   const bool vec = (a.cols % 8 == 0) && (a.t_ld % 8 == 0) &&
                    static_cast<uint64_t>(a.rows) * static_cast<uint64_t>(a.cols) / 8 < (1ull << 31);
-  const int64_t work = vec ? a.rows * a.cols / 8 : a.rows * a.cols;
+  const int64_t work = cdiv(a.rows * a.cols, 8);
   int64_t per = cdiv(work, 256);
   const int64_t cap = cdiv(static_cast<int64_t>(device_sm_count()) * 8, a.n);
   if (per > cap) per = cap;

@@ -87,6 +87,7 @@ inline int64_t cdiv(int64_t x, int64_t m) { return (x + m - 1) / m; }
 // ----------------------------------------------------------------------------
 // K1: momentum + relaxed tangent + diagonal-Gram normalization (normalize.cu)
 // ----------------------------------------------------------------------------
+constexpr int kColStatsRB = 256;  // most rows per block of the column sums
 struct NormLaunch {
   int n = 0;                      // matrices in this launch (<= kMaxBatch)
   int64_t rows = 0, cols = 0;     // stored shape
@@ -102,7 +103,9 @@ struct NormLaunch {
   int tangent = 0;                // 0 relaxed (paper), 1 none, 2 strict (Table 5a ablations)
   int* count = nullptr;           // [n_mats] nonzero active rows, accumulated
   int* flags = nullptr;
-  // column-active scratch (see normalize_cols_scratch_bytes)
+  // column-active scratch (see normalize_cols_scratch_bytes) and rows per
+  // block of the column sums, fixed for a group so that its slices sum alike
+  int col_rb = kColStatsRB;
   double* col_part = nullptr;
   float2* col_coef = nullptr;
 };
@@ -120,8 +123,9 @@ cudaError_t launch_normalize_cols(const NormLaunch& a, cudaStream_t s);
 // Orientation 3 ("Row+Column/Step"): the columns of a row-normalized Psi
 // normalized in place; count[] becomes the number of nonzero columns.
 cudaError_t launch_normalize_psi_cols(const NormLaunch& a, cudaStream_t s);
-size_t normalize_cols_scratch_bytes(int64_t rows, int64_t cols, int n);
-size_t normalize_cols_part_bytes(int64_t rows, int64_t cols, int n);   // col_part share of it
+int col_stats_rows(int64_t rows, int64_t cols, int n);   // col_rb of launches of up to n matrices
+size_t normalize_cols_scratch_bytes(int64_t rows, int64_t cols, int n, int rb = kColStatsRB);
+size_t normalize_cols_part_bytes(int64_t rows, int64_t cols, int n, int rb = kColStatsRB);   // col_part share of it
 
 // ----------------------------------------------------------------------------
 // K7: NormPre-G apply: W <- W - lr (target * sqrt(mn)/||T|| T + wd W) (apply.cu)

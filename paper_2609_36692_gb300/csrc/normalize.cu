@@ -5,7 +5,7 @@
 // Row-active steps (k = 0): one CTA per stored row; the row of M and W stays in
 // registers between the two block reductions (<m, w>, then ||x||^2), so the
 // step reads G, M_{t-1}, W once and writes M_t, Psi once, with 16-byte vector
-// accesses.
+// accesses, or (rows that are not whole 16-byte pieces) one element per lane.
 //
 // Column-active steps (k = 1): the reduction runs down the columns of the
 // row-major layout.  Pass A streams G, M_{t-1}, W once, writes M_t and per-
@@ -34,8 +34,7 @@
 
 namespace normpre {
 
-constexpr int kColStatsRB = 256;  // rows per block of pass A (one partial sum per block and column)
-constexpr int kColApplyRB = 64;   // rows per block of pass B
+constexpr int kColApplyRB = 64;   // rows per block of pass B (16 where that leaves SMs idle)
 constexpr int kColThreads = 256;  // 32 column chunks of 8 x 8 row lanes
 
 // c_i of the tangent step for mode 0 relaxed, 1 none, 2 strict (mw = <m_i, w_i>,
@@ -46,21 +45,58 @@ __device__ __forceinline__ float tangent_coef(int mode, float mw, float ww) {
   return 0.f;
 }
 
-size_t normalize_cols_part_bytes(int64_t rows, int64_t cols, int n) {
-  return static_cast<size_t>(n) * cdiv(rows, kColStatsRB) * cols * 3 * sizeof(double);
+// Rows per block of pass A: 256, halved down to 32 while the launch has fewer
+// than four blocks per SM.  A block walks its rows in rounds of eight, each a
+// round trip to HBM, so few tall blocks are latency-bound: one 256 x 1024
+// matrix took 28 us in four 256-row blocks.
+int col_stats_rows(int64_t rows, int64_t cols, int n) {
+  int rb = kColStatsRB;
+  const int64_t want = 4 * static_cast<int64_t>(device_sm_count());
+  while (rb > 32 && cdiv(cols, 256) * cdiv(rows, rb) * n < want) rb /= 2;
+  return rb;
 }
 
-size_t normalize_cols_scratch_bytes(int64_t rows, int64_t cols, int n) {
-  const int64_t nrb = cdiv(rows, kColStatsRB);
-  return static_cast<size_t>(n) * nrb * cols * 3 * sizeof(double) +
-         static_cast<size_t>(n) * cols * sizeof(float2) + 256;
+size_t normalize_cols_part_bytes(int64_t rows, int64_t cols, int n, int rb) {
+  return static_cast<size_t>(n) * cdiv(rows, rb) * cols * 3 * sizeof(double);
+}
+
+size_t normalize_cols_scratch_bytes(int64_t rows, int64_t cols, int n, int rb) {
+  return normalize_cols_part_bytes(rows, cols, n, rb) + static_cast<size_t>(n) * cols * sizeof(float2) + 256;
 }
 
 // ---------------------------------------------------------------------------
-// row-active, vector path (cols % 8 == 0, cols <= 16 * blockDim)
+// row-active, cols <= 16 * blockDim: 16 elements of the row per thread, in two
+// 8-element pieces (VEC: cols % 8 == 0) or one by one, lane next to lane.  The
+// element form keeps one pass over HBM for rows of any width (5461 columns,
+// bf16 G, fp32 W and Psi: 416 us with the re-reading kernel below, which is
+// left for rows past 16384).
 // ---------------------------------------------------------------------------
-template <typename TG, typename TW, typename TP>
-__global__ void __launch_bounds__(1024) k_norm_rows_vec(const __grid_constant__ NormLaunch a) {
+template <typename T, bool VEC>
+__device__ __forceinline__ void row_load(const T* p, int64_t j, int64_t cols, float* v) {
+  if constexpr (VEC) {
+    load8(p + j, v);
+  } else {
+#pragma unroll
+    for (int e = 0; e < 8; ++e) {
+      const int64_t je = j + static_cast<int64_t>(e) * blockDim.x;
+      v[e] = je < cols ? to_f32(p[je]) : 0.f;
+    }
+  }
+}
+template <typename T, bool VEC>
+__device__ __forceinline__ void row_store(T* p, int64_t j, int64_t cols, const float* v) {
+  if constexpr (VEC) {
+    store8(p + j, v);
+  } else {
+#pragma unroll
+    for (int e = 0; e < 8; ++e) {
+      const int64_t je = j + static_cast<int64_t>(e) * blockDim.x;
+      if (je < cols) p[je] = from_f32<T>(v[e]);
+    }
+  }
+}
+template <typename TG, typename TW, typename TP, bool VEC>
+__global__ void __launch_bounds__(1024) k_norm_rows(const __grid_constant__ NormLaunch a) {
   __shared__ float red[32];
   const int b = blockIdx.y;
   const int64_t row = blockIdx.x;
@@ -73,19 +109,21 @@ __global__ void __launch_bounds__(1024) k_norm_rows_vec(const __grid_constant__ 
   float dot = 0.f, wsq = 0.f;
 #pragma unroll
   for (int c = 0; c < 2; ++c) {
-    const int64_t j = (static_cast<int64_t>(c) * blockDim.x + threadIdx.x) * 8;
+    const int64_t j = VEC ? (static_cast<int64_t>(c) * blockDim.x + threadIdx.x) * 8
+                          : static_cast<int64_t>(c) * 8 * blockDim.x + threadIdx.x;
     if (j < cols) {
       float gv[8], mp[8];
-      load8(g + j, gv);
-      load8_cg(M + j, mp);
-      load8(w + j, wv[c]);
+      row_load<TG, VEC>(g, j, cols, gv);
+      if constexpr (VEC) load8_cg(M + j, mp);
+      else row_load<float, VEC>(M, j, cols, mp);
+      row_load<TW, VEC>(w, j, cols, wv[c]);
 #pragma unroll
       for (int e = 0; e < 8; ++e) {
         m[c][e] = fmaf(a.mu, mp[e], gv[e]);
         dot = fmaf(m[c][e], wv[c][e], dot);
         wsq = fmaf(wv[c][e], wv[c][e], wsq);
       }
-      store8(M + j, m[c]);
+      row_store<float, VEC>(M, j, cols, m[c]);
     } else {
 #pragma unroll
       for (int e = 0; e < 8; ++e) { m[c][e] = 0.f; wv[c][e] = 0.f; }
@@ -118,12 +156,13 @@ __global__ void __launch_bounds__(1024) k_norm_rows_vec(const __grid_constant__ 
   const float inv = ss > 0.f ? 1.f / sqrtf(ss) : 0.f;
 #pragma unroll
   for (int c = 0; c < 2; ++c) {
-    const int64_t j = (static_cast<int64_t>(c) * blockDim.x + threadIdx.x) * 8;
+    const int64_t j = VEC ? (static_cast<int64_t>(c) * blockDim.x + threadIdx.x) * 8
+                          : static_cast<int64_t>(c) * 8 * blockDim.x + threadIdx.x;
     if (j < cols) {
       float v[8];
 #pragma unroll
       for (int e = 0; e < 8; ++e) v[e] = m[c][e] * inv;
-      store8(psi + j, v);
+      row_store<TP, VEC>(psi, j, cols, v);
     }
   }
   if (threadIdx.x == 0) {
@@ -132,7 +171,7 @@ __global__ void __launch_bounds__(1024) k_norm_rows_vec(const __grid_constant__ 
   }
 }
 
-// row-active, scalar path (any shape): M is re-read by the thread that wrote it
+// row-active, rows past 16 * 1024 columns: M is re-read by the thread that wrote it
 template <typename TG, typename TW, typename TP>
 __global__ void __launch_bounds__(256) k_norm_rows_scalar(const __grid_constant__ NormLaunch a) {
   __shared__ float red[32];
@@ -185,8 +224,8 @@ __global__ void __launch_bounds__(kColThreads) k_norm_cols_stats(const __grid_co
   const int b = blockIdx.z, rb = blockIdx.y;
   const int cc = threadIdx.x & 31, rl = threadIdx.x >> 5;
   const int64_t rows = a.rows, cols = a.cols;
-  const int64_t r0 = static_cast<int64_t>(rb) * kColStatsRB;
-  const int64_t r1 = min(r0 + kColStatsRB, rows);
+  const int64_t r0 = static_cast<int64_t>(rb) * a.col_rb;
+  const int64_t r1 = min(r0 + a.col_rb, rows);
   const TG* g = static_cast<const TG*>(a.G[b]);
   float* M = a.M[b];
   const TW* w = static_cast<const TW*>(a.W[b]);
@@ -220,20 +259,33 @@ __global__ void __launch_bounds__(kColThreads) k_norm_cols_stats(const __grid_co
       part[rl][2][cc * 8 + e] = sww[e];
     }
   } else {
-    // scalar: thread handles columns cc + 32 e of the strip
+    // rows of any alignment: the thread's columns are cc + 32 e of the strip,
+    // so that a warp reads 32 consecutive elements, all of a row's eight at
+    // once (column by column, 5461 wide, took 503 us against the 140 of the
+    // 16-byte form on as many elements)
+    const int64_t j0 = static_cast<int64_t>(blockIdx.x) * 256 + cc;
+    const int ne = static_cast<int>(min(static_cast<int64_t>(8), (cols - j0 + 31) / 32));   // <= 0: none
+    for (int64_t r = r0 + rl; r < r1; r += 8) {
+      const int64_t o = r * cols + j0;
+      float gv[8], mp[8], wv[8];
+#pragma unroll
+      for (int e = 0; e < 8; ++e) {
+        const bool ok = e < ne;
+        gv[e] = ok ? to_f32(g[o + 32 * e]) : 0.f;
+        mp[e] = ok ? M[o + 32 * e] : 0.f;
+        wv[e] = ok ? to_f32(w[o + 32 * e]) : 0.f;
+      }
+#pragma unroll
+      for (int e = 0; e < 8; ++e) {
+        const float m = fmaf(a.mu, mp[e], gv[e]);
+        if (e < ne) M[o + 32 * e] = m;
+        smm[e] = fmaf(m, m, smm[e]);
+        smw[e] = fmaf(m, wv[e], smw[e]);
+        sww[e] = fmaf(wv[e], wv[e], sww[e]);
+      }
+    }
 #pragma unroll
     for (int e = 0; e < 8; ++e) {
-      const int64_t j = static_cast<int64_t>(blockIdx.x) * 256 + cc + 32 * e;
-      if (j < cols) {
-        for (int64_t r = r0 + rl; r < r1; r += 8) {
-          const float m = fmaf(a.mu, M[r * cols + j], to_f32(g[r * cols + j]));
-          const float wv = to_f32(w[r * cols + j]);
-          M[r * cols + j] = m;
-          smm[e] = fmaf(m, m, smm[e]);
-          smw[e] = fmaf(m, wv, smw[e]);
-          sww[e] = fmaf(wv, wv, sww[e]);
-        }
-      }
       part[rl][0][cc + 32 * e] = smm[e];
       part[rl][1][cc + 32 * e] = smw[e];
       part[rl][2][cc + 32 * e] = sww[e];
@@ -271,6 +323,7 @@ __global__ void __launch_bounds__(256) k_norm_cols_final(const __grid_constant__
   if (j < cols) {
     double s0 = 0, s1 = 0, s2 = 0;
     const double* p = a.col_part + (static_cast<int64_t>(b) * nrb * cols + j) * 3;
+#pragma unroll 8
     for (int rb = 0; rb < nrb; ++rb) {
       s0 += p[0]; s1 += p[1]; s2 += p[2];
       p += cols * 3;
@@ -311,8 +364,8 @@ __global__ void __launch_bounds__(kColThreads) k_norm_cols_xsq(const __grid_cons
   const int b = blockIdx.z, rb = blockIdx.y;
   const int cc = threadIdx.x & 31, rl = threadIdx.x >> 5;
   const int64_t rows = a.rows, cols = a.cols;
-  const int64_t r0 = static_cast<int64_t>(rb) * kColStatsRB;
-  const int64_t r1 = min(r0 + kColStatsRB, rows);
+  const int64_t r0 = static_cast<int64_t>(rb) * a.col_rb;
+  const int64_t r1 = min(r0 + a.col_rb, rows);
   const float* M = a.M[b];
   const TW* w = static_cast<const TW*>(a.W[b]);
   const float2* coef = a.col_coef + static_cast<int64_t>(b) * cols;
@@ -366,12 +419,12 @@ __global__ void __launch_bounds__(kColThreads) k_norm_cols_xsq(const __grid_cons
 
 // column-active pass B: Psi_ij = (m_ij - a_j w_ij) * inv_j
 template <typename TW, typename TP, bool VEC>
-__global__ void __launch_bounds__(kColThreads) k_norm_cols_apply(const __grid_constant__ NormLaunch a) {
+__global__ void __launch_bounds__(kColThreads) k_norm_cols_apply(const __grid_constant__ NormLaunch a, int nrows) {
   const int b = blockIdx.z, rb = blockIdx.y;
   const int cc = threadIdx.x & 31, rl = threadIdx.x >> 5;
   const int64_t rows = a.rows, cols = a.cols;
-  const int64_t r0 = static_cast<int64_t>(rb) * kColApplyRB;
-  const int64_t r1 = min(r0 + kColApplyRB, rows);
+  const int64_t r0 = static_cast<int64_t>(rb) * nrows;
+  const int64_t r1 = min(r0 + nrows, rows);
   const float* M = a.M[b];
   const TW* w = static_cast<const TW*>(a.W[b]);
   TP* psi = static_cast<TP*>(a.psi[b]);
@@ -382,6 +435,7 @@ __global__ void __launch_bounds__(kColThreads) k_norm_cols_apply(const __grid_co
     float ca[8], ci[8];
 #pragma unroll
     for (int e = 0; e < 8; ++e) { const float2 c = coef[j0 + e]; ca[e] = c.x; ci[e] = c.y; }
+#pragma unroll 2
     for (int64_t r = r0 + rl; r < r1; r += 8) {
       float mv[8], wv[8];
       load8(M + r * cols + j0, mv);
@@ -391,12 +445,25 @@ __global__ void __launch_bounds__(kColThreads) k_norm_cols_apply(const __grid_co
       store8(psi + r * a.psi_ld + j0, mv);
     }
   } else {
+    const int64_t j0 = static_cast<int64_t>(blockIdx.x) * 256 + cc;
+    const int ne = static_cast<int>(min(static_cast<int64_t>(8), (cols - j0 + 31) / 32));   // <= 0: none
+    float ca[8], ci[8];
+#pragma unroll
     for (int e = 0; e < 8; ++e) {
-      const int64_t j = static_cast<int64_t>(blockIdx.x) * 256 + cc + 32 * e;
-      if (j >= cols) break;
-      const float2 c = coef[j];
-      for (int64_t r = r0 + rl; r < r1; r += 8)
-        psi[r * a.psi_ld + j] = from_f32<TP>(fmaf(-c.x, to_f32(w[r * cols + j]), M[r * cols + j]) * c.y);
+      const float2 c = e < ne ? coef[j0 + 32 * e] : make_float2(0.f, 0.f);
+      ca[e] = c.x; ci[e] = c.y;
+    }
+    for (int64_t r = r0 + rl; r < r1; r += 8) {
+      const int64_t o = r * cols + j0;
+      float mv[8], wv[8];
+#pragma unroll
+      for (int e = 0; e < 8; ++e) {
+        mv[e] = e < ne ? M[o + 32 * e] : 0.f;
+        wv[e] = e < ne ? to_f32(w[o + 32 * e]) : 0.f;
+      }
+#pragma unroll
+      for (int e = 0; e < 8; ++e)
+        if (e < ne) psi[r * a.psi_ld + j0 + 32 * e] = from_f32<TP>(fmaf(-ca[e], wv[e], mv[e]) * ci[e]);
     }
   }
 }
@@ -490,10 +557,11 @@ cudaError_t launch_normalize_rows(const NormLaunch& a, cudaStream_t s) {
     using TG = std::remove_pointer_t<decltype(tg)>;
     using TW = std::remove_pointer_t<decltype(tw)>;
     using TP = std::remove_pointer_t<decltype(tp)>;
+    const int threads = static_cast<int>(round_up(cdiv(a.cols, 16), 32));
     if (vec) {
-      int threads = static_cast<int>(round_up(cdiv(a.cols, 16), 32));
-      threads = threads < 32 ? 32 : threads;
-      k_norm_rows_vec<TG, TW, TP><<<grid, threads, 0, s>>>(a);
+      k_norm_rows<TG, TW, TP, true><<<grid, threads, 0, s>>>(a);
+    } else if (a.cols <= 16 * 1024) {
+      k_norm_rows<TG, TW, TP, false><<<grid, threads, 0, s>>>(a);
     } else {
       k_norm_rows_scalar<TG, TW, TP><<<grid, 256, 0, s>>>(a);
     }
@@ -504,10 +572,11 @@ cudaError_t launch_normalize_rows(const NormLaunch& a, cudaStream_t s) {
 cudaError_t launch_normalize_cols(const NormLaunch& a, cudaStream_t s) {
   if (a.n <= 0 || a.rows <= 0 || a.cols <= 0) return cudaSuccess;
   const bool vec = (a.cols % 8 == 0) && (a.psi_ld % 8 == 0);
-  const int nrb = static_cast<int>(cdiv(a.rows, kColStatsRB));
+  const int nrb = static_cast<int>(cdiv(a.rows, a.col_rb));
   const dim3 grid(static_cast<unsigned>(cdiv(a.cols, 256)), static_cast<unsigned>(nrb),
                   static_cast<unsigned>(a.n));
-  const dim3 grid_b(grid.x, static_cast<unsigned>(cdiv(a.rows, kColApplyRB)), static_cast<unsigned>(a.n));
+  const int rb_b = grid.x * cdiv(a.rows, kColApplyRB) * a.n < 4 * static_cast<int64_t>(device_sm_count()) ? 16 : kColApplyRB;
+  const dim3 grid_b(grid.x, static_cast<unsigned>(cdiv(a.rows, rb_b)), static_cast<unsigned>(a.n));
   return dispatch3(a.g_dtype, a.w_dtype, a.psi_dtype, [&](auto* tg, auto* tw, auto* tp) {
     using TG = std::remove_pointer_t<decltype(tg)>;
     using TW = std::remove_pointer_t<decltype(tw)>;
@@ -529,8 +598,8 @@ cudaError_t launch_normalize_cols(const NormLaunch& a, cudaStream_t s) {
     }
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    if (vec) k_norm_cols_apply<TW, TP, true><<<grid_b, kColThreads, 0, s>>>(a);
-    else k_norm_cols_apply<TW, TP, false><<<grid_b, kColThreads, 0, s>>>(a);
+    if (vec) k_norm_cols_apply<TW, TP, true><<<grid_b, kColThreads, 0, s>>>(a, rb_b);
+    else k_norm_cols_apply<TW, TP, false><<<grid_b, kColThreads, 0, s>>>(a, rb_b);
     return cudaGetLastError();
   });
 }

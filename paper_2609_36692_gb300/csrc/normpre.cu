@@ -33,6 +33,7 @@ struct Group {
   int w_dtype, g_dtype;
   std::vector<int> mats;       // global matrix ids
   int* mat_ids_dev = nullptr;  // device copy of mats
+  int col_rb = kColStatsRB;    // rows per block of the column sums
   // NormPre-L
   SketchGroup sk;
 };
@@ -295,7 +296,9 @@ int normpre_init(const normpre_config* cfg, int n_mats, const int64_t* rows, con
     e = cudaMemcpy(g.mat_ids_dev, g.mats.data(), sizeof(int) * g.mats.size(), cudaMemcpyHostToDevice);
     if (e) return cuda_fail(nullptr, e, "cudaMemcpy");
     const int chunk = std::min<int>(kMaxBatch, static_cast<int>(g.mats.size()));
-    scratch = std::max(scratch, normalize_cols_scratch_bytes(g.rows, g.cols, chunk));
+    g.col_rb = col_stats_rows(g.rows, g.cols, chunk);
+    // (orientation 3 sums the columns of Psi in blocks of kColStatsRB >= col_rb rows)
+    scratch = std::max(scratch, normalize_cols_scratch_bytes(g.rows, g.cols, chunk, g.col_rb));
   }
   if ((e = dalloc(hp, &h->col_part, scratch))) return cuda_fail(nullptr, e, "cudaMalloc");
   {
@@ -428,6 +431,7 @@ int step_impl(normpre_handle* h, int64_t t, float lr, void* const* W, const void
       a.tangent = c.tangent;
       a.count = h->count;
       a.flags = h->flags;
+      a.col_rb = g.col_rb;
       a.col_part = h->col_part;
       a.col_coef = h->col_coef;
       if (is_muon) {

@@ -59,3 +59,60 @@ def test_newton_schulz_workspace():
     assert e.value.status == C.NORMPRE_ERR_ARG
 
 
+# ---------------------------------------------------------------------------
+# momentum + tangent + normalization: rows that are not whole 16-byte pieces,
+# rows past the register form, blocks of 32 to 256 rows in the column sums
+# ---------------------------------------------------------------------------
+@pytest.mark.parametrize("w_dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("t", [0, 1])
+@pytest.mark.parametrize("rows,cols,n", [(33, 1, 1), (1, 33, 2), (257, 1029, 2), (520, 2047, 1), (3, 16391, 1),
+                                         (70, 16384, 1), (4097, 264, 3), (2000, 3001, 2)])
+def test_normalize_any_width(rows, cols, n, t, w_dtype):
+    """Psi per active row against the oracle at 1e-5 (fp32 sums), M_t to its
+    rounding, and the G update of odd widths."""
+    import torch
+    from paper_2609_36692_gb300 import normpre as C
+    from paper_2609_36692_gb300.optim import NormPre
+    cs = S.custom_config("width_%dx%d" % (rows, cols), [(rows, cols)] * n, g_dtype="bf16", w_dtype=w_dtype,
+                         row_sigma=1.0, col_sigma=1.0)
+    mats = [S.make_matrix(cs, i) for i in range(n)]
+    W, G, M = to_device(mats, "bf16", w_dtype)
+    opt = NormPre([(rows, cols)] * n, [w_dtype] * n, ["bf16"] * n, variant=C.NORMPRE_L, precision=1, rank=4,
+                  oversample=4)
+    opt.step(t, 0.02, W, G, M)
+    torch.cuda.synchronize()
+    opt.status()
+    for i in range(n):
+        m = mats[i]["M"].astype(np.float64) * f32(0.95) + mats[i]["G"]
+        assert np.all(np.abs(to_host(M[i]) - m) <= 2.5e-7 * np.abs(m) + 1e-30)
+        x, w = (m, mats[i]["W"].astype(np.float64)) if t == 0 else (m.T, mats[i]["W"].astype(np.float64).T)
+        x = x - (x * w).sum(1, keepdims=True) * w
+        nrm = np.linalg.norm(x, axis=1, keepdims=True)
+        psi = opt.read(i, C.NORMPRE_BUF_PSI).astype(np.float64)
+        assert max_row_rel(psi if t == 0 else psi.T, x / nrm) <= 1e-5
+        assert int(opt.read(i, C.NORMPRE_BUF_STATS)[0][1]) == x.shape[0]
+    opt.close()
+
+
+@pytest.mark.parametrize("w_dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("rows,cols", [(1, 5), (37, 1), (9, 255), (50, 2049), (300, 257)])
+def test_update_g_any_width(rows, cols, w_dtype):
+    """The RMS-matched update from the library's own T: one fp32 rounding."""
+    import torch
+    from paper_2609_36692_gb300 import normpre as C
+    from paper_2609_36692_gb300.optim import NormPre
+    cs = S.custom_config("upd_%dx%d" % (rows, cols), [(rows, cols)], g_dtype="bf16", w_dtype=w_dtype)
+    mats = [S.make_matrix(cs, 0)]
+    W, G, M = to_device(mats, "bf16", w_dtype)
+    opt = NormPre([(rows, cols)], [w_dtype], ["bf16"])
+    opt.step(0, 0.02, W, G, M)
+    torch.cuda.synchronize()
+    opt.status()
+    T = opt.read(0, C.NORMPRE_BUF_T).astype(np.float64)
+    w0 = mats[0]["W"].astype(np.float64)
+    ref = w0 - f32(0.02) * (f32(0.2) * T / np.sqrt((T * T).mean()) + f32(0.1) * w0)
+    tol = 1e-6 if w_dtype == "f32" else 2.0 ** -8   # fp32 fma and scale; half a bf16 spacing, doubled for ties
+    assert np.all(np.abs(to_host(W[0]) - ref) <= tol * (np.abs(ref) + 0.004))
+    opt.close()
+
+
