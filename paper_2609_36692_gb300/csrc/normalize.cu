@@ -10,7 +10,7 @@
 // Column-active steps (k = 1): the reduction runs down the columns of the
 // row-major layout.  Pass A streams G, M_{t-1}, W once, writes M_t and per-
 // (row block, column) partial sums of ||m||^2, <m, w> and ||w||^2; a small
-// pass folds the partials (in fp64, fixed order, no atomics on floats) into
+// pass folds the partials (error-free, fixed order, no atomics on floats) into
 // a_j = <m_j, w_j> and 1/||x_j|| with ||x||^2 = ||m||^2 - a^2 (2 - ||w||^2);
 // pass B re-reads M_t and W and writes Psi.
 //
@@ -36,6 +36,8 @@ namespace normpre {
 
 constexpr int kColApplyRB = 64;   // rows per block of pass B (16 where that leaves SMs idle)
 constexpr int kColThreads = 256;  // 32 column chunks of 8 x 8 row lanes
+
+__device__ __forceinline__ float2* col_pairs(const NormLaunch& a) { return reinterpret_cast<float2*>(a.col_part); }
 
 // c_i of the tangent step for mode 0 relaxed, 1 none, 2 strict (mw = <m_i, w_i>,
 // ww = ||w_i||^2).
@@ -215,7 +217,8 @@ __global__ void __launch_bounds__(256) k_norm_rows_scalar(const __grid_constant_
 }
 
 // ---------------------------------------------------------------------------
-// column-active pass A: momentum + column partial sums
+// column-active pass A: momentum + column partial sums (three pairs s + e per
+// row block and column, 8 bytes each)
 // grid (ceil(cols / 256), nrb, n); thread = (column chunk cc = tid % 32, row lane rl = tid / 32)
 // ---------------------------------------------------------------------------
 template <typename TG, typename TW, bool VEC>
@@ -292,20 +295,22 @@ __global__ void __launch_bounds__(kColThreads) k_norm_cols_stats(const __grid_co
     }
   }
   __syncthreads();
-  // fold the 8 row lanes (fp64, fixed order) and write this block's partials
+  // fold the 8 row lanes (error-free, fixed order) and write this block's
+  // partials: 24 fp64 additions and conversions per column kept the fp64 pipe
+  // busy for 3 us a block
   const int col = threadIdx.x;   // 0..255
   const int64_t j = static_cast<int64_t>(blockIdx.x) * 256 + col;
   if (j < cols) {
-    double s0 = 0, s1 = 0, s2 = 0;
+    PairSum s0, s1, s2;
 #pragma unroll
     for (int l = 0; l < 8; ++l) {
-      s0 += part[l][0][col];
-      s1 += part[l][1][col];
-      s2 += part[l][2][col];
+      s0.add(part[l][0][col]);
+      s1.add(part[l][1][col]);
+      s2.add(part[l][2][col]);
     }
     const int64_t nrb = gridDim.y;
-    double* p = a.col_part + ((static_cast<int64_t>(b) * nrb + rb) * cols + j) * 3;
-    p[0] = s0; p[1] = s1; p[2] = s2;
+    float2* p = col_pairs(a) + ((static_cast<int64_t>(b) * nrb + rb) * cols + j) * 3;
+    p[0] = make_float2(s0.s, s0.e); p[1] = make_float2(s1.s, s1.e); p[2] = make_float2(s2.s, s2.e);
   }
 }
 
@@ -314,20 +319,23 @@ __global__ void __launch_bounds__(kColThreads) k_norm_cols_stats(const __grid_co
 // stage 1 (strict): a_j = <m_j, w_j> / ||w_j||^2 only.
 // stage 2 (strict): ||x_j||^2 from the direct sums of k_norm_cols_xsq (slot 1),
 // ||m_j||^2 from pass A (slot 0), a_j kept.
-__global__ void __launch_bounds__(256) k_norm_cols_final(const __grid_constant__ NormLaunch a, int nrb, int stage) {
-  __shared__ float red[32];
+// One warp per 32 columns: the few fp64 operations of a column spread over all
+// SMs.
+__global__ void __launch_bounds__(32) k_norm_cols_final(const __grid_constant__ NormLaunch a, int nrb, int stage) {
   const int b = blockIdx.y;
   const int64_t cols = a.cols;
-  const int64_t j = static_cast<int64_t>(blockIdx.x) * 256 + threadIdx.x;
+  const int64_t j = static_cast<int64_t>(blockIdx.x) * 32 + threadIdx.x;
   float nz = 0.f;
   if (j < cols) {
-    double s0 = 0, s1 = 0, s2 = 0;
-    const double* p = a.col_part + (static_cast<int64_t>(b) * nrb * cols + j) * 3;
+    PairSum p0, p1, p2;
+    const float2* p = col_pairs(a) + (static_cast<int64_t>(b) * nrb * cols + j) * 3;
 #pragma unroll 8
     for (int rb = 0; rb < nrb; ++rb) {
-      s0 += p[0]; s1 += p[1]; s2 += p[2];
+      const float2 v0 = p[0], v1 = p[1], v2 = p[2];
+      p0.add(PairSum{v0.x, v0.y}); p1.add(PairSum{v1.x, v1.y}); p2.add(PairSum{v2.x, v2.y});
       p += cols * 3;
     }
+    const double s0 = p0.value(), s1 = p1.value(), s2 = p2.value();
     float2* out = a.col_coef + static_cast<int64_t>(b) * cols + j;
     if (stage == 1) {
       // strict: only the projection coefficient; the norm comes from the direct pass
@@ -350,7 +358,7 @@ __global__ void __launch_bounds__(256) k_norm_cols_final(const __grid_constant__
       if (!isfinite(d2) || !isfinite(aa)) raise_flag(a.flags, kFlagNonfinite);
     }
   }
-  nz = block_sum(nz, red);
+  nz = warp_sum(nz);
   if (threadIdx.x == 0 && nz > 0.f) atomicAdd(&a.count[a.mat_id[b]], static_cast<int>(nz));
 }
 
@@ -410,10 +418,10 @@ __global__ void __launch_bounds__(kColThreads) k_norm_cols_xsq(const __grid_cons
   const int col = threadIdx.x;
   const int64_t j = static_cast<int64_t>(blockIdx.x) * 256 + col;
   if (j < cols) {
-    double s = 0;
+    PairSum s;
 #pragma unroll
-    for (int l = 0; l < 8; ++l) s += part[l][col];
-    a.col_part[((static_cast<int64_t>(b) * gridDim.y + rb) * cols + j) * 3 + 1] = s;
+    for (int l = 0; l < 8; ++l) s.add(part[l][col]);
+    col_pairs(a)[((static_cast<int64_t>(b) * gridDim.y + rb) * cols + j) * 3 + 1] = make_float2(s.s, s.e);
   }
 }
 
@@ -587,14 +595,14 @@ cudaError_t launch_normalize_cols(const NormLaunch& a, cudaStream_t s) {
     if (e != cudaSuccess) return e;
     if (a.tangent == 2) {
       // strict: the coefficient first, then ||x_j||^2 summed from x itself
-      k_norm_cols_final<<<dim3(grid.x, a.n), 256, 0, s>>>(a, nrb, 1);
+      k_norm_cols_final<<<dim3(static_cast<unsigned>(cdiv(a.cols, 32)), a.n), 32, 0, s>>>(a, nrb, 1);
       if ((e = cudaGetLastError()) != cudaSuccess) return e;
       if (vec) k_norm_cols_xsq<TW, true><<<grid, kColThreads, 0, s>>>(a);
       else k_norm_cols_xsq<TW, false><<<grid, kColThreads, 0, s>>>(a);
       if ((e = cudaGetLastError()) != cudaSuccess) return e;
-      k_norm_cols_final<<<dim3(grid.x, a.n), 256, 0, s>>>(a, nrb, 2);
+      k_norm_cols_final<<<dim3(static_cast<unsigned>(cdiv(a.cols, 32)), a.n), 32, 0, s>>>(a, nrb, 2);
     } else {
-      k_norm_cols_final<<<dim3(grid.x, a.n), 256, 0, s>>>(a, nrb, 0);
+      k_norm_cols_final<<<dim3(static_cast<unsigned>(cdiv(a.cols, 32)), a.n), 32, 0, s>>>(a, nrb, 0);
     }
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;

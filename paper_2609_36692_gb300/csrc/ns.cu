@@ -645,25 +645,10 @@ __global__ void k_scale_from_count(const ScaleArgs a) {
 // k_ns_load: X [rows][cols] -> the padded first buffer (zeros past rows and
 // cols), or nothing when `dst` is null (the products then read X itself), and
 // per CTA the sum of squares of its rows.  Bound by HBM (X read, X written);
-// the sums run in fp32 pairs with error-free additions (TwoSum, and the
-// product's own error for fp32 X; x * x of a bf16 x is exact), about 2^-46
-// relative, because fp64 runs at 1/64 of the fp32 rate here: one 512-thread
+// the sums run in fp32 pairs (PairSum): one 512-thread
 // CTA per matrix summing in fp64 took 2256 us on 4 x 1024 x 4096.  Where a
 // square could overflow or vanish in fp32 the CTA sums its rows in fp64.
 // ---------------------------------------------------------------------------
-struct PairSum {
-  float s = 0.f, e = 0.f;
-  __device__ __forceinline__ void add_square(float x, bool exact) {
-    const float p = __fmul_rn(x, x);
-    const float t = __fadd_rn(s, p);
-    const float bb = __fadd_rn(t, -s);
-    float err = __fadd_rn(__fadd_rn(s, -__fadd_rn(t, -bb)), __fadd_rn(p, -bb));
-    if (!exact) err = __fadd_rn(err, __fmaf_rn(x, x, -p));
-    e = __fadd_rn(e, err);
-    s = t;
-  }
-};
-
 struct NsCopyArgs {
   const void* src;              // load: X; store: T's buffer
   void* dst;
@@ -707,7 +692,8 @@ __global__ void __launch_bounds__(256) k_ns_load(const __grid_constant__ NsCopyA
       top = fmaxf(top, fabsf(v[e]));
     }
   }
-  double s = (static_cast<double>(ps[0].s) + ps[1].s) + (static_cast<double>(ps[0].e) + ps[1].e);
+  ps[0].add(ps[1]);
+  double s = ps[0].value();
   s = block_sum(s, red);
   top = warp_max(top);
   if ((threadIdx.x & 31) == 0) redf[threadIdx.x >> 5] = top;
