@@ -1213,16 +1213,40 @@ __global__ void __launch_bounds__(256) k_rowmul(const __grid_constant__ RowMulAr
 // ---------------------------------------------------------------------------
 // Parallel cyclic Jacobi (round-robin pairing) of Gamma_Q in fp32, then the
 // descending sort, the selection C and K.  One CTA per matrix.  The thread
-// that owns 2 x 2 block (k, k') of the n/2 x n/2 block grid keeps the players
-// of pairs k and k' in registers (advanced every step), forms both pairs'
-// rotations from the current copy of A itself (every owner of a pair forms
-// the same rotation from the same values), writes J^T A J for its block (rows
+// that owns 2 x 2 block (k, k') of the n/2 x n/2 block grid forms a pair's
+// rotation from the current copy of A itself (every owner of a pair forms the
+// same rotation from the same values), writes J^T A J for its block (rows
 // rotated by pair k, columns by pair k') into the other copy of A and rotates
 // rows k', k' + n/2 of V in pair k's columns: one barrier per rotation step.
-// When l is odd the matrices are padded with a zero row and column whose pair
-// is never rotated.
+// When l is odd the matrices are padded with a zero row and column, whose zero
+// off-diagonal entries rotate nothing.
+//
+// Bound by the instructions and shared-memory accesses of a step (13 warps at
+// l = 40), not by data.  So the pairs' shared-memory offsets come from a table
+// built once (the next step's entry is loaded before the barrier), a thread
+// forms one rotation and takes the other from a lane of its warp, the two
+// copies of A lie a constant apart, the two rows of V that a thread rotates
+// are stored as pairs, a rotation takes two reciprocal square roots and no
+// division, and the off-diagonal mass is summed from the last step's results
+// in registers.  The row stride of A is even: the entries (i, i), and (i, j) of
+// a step's pairs, for which i + j is constant up to the wrap, then lie in
+// different banks (with n + 1 the latter shared four), and the row of pair
+// k + 1 follows that of pair k in the banks.  40 x 40: 135 -> 88 us, 24 x 24:
+// 57 -> 36 us.  (A warp of its own that forms the rotations of the next step
+// during the present one, from the values before it: 93 and 35 us.)
 // ---------------------------------------------------------------------------
-constexpr size_t kJacSmem = 3 * static_cast<size_t>(kLmax) * (kLmax + 1) * sizeof(float);
+// A (two copies, kJacCopy bytes apart, row stride jac_ld), V as [n / 2][n + 1]
+// pairs of rows, the table [n - 1][n / 2] of offsets
+__host__ __device__ constexpr int jac_ld(int n) {
+  // even, at least n, and n / 2 modulo 32 (or one more)
+  const int want = ((n / 2 + 1) & ~1) & 31;
+  return n + ((want - n) & 31);
+}
+constexpr uint32_t kJacCopy = kLmax * jac_ld(kLmax) * sizeof(float);
+inline size_t jacobi_smem(int l) {
+  const size_t n = (l + 1) & ~1;
+  return 2 * kJacCopy + n / 2 * (n + 1) * sizeof(float2) + (n - 1) * (n / 2) * sizeof(uint2);
+}
 struct EigArgs {
   const float* part; int64_t part_bs; int nsplit;   // Gram partials of B^T
   float* ritz; int64_t ritz_bs;      // [l]
@@ -1236,128 +1260,171 @@ struct EigArgs {
   int* flags;
 };
 static_assert(sizeof(EigArgs) + 64 <= 4096, "kernel arguments beyond 4 KB");
-// threads of k_jacobi for width l: one per 2 x 2 block (two each past 1024 blocks)
-constexpr int kJacBlocks = ((kLmax / 2) * (kLmax / 2) + 1023) / 1024;
-inline int64_t jacobi_threads(int l) {
-  const int64_t np = (l + 1) / 2;
-  return std::min<int64_t>(1024, ((np * np + 31) / 32) * 32);
+// threads of k_jacobi for width l: one per 2 x 2 block, two blocks each past
+// 1024 (l > 64)
+inline int jacobi_threads(int l) {
+  const int np = (l + 1) / 2;
+  return std::min(1024, ((np * np + 31) / 32) * 32);
 }
-// the rotation (c, s) that annihilates a_ij: t = tan(theta) is the smaller
-// root of t^2 + 2 t cot(2 theta) - 1 = 0, cot(2 theta) = (a_jj - a_ii) / (2 a_ij)
-__device__ __forceinline__ void jac_rot(float aii, float ajj, float aij, bool pad, float& c, float& s) {
-  // branch-free: both branches of the guard are evaluated, then selected
-  const bool skip = pad || !(fabsf(aij) > 1e-30f);
-  const float th = __fdividef(ajj - aii, 2.f * aij);
-  const float w = fmaf(th, th, 1.f);
-  const float t_far = __fdividef(0.5f, th);    // t -> 1 / (2 cot(2 theta))
-  const float t_near = __fdividef(copysignf(1.f, th), fabsf(th) + w * rsqrtf(w));
-  const float t = fabsf(th) > 1e15f ? t_far : t_near;
-  const float cc = rsqrtf(fmaf(t, t, 1.f));
-  c = skip ? 1.f : cc;
-  s = skip ? 0.f : t * cc;
+__device__ __forceinline__ float rsqrt_ftz(float x) {
+  float y;
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
 }
+// The rotation (c, s) that annihilates a_ij, |theta| <= pi / 4: with
+// d = a_jj - a_ii and h = sqrt(d^2 + 4 a_ij^2), cos 2 theta = |d| / h gives
+// c^2 = (1 + |d| / h) / 2 and |s| = |a_ij| / (h c), with the sign of d a_ij.
+// The last step restores c^2 + s^2 = 1 to rounding: V collects hundreds of
+// rotations.  Entries too small to square (and the padding) rotate nothing.
+__device__ __forceinline__ void jac_rot(float aii, float ajj, float aij, float& c, float& s) {
+  const float d = ajj - aii;
+  const float inv = rsqrt_ftz(fmaf(d, d, 4.f * aij * aij));
+  const float u = fmaf(0.5f * fabsf(d), inv, 0.5f);
+  const float rc = rsqrt_ftz(u);
+  const float c0 = u * rc;
+  const float s1 = aij * inv * rc;
+  const float s0 = __uint_as_float(__float_as_uint(s1) ^ (__float_as_uint(d) & 0x80000000u));
+  const float e = -0.5f * fmaf(s0, s0, fmaf(c0, c0, -1.f));
+  const bool rotate = fabsf(aij) > 1e-18f;
+  c = rotate ? fmaf(e, c0, c0) : 1.f;
+  s = rotate ? fmaf(e, s0, s0) : 0.f;
+}
+// NB: 2 x 2 blocks per thread.  With one (n / 2 <= 32), 32 consecutive threads
+// hold every k' (e mod n / 2), so a thread forms the rotation of its k' and
+// takes that of its k from the lane that formed it.
+template <int NB>
 __global__ void __launch_bounds__(1024) k_jacobi(const __grid_constant__ EigArgs a) {
   extern __shared__ float4 jc_smem4[];
-  float* dsm = reinterpret_cast<float*>(jc_smem4);
+  char* sm = reinterpret_cast<char*>(jc_smem4);
   __shared__ float red[32];
   __shared__ int order[kLmax];
+  __shared__ float gain[kLmax];
   const int b = blockIdx.x, l = a.l, tid = threadIdx.x, nt = blockDim.x;
   const int n = (l + 1) & ~1;          // even number of players (one padding player if l is odd)
   const int npairs = n / 2;
-  const int ld = n + 1;
-  float* cur = dsm;                    // A [n][ld], two copies
-  float* nxt = dsm + n * ld;
-  float* Vm = dsm + 2 * n * ld;        // V [n][ld]
-#define V(i, j) Vm[(i) * ld + (j)]
-  fold_partials(a.part + b * a.part_bs, a.nsplit, l, cur, ld);
+  const int ld = jac_ld(n), ldv = n + 1;
+  float* A0 = reinterpret_cast<float*>(sm);
+  constexpr uint32_t kV = 2 * kJacCopy;
+  float* Vm = reinterpret_cast<float*>(sm + kV);   // row r < n / 2, column c: [2 (r ldv + c)]; row r + n / 2 next to it
+  uint2* table = reinterpret_cast<uint2*>(sm + kV + npairs * ldv * 8);
+  auto vat = [&](int r, int c) -> float& { return r < npairs ? Vm[2 * (r * ldv + c)] : Vm[2 * ((r - npairs) * ldv + c) + 1]; };
+  auto at = [&](uint32_t off) -> float& { return *reinterpret_cast<float*>(sm + off); };
+  auto at2 = [&](uint32_t off) -> float2& { return *reinterpret_cast<float2*>(sm + off); };
+  fold_partials(a.part + b * a.part_bs, a.nsplit, l, A0, ld);
   for (int e = tid; e < n * n; e += nt) {
     const int i = e / n, j = e - (e / n) * n;
-    if (i >= l || j >= l) cur[i * ld + j] = 0.f;
-    V(i, j) = (i == j) ? 1.f : 0.f;
+    if (i >= l || j >= l) A0[i * ld + j] = 0.f;
+    vat(i, j) = (i == j) ? 1.f : 0.f;
+  }
+  // pair k plays (k or 0, n - 1 - k) at step 0; every step moves each player
+  // but player 0 on by one place in 1 .. n - 1.  Entry: byte offsets of rows
+  // i < j in a matrix, and of columns i, j in a row
+  for (int e = tid; e < (n - 1) * npairs; e += nt) {
+    const int step = e / npairs, k = e - step * npairs;
+    auto moved = [&](int p) { return (p - 1 + step) % (n - 1) + 1; };
+    const int p = k == 0 ? 0 : moved(k), q = moved(n - 1 - k);
+    const uint32_t i = static_cast<uint32_t>(min(p, q)), j = static_cast<uint32_t>(max(p, q));
+    table[e] = make_uint2(i * ld * 4 | (j * ld * 4) << 16, i * 4 | (j * 4) << 16);
   }
   __syncthreads();
   // exact symmetry
+  float s2 = 0.f;
   for (int e = tid; e < l * l; e += nt) {
     const int i = e / l, j = e % l;
     if (i < j) {
-      const float v = 0.5f * (cur[i * ld + j] + cur[j * ld + i]);
-      cur[i * ld + j] = v;
-      cur[j * ld + i] = v;
+      const float v = 0.5f * (A0[i * ld + j] + A0[j * ld + i]);
+      A0[i * ld + j] = v;
+      A0[j * ld + i] = v;
+      s2 += 2.f * v * v;
+    } else if (i == j) {
+      s2 += A0[i * ld + i] * A0[i * ld + i];
     }
   }
+  const float frob2 = block_sum(s2, red);
   __syncthreads();
-  float frob2;
-  {
-    float s = 0.f;
-    for (int e = tid; e < l * l; e += nt) {
-      const float v = cur[(e / l) * ld + e % l];
-      s += v * v;
-    }
-    frob2 = block_sum(s, red);
-  }
-  // pair k plays (p, q) = (k or 0, n - 1 - k) at step 0; every step moves
-  // each player but player 0 on by one place in 1 .. n - 1
-  int bk[kJacBlocks], bk2[kJacBlocks];
-  int pa[kJacBlocks], qa[kJacBlocks], pb[kJacBlocks], qb[kJacBlocks];
+  int bk[NB], bk2[NB];
+  bool own[NB];
+  uint32_t vrow[NB];                   // this thread's pair of rows of V
 #pragma unroll
-  for (int it = 0; it < kJacBlocks; ++it) {
+  for (int it = 0; it < NB; ++it) {
     const int e = tid + nt * it;
-    bk[it] = (e < npairs * npairs) ? e / npairs : -1;
-    bk2[it] = (e < npairs * npairs) ? e % npairs : 0;
+    own[it] = e < npairs * npairs;
+    bk[it] = own[it] ? e / npairs : 0;
+    bk2[it] = e % npairs;
+    vrow[it] = kV + static_cast<uint32_t>(bk2[it] * ldv * 8);
   }
-  auto advance = [&](int& p, int& q, int k) {
-    if (k != 0) p = (p == n - 1) ? 1 : p + 1;
-    q = (q == n - 1) ? 1 : q + 1;
+  float so = 0.f;
+  uint2 ta[NB], tb[NB];
+  auto unpack = [](uint2 w) { return make_uint4(w.x & 0xffffu, w.x >> 16, w.y & 0xffffu, w.y >> 16); };
+  // the lane of this warp that forms the rotation of pair bk[0] (lane 0 has
+  // k' = (tid & ~31) mod n / 2)
+  const int src = (bk[0] - (tid & ~31) % npairs + npairs) % npairs;
+  // one rotation step from copy P of A (a constant) into the other; step n - 2
+  // is the sweep's last
+  auto rotate = [&](auto parity, int step) {
+    constexpr uint32_t C0 = decltype(parity)::value ? kJacCopy : 0, C1 = kJacCopy - C0;
+#pragma unroll
+    for (int it = 0; it < NB; ++it) {
+      if (NB == 1 || own[it]) {
+        const uint4 p = unpack(ta[it]), q = unpack(tb[it]);
+        float c, s, c2, sn2;
+        jac_rot(at(q.x + q.z + C0), at(q.y + q.w + C0), at(q.x + q.w + C0), c2, sn2);
+        if (NB == 1) {
+          c = __shfl_sync(0xffffffffu, c2, src);
+          s = __shfl_sync(0xffffffffu, sn2, src);
+        } else {
+          jac_rot(at(p.x + p.z + C0), at(p.y + p.w + C0), at(p.x + p.w + C0), c, s);
+        }
+        if (step < n - 2) {
+          ta[it] = table[(step + 1) * npairs + bk[it]];
+          tb[it] = table[(step + 1) * npairs + bk2[it]];
+        }
+        if (!own[it]) continue;
+        const uint32_t o00 = p.x + q.z, o01 = p.x + q.w, o10 = p.y + q.z, o11 = p.y + q.w;
+        const float a00 = at(o00 + C0), a01 = at(o01 + C0), a10 = at(o10 + C0), a11 = at(o11 + C0);
+        const uint32_t vi = vrow[it] + 2 * p.z, vj = vrow[it] + 2 * p.w;
+        const float2 xi = at2(vi), xj = at2(vj);
+        // columns i2, j2 (A J), then rows i, j (J^T A)
+        const float u0 = c2 * a00 - sn2 * a01, w0 = sn2 * a00 + c2 * a01;
+        const float u1 = c2 * a10 - sn2 * a11, w1 = sn2 * a10 + c2 * a11;
+        const float n00 = c * u0 - s * u1, n10 = s * u0 + c * u1;
+        const float n01 = c * w0 - s * w1, n11 = s * w0 + c * w1;
+        at(o00 + C1) = n00; at(o10 + C1) = n10;
+        at(o01 + C1) = n01; at(o11 + C1) = n11;
+        // V <- V J: rows k2 and k2 + n/2, columns of pair k
+        at2(vi) = make_float2(c * xi.x - s * xj.x, c * xi.y - s * xj.y);
+        at2(vj) = make_float2(s * xi.x + c * xj.x, s * xi.y + c * xj.y);
+        if (step == n - 2) {
+          so = fmaf(n01, n01, fmaf(n10, n10, so));
+          if (bk[it] != bk2[it]) so = fmaf(n00, n00, fmaf(n11, n11, so));
+        }
+      }
+    }
+    __syncthreads();
   };
   int sweep = 0;
   float off = frob2, prev = frob2;
   for (; sweep < a.max_sweeps; ++sweep) {
+    so = 0.f;
 #pragma unroll
-    for (int it = 0; it < kJacBlocks; ++it) {
-      const int k = bk[it] < 0 ? 0 : bk[it], k2 = bk2[it];
-      pa[it] = k; qa[it] = n - 1 - k;
-      pb[it] = k2; qb[it] = n - 1 - k2;
+    for (int it = 0; it < NB; ++it) {
+      ta[it] = table[bk[it]];
+      tb[it] = table[bk2[it]];
     }
-    for (int step = 0; step < n - 1; ++step) {
+    for (int step = 0; step + 1 < n - 1; step += 2) {
+      rotate(std::false_type(), step);
+      rotate(std::true_type(), step + 1);
+    }
+    // n - 1 steps, an odd number: the result goes back to copy 0 (the offsets
+    // are still those of the last step)
+    rotate(std::false_type(), n - 2);
 #pragma unroll
-      for (int it = 0; it < kJacBlocks; ++it) {
-        const int k = bk[it], k2 = bk2[it];
-        if (k >= 0) {
-          const int i = min(pa[it], qa[it]), j = max(pa[it], qa[it]);
-          const int i2 = min(pb[it], qb[it]), j2 = max(pb[it], qb[it]);
-          float c, s, c2, s2;
-          jac_rot(cur[i * ld + i], cur[j * ld + j], cur[i * ld + j], j >= l, c, s);
-          jac_rot(cur[i2 * ld + i2], cur[j2 * ld + j2], cur[i2 * ld + j2], j2 >= l, c2, s2);
-          const float* ri = cur + i * ld;
-          const float* rj = cur + j * ld;
-          const float a00 = ri[i2], a01 = ri[j2], a10 = rj[i2], a11 = rj[j2];
-          // columns i2, j2 (A J), then rows i, j (J^T A)
-          const float u0 = c2 * a00 - s2 * a01, w0 = s2 * a00 + c2 * a01;
-          const float u1 = c2 * a10 - s2 * a11, w1 = s2 * a10 + c2 * a11;
-          float* ni = nxt + i * ld;
-          float* nj = nxt + j * ld;
-          ni[i2] = c * u0 - s * u1; nj[i2] = s * u0 + c * u1;
-          ni[j2] = c * w0 - s * w1; nj[j2] = s * w0 + c * w1;
-          // V <- V J: rows k2 and k2 + n/2, columns of pair k
-#pragma unroll
-          for (int h = 0; h < 2; ++h) {
-            float* vr = Vm + (k2 + h * npairs) * ld;
-            const float vi = vr[i], vj = vr[j];
-            vr[i] = c * vi - s * vj;
-            vr[j] = s * vi + c * vj;
-          }
-          advance(pa[it], qa[it], k);
-          advance(pb[it], qb[it], k2);
-        }
+    for (int it = 0; it < NB; ++it)
+      if (own[it]) {
+        const uint4 p = unpack(ta[it]), q = unpack(tb[it]);
+        at(p.x + q.z) = at(p.x + q.z + kJacCopy); at(p.x + q.w) = at(p.x + q.w + kJacCopy);
+        at(p.y + q.z) = at(p.y + q.z + kJacCopy); at(p.y + q.w) = at(p.y + q.w + kJacCopy);
       }
-      __syncthreads();
-      float* t = cur; cur = nxt; nxt = t;
-    }
-    float so = 0.f;
-    for (int e = tid; e < l * l; e += nt) {
-      const int i = e / l, j = e % l;
-      if (i != j) so += cur[i * ld + j] * cur[i * ld + j];
-    }
     prev = off;
     off = block_sum(so, red);
     // converged, or stalled at the fp32 rounding floor (~ l^2 (u ||A||)^2):
@@ -1365,48 +1432,61 @@ __global__ void __launch_bounds__(1024) k_jacobi(const __grid_constant__ EigArgs
     // off-diagonal mass once it is tiny has reached that floor
     if (off <= 1e-12f * frob2 || (off <= 1e-9f * frob2 && off > 0.5f * prev)) { ++sweep; break; }
   }
-#define A(i, j) cur[(i) * ld + (j)]
+  const float* Af = A0;
+  float* Zs = reinterpret_cast<float*>(sm + kJacCopy);   // Z, column c at [c * n]
   if (tid == 0 && sweep >= a.max_sweeps && off > 1e-8f * frob2) raise_flag(a.flags, kFlagNumeric);
   // sort eigenvalues descending, ties by lower index (stable)
+  float* ritz = a.ritz + b * a.ritz_bs;
   for (int i = tid; i < l; i += nt) {
-    const float li = A(i, i);
+    const float li = Af[i * ld + i];
     int pos = 0;
+#pragma unroll 8
     for (int j = 0; j < l; ++j) {
-      const float lj = A(j, j);
+      const float lj = Af[j * ld + j];
       if (lj > li || (lj == li && j < i)) ++pos;
     }
     order[pos] = i;
+    ritz[pos] = li;
+    gain[pos] = rsqrtf(li) - 1.f;
   }
   __syncthreads();
+  // C: the first min(r, l) values down to the last above one
   const int rr = min(a.rank, l);
-  float* ritz = a.ritz + b * a.ritz_bs;
+  int nc = 0;
+  while (nc < rr && Af[order[nc] * ld + order[nc]] > 1.f) ++nc;
   float* z = a.z + b * a.z_bs;
-  for (int c = tid; c < l; c += nt) ritz[c] = A(order[c], order[c]);
   for (int e = tid; e < l * l; e += nt) {
-    const int r = e / l, c = e % l;
-    z[e] = V(r, order[c]);
+    const int r = e / l, c = e - r * l;
+    const float v = vat(r, order[c]);
+    z[e] = v;
+    Zs[c * n + r] = v;
   }
-  // K = sum_{c in C} (lam_c^{-1/2} - 1) z_c z_c^T
+  __syncthreads();
+  // K = sum_{c in C} (lam_c^{-1/2} - 1) z_c z_c^T, symmetric entry for entry
   float* km = a.kmat + b * a.k_bs;
-  for (int e = tid; e < l * l; e += nt) {
-    const int r = e / l, s = e % l;
-    float acc = 0.f;
-    for (int c = 0; c < rr; ++c) {
-      const float lam = A(order[c], order[c]);
-      if (!(lam > 1.f)) break;       // descending: the first lam <= 1 ends C
-      acc = fmaf(rsqrtf(lam) - 1.f, V(r, order[c]) * V(s, order[c]), acc);
+#pragma unroll
+  for (int it = 0; it < NB; ++it) {
+    if (!own[it]) continue;
+    const int r = 2 * bk[it], q = 2 * bk2[it];
+    float k00 = 0.f, k01 = 0.f, k10 = 0.f, k11 = 0.f;
+#pragma unroll 4
+    for (int c = 0; c < nc; ++c) {
+      const float2 zr = *reinterpret_cast<const float2*>(Zs + c * n + r);
+      const float2 zq = *reinterpret_cast<const float2*>(Zs + c * n + q);
+      const float g = gain[c];
+      k00 = fmaf(g, zr.x * zq.x, k00); k01 = fmaf(g, zr.x * zq.y, k01);
+      k10 = fmaf(g, zr.y * zq.x, k10); k11 = fmaf(g, zr.y * zq.y, k11);
     }
-    km[e] = acc;
+    km[r * l + q] = k00;
+    if (q + 1 < l) km[r * l + q + 1] = k01;
+    if (r + 1 < l) {
+      km[(r + 1) * l + q] = k10;
+      if (q + 1 < l) km[(r + 1) * l + q + 1] = k11;
+    }
   }
   if (tid == 0) {
-    int nc = 0;
     float excess = 0.f;
-    for (int c = 0; c < rr; ++c) {
-      const float lam = A(order[c], order[c]);
-      if (!(lam > 1.f)) break;
-      ++nc;
-      excess += lam - 1.f;
-    }
+    for (int c = 0; c < nc; ++c) excess += Af[order[c] * ld + order[c]] - 1.f;
     const float mprime = static_cast<float>(a.count[a.mat_id[b]]);
     float* st = a.stats + b * a.stats_bs;
     st[0] = static_cast<float>(a.k_orient);
@@ -1418,8 +1498,6 @@ __global__ void __launch_bounds__(1024) k_jacobi(const __grid_constant__ EigArgs
     st[6] = static_cast<float>(a.m_a);
     st[7] = static_cast<float>(sweep);
   }
-#undef A
-#undef V
 }
 
 
@@ -1967,7 +2045,8 @@ cudaError_t sketch_group_alloc(SketchGroup& g, int rank, int oversample, std::ve
     if (g.psi_bf16 && (e = alloc(&g.vb, static_cast<size_t>(g.batch) * g.vb_bs * sizeof(uint16_t)))) return e;
   }
   // the largest Jacobi footprint, so that groups of any width can share the kernel
-  cudaFuncSetAttribute(k_jacobi, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kJacSmem));
+  cudaFuncSetAttribute(k_jacobi<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(jacobi_smem(64)));
+  cudaFuncSetAttribute(k_jacobi<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(jacobi_smem(kLmax)));
   return cudaGetLastError();
 }
 
@@ -2219,10 +2298,8 @@ cudaError_t run_sketch_group(SketchGroup& g, const SketchParams& p, const int* m
       ea.m_a = m_a; ea.n_a = n_a;
       ea.max_sweeps = p.max_sweeps;
       ea.flags = flags;
-      const int jthreads = static_cast<int>(jacobi_threads(l));
-      const int nj = (l + 1) & ~1;
-      const size_t jsmem = 3 * static_cast<size_t>(nj) * (nj + 1) * sizeof(float);
-      k_jacobi<<<B, jthreads, jsmem, s>>>(ea);
+      if (l <= 64) k_jacobi<1><<<B, jacobi_threads(l), jacobi_smem(l), s>>>(ea);
+      else k_jacobi<2><<<B, jacobi_threads(l), jacobi_smem(l), s>>>(ea);
       NP_CHECK();
     }
   }
