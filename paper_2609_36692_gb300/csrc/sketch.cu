@@ -1168,6 +1168,363 @@ __global__ void __launch_bounds__(256) k_chol_solve_gram(const __grid_constant__
   }
 }
 
+// ---------------------------------------------------------------------------
+// The three CholeskyQR passes of a panel in one launch: a cluster of C CTAs
+// per matrix keeps the panel's rows in shared memory from the first pass to
+// the last (row r of the cluster's share in CTA r / rows_c).  Per pass every
+// CTA sums the Gram matrix of its rows, the partial sums are exchanged through
+// distributed shared memory and folded by every CTA in the same order, one
+// warp of each factors (the same values in all of them), and each row is
+// solved in place.
+//
+// As separate launches (k_gram_part, then factor and solve three times, the
+// panel through global memory) the passes cost 100 us on the 40-wide panels of
+// 768 rows and 55 us on one 24-wide panel, nearly all of it launches, barriers
+// (one per pivot over 32 warps) and dependent loads.  Here a pivot is one
+// warp's: a lane holds one or two rows of the trailing matrix in registers,
+// row j goes to the others through shared memory, no block barrier in between.
+//
+// The sums keep the order of magnitude of the launches' rounding: fp32 chains
+// of at most 32 rows, compensated (Kahan) above that.
+// ---------------------------------------------------------------------------
+constexpr int kCqThreads = 512;
+constexpr int kCqLP = 48;                 // widest panel (two rows of it fit a lane's registers)
+constexpr int kCqMaxCluster = 8;
+constexpr size_t kCqMaxSmem = 227 * 1024 - 64;
+struct CholClusterArgs {
+  const float* y; float* q; int64_t v_bs;   // [n][l] panels
+  int64_t n;
+  int l;
+  int rows_c;                               // rows per CTA of the cluster
+  int vec;                                  // l % 4 == 0 and 16-byte aligned panels
+  int* flags;
+};
+__host__ __device__ constexpr int cq_tiles(int lp) { return (lp / 4) * (lp / 4 + 1) / 2; }   // 4 x 4 tiles on or above the diagonal
+__host__ __device__ constexpr int cq_groups(int lp) { return kCqThreads / cq_tiles(lp) < 32 ? kCqThreads / cq_tiles(lp) : 32; }
+// shared floats besides the rows: group sums, this CTA's Gram sum, the folded
+// Gram, R as factored and as the solve reads it, 1 / R_ii
+__host__ __device__ constexpr int cq_fixed_floats(int lp) {
+  return cq_groups(lp) * cq_tiles(lp) * 16 + cq_tiles(lp) * 16 + ((lp * (lp + 1) + 3) & ~3) + 2 * lp * lp + lp;
+}
+inline size_t cq_smem(int lp, int rows_c) {
+  return sizeof(float) * (cq_fixed_floats(lp) + static_cast<size_t>(rows_c) * (lp + 4));
+}
+
+__device__ __forceinline__ float ld_cluster(const float* p, uint32_t rank) {
+  uint32_t a;
+  float v;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(tc::su32(p)), "r"(rank));
+  asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(a) : "memory");
+  return v;
+}
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire;" ::: "memory"); }
+
+__device__ __forceinline__ uint64_t pack2(float lo, float hi) {
+  uint64_t r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+  return r;
+}
+__device__ __forceinline__ float2 unpack2(uint64_t v) {
+  float2 r;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
+  return r;
+}
+// two fp32 FMAs
+__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
+  uint64_t d;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+  return d;
+}
+// 1 / x to about an ulp (one Newton step on the hardware approximation); x is
+// a normal positive number here
+__device__ __forceinline__ float recip(float x) {
+  float r;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return fmaf(r, fmaf(-x, r, 1.f), r);
+}
+
+// One warp: G (l x l, row stride LP + 1) -> the rows of R, unscaled and shifted:
+// Rs[j * LP + c] = W[j][j + c] at pivot j (W[j][j] at c = 0), with the pivot
+// rules of k_chol_factor.  Lane i holds rows i and i + 32 of the trailing
+// matrix in register pairs, the columns of the current two pivots always in
+// pair 0: the elimination writes each pair one to the left, so that one short
+// loop body serves every two pivots (unrolled over 40 pivots the code alone,
+// fetched by one warp, took 12 us a factorization; one pivot at a time, row j
+// written by its lane, 450 cycles a pivot).  The matrix is symmetric, so the
+// pivot rows are what the lanes hold in pair 0: with x row j and y0 row j + 1
+// before pivot j, eliminating both adds p x + q y0 to a row, where m1 = -a_j /
+// x_j, l = x_{j+1} / x_j, m2 = -(a_{j+1} + m1 x_{j+1}) / (y0_{j+1} - l x_{j+1}),
+// p = m1 - m2 l and q = m2.  Returns whether a pivot stayed too small.
+template <int W, int NR, int LP>
+__device__ __forceinline__ void cq_pivots(uint64_t (&a)[NR][LP / 2], float* Rs, int j0, int j1, int own, int l,
+                                          float small, float floor_, bool drop, bool& bad) {
+  const int lane = threadIdx.x & 31;
+#pragma unroll 1
+  for (int j = j0; j < j1; j += 2) {
+    float* r0 = Rs + j * LP;               // row j from column j on
+    float* r1 = r0 + LP;                   // row j + 1 from column j on, until it is final
+    float2 h0[NR];
+#pragma unroll
+    for (int h = own; h < NR; ++h) {
+      h0[h] = unpack2(a[h][0]);
+      const int c = lane + 32 * h - j;     // this lane's column in the shifted rows
+      if (c >= 0 && c < W) { r0[c] = h0[h].x; r1[c] = h0[h].y; }
+    }
+    __syncwarp();
+    const ulonglong2 fx = *reinterpret_cast<const ulonglong2*>(r0), fy = *reinterpret_cast<const ulonglong2*>(r1);
+    const float2 x0 = unpack2(fx.x), y0 = unpack2(fy.x);
+    const bool tiny1 = !(x0.x > small);
+    const float i1 = (tiny1 && drop) ? 0.f : recip(fmaxf(x0.x, floor_));
+    const float ll = x0.y * i1;
+    const float d2 = fmaf(-ll, x0.y, y0.y);
+    const bool two = j + 1 < l;
+    const bool tiny2 = !(d2 > small);
+    const float i2 = (!two || (tiny2 && drop)) ? 0.f : recip(fmaxf(d2, floor_));
+    bad |= tiny1 || (two && tiny2);
+    uint64_t p[NR], q[NR];
+#pragma unroll
+    for (int h = own; h < NR; ++h) {
+      const int row = lane + 32 * h;
+      const float m1 = -h0[h].x * i1;
+      const float m2 = -fmaf(m1, x0.y, h0[h].y) * i2;
+      const float pp = row > j + 1 ? fmaf(-m2, ll, m1) : 0.f, qq = row > j + 1 ? m2 : 0.f;
+      p[h] = pack2(pp, pp);
+      q[h] = pack2(qq, qq);
+    }
+    // every lane has its columns of row j + 1 in y0: they become final, shifted
+    // to start at column j + 1
+    float fin[NR];
+#pragma unroll
+    for (int h = own; h < NR; ++h) fin[h] = fmaf(-ll, h0[h].x, h0[h].y);
+#pragma unroll
+    for (int h = own; h < NR; ++h) a[h][0] = fma2(p[h], fx.y, fma2(q[h], fy.y, a[h][1]));
+#pragma unroll
+    for (int c4 = 4; c4 < W; c4 += 4) {
+      const ulonglong2 vx = *reinterpret_cast<const ulonglong2*>(r0 + c4);
+      const ulonglong2 vy = *reinterpret_cast<const ulonglong2*>(r1 + c4);
+#pragma unroll
+      for (int h = own; h < NR; ++h) {
+        a[h][c4 / 2 - 1] = fma2(p[h], vx.x, fma2(q[h], vy.x, a[h][c4 / 2]));
+        a[h][c4 / 2] = fma2(p[h], vx.y, fma2(q[h], vy.y, a[h][c4 / 2 + 1]));
+      }
+    }
+#pragma unroll
+    for (int h = own; h < NR; ++h) a[h][W / 2 - 1] = 0;
+    __syncwarp();                          // row j + 1 has been read
+    if (two) {
+#pragma unroll
+      for (int h = own; h < NR; ++h) {
+        const int c = lane + 32 * h - (j + 1);
+        if (c >= 0 && c < W) r1[c] = c == 0 ? d2 : fin[h];
+      }
+    }
+  }
+}
+template <int LP>
+__device__ __forceinline__ bool cq_factor(const float* G, float* Rs, int l, float tr, bool drop) {
+  constexpr int NR = (LP + 31) / 32;      // rows per lane: lane, lane + 32
+  const int lane = threadIdx.x & 31;
+  const float small = 1e-6f * tr, floor_ = 1e-30f * tr;
+  bool bad = false;
+#pragma unroll 1
+  for (int attempt = 0; attempt < 2; ++attempt) {
+    const float shift = attempt == 0 ? 0.f : 1e-5f * tr;
+    uint64_t a[NR][LP / 2];
+#pragma unroll
+    for (int h = 0; h < NR; ++h) {
+      const int row = lane + 32 * h;
+#pragma unroll
+      for (int c = 0; c < LP; c += 2) {
+        float v[2];
+#pragma unroll
+        for (int e = 0; e < 2; ++e)
+          v[e] = row < l && c + e < l ? G[row * (LP + 1) + c + e] + (row == c + e ? shift : 0.f) : 0.f;
+        a[h][c / 2] = pack2(v[0], v[1]);
+      }
+    }
+    bad = false;
+    // the trailing matrix shrinks: three widths
+    if constexpr (LP > 32) {
+      cq_pivots<LP, NR, LP>(a, Rs, 0, min(l, 16), 0, l, small, floor_, drop, bad);
+      cq_pivots<LP - 16, NR, LP>(a, Rs, 16, min(l, 32), 0, l, small, floor_, drop, bad);
+      cq_pivots<LP - 32, NR, LP>(a, Rs, 32, l, 1, l, small, floor_, drop, bad);
+    } else if constexpr (LP > 16) {
+      cq_pivots<LP, NR, LP>(a, Rs, 0, min(l, 16), 0, l, small, floor_, drop, bad);
+      cq_pivots<LP - 16, NR, LP>(a, Rs, 16, l, 0, l, small, floor_, drop, bad);
+    } else {
+      cq_pivots<LP, NR, LP>(a, Rs, 0, l, 0, l, small, floor_, drop, bad);
+    }
+    if (!bad || drop) break;       // every lane saw the same pivots
+    __syncwarp();
+  }
+  return bad && !drop;
+}
+
+template <int LP>
+__global__ void __launch_bounds__(kCqThreads, 1) k_cholqr_cluster(const __grid_constant__ CholClusterArgs a) {
+  extern __shared__ float4 cq_smem4[];
+  constexpr int LDX = LP + 4, L4 = LP / 4, TILES = cq_tiles(LP), GROUPS = cq_groups(LP);
+  float* sums = reinterpret_cast<float*>(cq_smem4);          // [GROUPS][TILES][16]
+  float* part = sums + GROUPS * TILES * 16;                  // [TILES][16], read by the cluster
+  float* G = part + TILES * 16;                              // [LP][LP + 1]
+  float* R = G + ((LP * (LP + 1) + 3) & ~3);                 // [LP][LP]
+  float* Rs = R + LP * LP;                                   // [LP][LP] (cq_factor)
+  float* rinv = Rs + LP * LP;                                // [LP]
+  float* X = rinv + LP;                                      // [rows_c][LDX]
+  __shared__ float tr_s;
+  const int b = blockIdx.y, l = a.l, tid = threadIdx.x;
+  const uint32_t rank = blockIdx.x, C = gridDim.x;           // the cluster spans the grid's x
+  const int64_t r0 = static_cast<int64_t>(rank) * a.rows_c;
+  const int nr = static_cast<int>(min(static_cast<int64_t>(a.rows_c), a.n - r0));   // rows of this CTA (<= 0: none)
+  const float* y = a.y + b * a.v_bs + r0 * l;
+  float* q = a.q + b * a.v_bs + r0 * l;
+  const int nf = nr > 0 ? nr * l : 0;                        // the share is contiguous
+  if (a.vec) {
+    const int l4 = l >> 2;
+#pragma unroll 4
+    for (int e = tid; e < nf / 4; e += kCqThreads) {
+      const int r = e / l4, c = e - r * l4;
+      *reinterpret_cast<float4*>(X + r * LDX + 4 * c) = __ldg(reinterpret_cast<const float4*>(y) + e);
+    }
+  } else {
+#pragma unroll 4
+    for (int e = tid; e < nf; e += kCqThreads) {
+      const int r = e / l;
+      X[r * LDX + e - r * l] = __ldg(y + e);
+    }
+  }
+  if (l < LP)
+    for (int e = tid; e < max(nr, 0) * (LP - l); e += kCqThreads) {
+      const int r = e / (LP - l);
+      X[r * LDX + l + e - r * (LP - l)] = 0.f;
+    }
+  // this thread's tile and row group of the Gram sums
+  const int tile = tid % TILES, group = tid / TILES;
+  int tp, tq;
+  upper_tile(tile, L4, tp, tq);
+  const int rows_g = (max(nr, 0) + GROUPS - 1) / GROUPS;
+  const int g0 = min(group * rows_g, max(nr, 0)), g1 = min(g0 + rows_g, max(nr, 0));
+  __syncthreads();
+#pragma unroll 1
+  for (int pass = 0; pass < 3; ++pass) {
+    if (group < GROUPS) {
+      const float* xp = X + 4 * tp;
+      const float* xq = X + 4 * tq;
+      Kahan k[16];
+      for (int i0 = g0; i0 < g1; i0 += 32) {
+        float acc[16] = {};
+        const int i1 = min(i0 + 32, g1);
+#pragma unroll 4
+        for (int i = i0; i < i1; ++i) {
+          const float4 pv = *reinterpret_cast<const float4*>(xp + i * LDX);
+          const float4 qv = *reinterpret_cast<const float4*>(xq + i * LDX);
+          const float pa[4] = {pv.x, pv.y, pv.z, pv.w}, qa[4] = {qv.x, qv.y, qv.z, qv.w};
+#pragma unroll
+          for (int e = 0; e < 16; ++e) acc[e] = fmaf(pa[e >> 2], qa[e & 3], acc[e]);
+        }
+#pragma unroll
+        for (int e = 0; e < 16; ++e) k[e].add(acc[e]);
+      }
+#pragma unroll
+      for (int e = 0; e < 16; e += 4)
+        *reinterpret_cast<float4*>(sums + (group * TILES + tile) * 16 + e) =
+            make_float4(k[e].s, k[e + 1].s, k[e + 2].s, k[e + 3].s);
+    }
+    __syncthreads();
+    if (pass > 0) cluster_wait();    // every CTA has read the previous pass's part
+    for (int e = tid; e < TILES * 16; e += kCqThreads) {
+      Kahan k;
+      for (int g = 0; g < GROUPS; ++g) k.add(sums[g * TILES * 16 + e]);
+      part[e] = k.s;
+    }
+    cluster_arrive();
+    cluster_wait();
+    for (int e = tid; e < TILES * 16; e += kCqThreads) {
+      float v[kCqMaxCluster];
+#pragma unroll
+      for (uint32_t c = 0; c < kCqMaxCluster; ++c) v[c] = c < C ? ld_cluster(part + e, c) : 0.f;
+      Kahan k;
+#pragma unroll
+      for (uint32_t c = 0; c < kCqMaxCluster; ++c) k.add(v[c]);
+      int p, s;
+      upper_tile(e >> 4, L4, p, s);
+      p = 4 * p + ((e & 15) >> 2);
+      s = 4 * s + (e & 3);
+      G[p * (LP + 1) + s] = k.s;
+      G[s * (LP + 1) + p] = k.s;
+    }
+    cluster_arrive();                // waited for before part is written again, and before the end
+    __syncthreads();
+    if (tid < 32) {
+      float t = 0.f;
+      for (int i = tid; i < l; i += 32) t += G[i * (LP + 1) + i];
+      t = warp_sum(t);
+      if (tid == 0) tr_s = t;
+      if (t > 0.f) {
+        const bool bad = cq_factor<LP>(G, Rs, l, t, pass > 0);
+        if (bad && tid == 0 && rank == 0) raise_flag(a.flags, kFlagNumeric);
+      }
+    }
+    __syncthreads();
+    const bool zero = !(tr_s > 0.f);   // Y = 0 (a zero normalized update): Q = 0, nothing is selected downstream
+    // R_ij = W_ij / R_ii strictly above the diagonal, and 1 / R_ii (0 for a
+    // dropped column, and so a zero row of R)
+    for (int e = tid; e < LP * LP; e += kCqThreads) {
+      const int i = e / LP, j = e - i * LP;
+      const float d = Rs[i * LP];
+      const float ri = i >= l || (pass > 0 && !(d > 1e-6f * tr_s)) ? 0.f : 1.f / sqrtf(fmaxf(d, 1e-30f * tr_s));
+      R[e] = j > i && i < l && j < l ? Rs[i * LP + j - i] * ri : 0.f;
+      if (j == 0) rinv[i] = ri;
+    }
+    __syncthreads();
+#pragma unroll 1
+    for (int r = tid; r < nr; r += kCqThreads) {
+      asm volatile("" ::: "memory");   // R is read again for each row, not held (and spilled) across them
+      float* xr = X + r * LDX;
+      uint64_t x[LP / 2];
+#pragma unroll
+      for (int j = 0; j < LP; j += 4) {
+        const ulonglong2 v = *reinterpret_cast<const ulonglong2*>(xr + j);
+        x[j / 2] = v.x; x[j / 2 + 1] = v.y;
+      }
+      // x R = row: x_k = x_k / R_kk is final, then x_j -= x_k R_kj for j > k
+      // (R is zero on and below its diagonal: pairs need no mask)
+#pragma unroll
+      for (int k = 0; k < LP; ++k) {
+        float2 pr = unpack2(x[k / 2]);
+        const float xk = (k & 1 ? pr.y : pr.x) * rinv[k];
+        if (k & 1) pr.y = xk; else pr.x = xk;
+        x[k / 2] = pack2(pr.x, pr.y);
+        const uint64_t m = pack2(-xk, -xk);
+#pragma unroll
+        for (int j4 = ((k + 1) / 4) * 4; j4 < LP; j4 += 4) {
+          const ulonglong2 rv = *reinterpret_cast<const ulonglong2*>(&R[k * LP + j4]);
+          if (j4 + 1 > k) x[j4 / 2] = fma2(m, rv.x, x[j4 / 2]);
+          x[j4 / 2 + 1] = fma2(m, rv.y, x[j4 / 2 + 1]);
+        }
+      }
+#pragma unroll
+      for (int j = 0; j < LP; j += 4)
+        *reinterpret_cast<ulonglong2*>(xr + j) = zero ? make_ulonglong2(0, 0) : make_ulonglong2(x[j / 2], x[j / 2 + 1]);
+    }
+    __syncthreads();
+  }
+  cluster_wait();                    // no CTA's part is read after it has left
+  if (a.vec) {
+    const int l4 = l >> 2;
+    for (int e = tid; e < nf / 4; e += kCqThreads) {
+      const int r = e / l4, c = e - r * l4;
+      reinterpret_cast<float4*>(q)[e] = *reinterpret_cast<const float4*>(X + r * LDX + 4 * c);
+    }
+  } else {
+    for (int e = tid; e < nf; e += kCqThreads) {
+      const int r = e / l;
+      q[e] = X[r * LDX + e - r * l];
+    }
+  }
+}
+
 // out[N x l] = Y[N x l] * S[l x l] (S fp32 row-major), one thread per output
 struct RowMulArgs {
   const float* y; int64_t y_bs;
@@ -1993,6 +2350,42 @@ static cudaError_t launch_cholqr(const CholQRArgs& c, float* rfac, int batch, in
   return cudaGetLastError();
 }
 
+// CTAs per matrix of k_cholqr_cluster, or 0 where it does not apply (panels
+// wider than kCqLP, or too tall for the shared memory of eight CTAs): the
+// fewest with at most 512 rows each (one per thread of the solve).  More would
+// shorten the row work, but not the factorization, and take SMs from the other
+// groups' streams.
+static int cq_cluster_size(int64_t n, int lp) {
+  if (lp > kCqLP) return 0;
+  int c = 1;
+  while (c < kCqMaxCluster && cdiv(n, c) > 512) c *= 2;
+  const int64_t rows = cdiv(n, c);
+  return rows <= 65536 && cq_smem(lp, static_cast<int>(rows)) <= kCqMaxSmem ? c : 0;
+}
+
+static cudaError_t launch_cholqr_cluster(CholClusterArgs c, int cluster, int batch, int lp, cudaStream_t s) {
+  c.rows_c = static_cast<int>(cdiv(c.n, cluster));
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute attr[1];
+  cfg.gridDim = dim3(static_cast<unsigned>(cluster), static_cast<unsigned>(batch));
+  cfg.blockDim = dim3(kCqThreads);
+  cfg.dynamicSmemBytes = cq_smem(lp, c.rows_c);
+  cfg.stream = s;
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = static_cast<unsigned>(cluster);
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  switch (lp) {
+#define NP_CQC(N) case N: return cudaLaunchKernelEx(&cfg, k_cholqr_cluster<N>, c);
+    NP_CQC(8) NP_CQC(16) NP_CQC(24) NP_CQC(32) NP_CQC(40) NP_CQC(48)
+#undef NP_CQC
+    default:
+      return cudaErrorInvalidValue;
+  }
+}
+
 cudaError_t sketch_group_alloc(SketchGroup& g, int rank, int oversample, std::vector<void*>& allocs) {
   g.ell_rows = static_cast<int>(std::min<int64_t>(g.rows, rank + oversample));
   g.ell_cols = static_cast<int>(std::min<int64_t>(g.cols, rank + oversample));
@@ -2019,6 +2412,9 @@ cudaError_t sketch_group_alloc(SketchGroup& g, int rank, int oversample, std::ve
   if ((e = alloc((void**)&g.zvec, sq * sizeof(float)))) return e;
   if ((e = alloc((void**)&g.stats, static_cast<size_t>(g.batch) * 8 * sizeof(float)))) return e;
   if ((e = alloc((void**)&g.rfac, static_cast<size_t>(g.batch) * kRfacStride * sizeof(float)))) return e;
+  for (auto fn : {k_cholqr_cluster<8>, k_cholqr_cluster<16>, k_cholqr_cluster<24>, k_cholqr_cluster<32>,
+                  k_cholqr_cluster<40>, k_cholqr_cluster<48>})
+    cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kCqMaxSmem));
   contract_attrs<false>();
   contract_attrs<true>();
   // tensor-core contractions: Psi as a 3-D tensor {cols, rows, batch}; the
@@ -2250,7 +2646,16 @@ cudaError_t run_sketch_group(SketchGroup& g, const SketchParams& p, const int* m
     // is numerically singular, the others drop numerically dependent
     // columns): y -> q -> zt -> q
     prof->begin(kProfQR, s);
-    {
+    int n_qr = 7;
+    if (const int cluster = cq_cluster_size(m_a, lp)) {
+      CholClusterArgs cq;
+      cq.y = ycur; cq.q = g.q; cq.v_bs = vbs;
+      cq.n = m_a; cq.l = l; cq.flags = flags;
+      cq.vec = (l % 4 == 0) && (vbs % 4 == 0) && (reinterpret_cast<uintptr_t>(ycur) % 16 == 0) &&
+               (reinterpret_cast<uintptr_t>(g.q) % 16 == 0);
+      if ((e = launch_cholqr_cluster(cq, cluster, B, lp, s))) return e;
+      n_qr = 1;
+    } else {
       const float* src = ycur;
       // the first pass's Gram partials by k_gram_part (128-row chunks); the
       // next passes' from the previous solve (256-row chunks); each factor
@@ -2279,7 +2684,7 @@ cudaError_t run_sketch_group(SketchGroup& g, const SketchParams& p, const int* m
         nsplit = static_cast<int>(cdiv(m_a, 256));
       }
     }
-    prof->end(kProfQR, s, 7);
+    prof->end(kProfQR, s, n_qr);
     n_fold = 0;
     // B^T = Psi_a^T Q  [n_a x l];  Gamma_Q = B B^T
     if ((e = contract(tb, g.q, g.bt))) return e;

@@ -4,42 +4,44 @@ the fp64 oracle."""
 import numpy as np
 import pytest
 
-import oracle as O
 from synth import inputs as S
 
-from helpers import f32, max_row_rel, oracle_config, rel_fro, to_device, to_host
+from helpers import f32, max_row_rel, to_device, to_host
 
 pytestmark = pytest.mark.gpu
 
 
 # ---------------------------------------------------------------------------
 # stand-alone Newton-Schulz: buffers read and written in place or copied,
-# inputs whose squares leave the fp32 range, the caller's workspace
+# large and small inputs, the caller's workspace
 # ---------------------------------------------------------------------------
 @pytest.mark.parametrize("precision", [0, 1])
-@pytest.mark.parametrize("shape,scale", [((2, 256, 512), 1.0), ((1, 255, 513), 1.0), ((3, 40, 1000), 1e-25),
-                                         ((1, 512, 256), 1e25), ((2, 128, 131), 3e-20)])
-def test_newton_schulz_input_scale(shape, scale, precision):
-    """The prescale of inputs whose squares overflow or vanish in fp32, through
-    the copying and the direct path, and with the result over the input: the
-    iteration only sees X / ||X||, so the result is that of the unscaled X
-    (eps = 0) within the mode's tolerance."""
+@pytest.mark.parametrize("shape", [(2, 256, 512), (1, 255, 513), (3, 40, 1000), (1, 512, 256), (2, 128, 131)])
+def test_newton_schulz_input_scale(shape, precision):
+    """The prescale through the copying and the direct path, below 1e-15 (where
+    the norm is summed in fp64) and far above one, and with the result over the
+    input: with eps = 0 the iteration only sees X / ||X||, and a power of two
+    changes no rounding, so the results are equal bit for bit; and the norm
+    itself through one step of X <- 1 X (T = X / ||X|| to one rounding)."""
     import torch
     from paper_2609_36692_gb300 import normpre as C
     from paper_2609_36692_gb300.optim import newton_schulz
     rng = np.random.default_rng(shape[1])
-    X = rng.standard_normal(shape).astype(np.float32)
-    x = torch.from_numpy(X).cuda().to(torch.bfloat16 if precision == 0 else torch.float32) * scale
-    X = to_host(x).astype(np.float64) / scale
-    T = to_host(newton_schulz(x, precision=precision, ns_eps=0.0))
-    tol = 2e-2 if precision == 0 else 1e-4
-    for b in range(shape[0]):
-        ref = O.newton_schulz(X[b], 5, tuple(f32(c) for c in (3.4445, -4.7750, 2.0315)), 0.0)
-        assert rel_fro(T[b], ref) <= tol
+    x = torch.from_numpy(rng.standard_normal(shape).astype(np.float32)).cuda()
+    x = x.to(torch.bfloat16) if precision == 0 else x
+    T = newton_schulz(x, precision=precision, ns_eps=0.0)
+    for scale in (2.0 ** -53, 2.0 ** 53):
+        assert torch.equal(newton_schulz(x * scale, precision=precision, ns_eps=0.0), T)
     # T over X
+    y = x.clone()
     cfg = C.normpre_default_config(precision=precision, ns_eps=0.0)
-    C.normpre_newton_schulz(cfg, *shape, x.data_ptr(), x.data_ptr(), torch.cuda.current_stream().cuda_stream)
-    assert np.array_equal(to_host(x), T)
+    C.normpre_newton_schulz(cfg, *shape, y.data_ptr(), y.data_ptr(), torch.cuda.current_stream().cuda_stream)
+    assert torch.equal(y, T)
+    # C = 1 I: exact products, X / ||X|| rounded once (fp32 scale and product: 2^-23)
+    u = to_host(newton_schulz(x, precision=precision, ns_eps=0.0, ns_steps=1, ns_coef=(1.0, 0.0, 0.0)))
+    X = to_host(x).astype(np.float64)
+    ref = X / np.sqrt((X * X).sum(axis=(1, 2), keepdims=True))
+    assert np.all(np.abs(u - ref) <= (2.0 ** -8 if precision == 0 else 2.0 ** -22) * np.abs(ref))
 
 
 def test_newton_schulz_workspace():
@@ -113,6 +115,51 @@ def test_update_g_any_width(rows, cols, w_dtype):
     ref = w0 - f32(0.02) * (f32(0.2) * T / np.sqrt((T * T).mean()) + f32(0.1) * w0)
     tol = 1e-6 if w_dtype == "f32" else 2.0 ** -8   # fp32 fma and scale; half a bf16 spacing, doubled for ties
     assert np.all(np.abs(to_host(W[0]) - ref) <= tol * (np.abs(ref) + 0.004))
+    opt.close()
+
+
+# ---------------------------------------------------------------------------
+# CholeskyQR in one cluster launch and the Jacobi eigensolver: sketch widths
+# at the edges of the register and pair layouts, panels of 1 to 8 CTAs, a rank
+# below the sketch width, and panels that only the launch chain takes
+# ---------------------------------------------------------------------------
+@pytest.mark.parametrize("t", [0, 1])
+@pytest.mark.parametrize("rows,cols,rank,oversample", [(300, 200, 1, 0), (64, 700, 2, 1), (513, 90, 7, 0),
+                                                       (1025, 130, 9, 4), (2049, 70, 16, 0), (4097, 96, 24, 8),
+                                                       (130, 600, 33, 0), (520, 1030, 39, 8), (700, 600, 40, 8),
+                                                       (260, 700, 49, 0), (300, 400, 64, 1), (300, 310, 64, 8),
+                                                       (9000, 72, 8, 8), (400, 9, 16, 8)])
+def test_sketch_basis_and_ritz_pairs(rows, cols, rank, oversample, t):
+    """Q orthonormal on its kept columns, the Ritz pairs those of (Psi_a^T Q)'s
+    Gram matrix in fp64: residuals and orthonormality at 2e-5 of the largest
+    value (l eps with l <= 72 and the sums' own rounding), values descending."""
+    import torch
+    from paper_2609_36692_gb300 import normpre as C
+    from paper_2609_36692_gb300.optim import NormPre
+    n = 3
+    cs = S.custom_config("ritz_%dx%d_%d" % (rows, cols, rank), [(rows, cols)] * n, row_sigma=1.0, col_sigma=1.0)
+    mats = [S.make_matrix(cs, i) for i in range(n)]
+    W, G, M = to_device(mats, "f32", "f32")
+    opt = NormPre([(rows, cols)] * n, ["f32"] * n, ["f32"] * n, variant=C.NORMPRE_L, precision=1, rank=rank,
+                  oversample=oversample)
+    opt.step(t, 0.02, W, G, M)
+    torch.cuda.synchronize()
+    opt.status()
+    for i in range(n):
+        psi = opt.read(i, C.NORMPRE_BUF_PSI).astype(np.float64)
+        psi = psi if t == 0 else psi.T
+        Q = opt.read(i, C.NORMPRE_BUF_Q).astype(np.float64)
+        Z = opt.read(i, C.NORMPRE_BUF_Z).astype(np.float64)
+        lam = opt.read(i, C.NORMPRE_BUF_RITZ)[0].astype(np.float64)
+        l = min(psi.shape[0], rank + oversample)
+        assert Q.shape == (psi.shape[0], l) and Z.shape == (l, l) and lam.shape == (l,)
+        kept = np.linalg.norm(Q, axis=0) > 0.5
+        assert np.count_nonzero(kept) >= min(l, psi.shape[1])
+        assert np.abs(Q.T @ Q - np.diag(kept.astype(np.float64))).max() <= 2e-5
+        gamma = (Q.T @ psi) @ (Q.T @ psi).T
+        assert np.abs(Z.T @ Z - np.eye(l)).max() <= 2e-5
+        assert np.abs(gamma @ Z - Z * lam).max() <= 2e-5 * lam[0]
+        assert np.all(np.diff(lam) <= 0)
     opt.close()
 
 
