@@ -2013,15 +2013,16 @@ __global__ void __launch_bounds__(256) k_apply_l(const __grid_constant__ LApplyA
 // across its 32 lanes, and the kernel is left with the compulsory HBM stream
 // (Psi read, W read and write) instead of l fp32 FMAs per element.
 //
-// Persistent: CTA c takes a contiguous range of units (matrix, row tile,
-// column tile), column tiles fastest, so the Lm tile is split once per row
-// tile.  Warps 0-1 split the panel rows into the shared-memory operands
+// Persistent: CTA c takes a contiguous range of units (matrix, row tile of nt
+// rows, column tile), column tiles fastest, so the Lm tile is split once per
+// row tile.  nt is 256, or less where that leaves SMs idle: one 256 x 1024
+// matrix is 8 units of 256 rows or 32 of 64.  Warps 0-1 split the panel rows into the shared-memory operands
 // (K-major, 128-byte swizzle, 32-wide K atoms), warp 2 issues the MMAs into
 // one of two TMEM accumulators (256 columns each), warps 3-10 drain an
 // accumulator into the weight update while the next unit's operands and MMAs
 // proceed.
 // ---------------------------------------------------------------------------
-constexpr int kAtcRows = 256;                         // W rows per unit (MMA N)
+constexpr int kAtcRows = 256;                         // most W rows per unit (MMA N = nt)
 constexpr int kAtcCols = 128;                         // W columns per unit (MMA M)
 constexpr int kAtcProd = 2, kAtcEpi = 8;
 constexpr int kAtcChunk = 16, kAtcSlots = 3;       // epilogue: rows per chunk, register ring slots
@@ -2033,8 +2034,7 @@ static size_t atc_smem(int natoms) { return 1024 + static_cast<size_t>(natoms) *
 // rows [r0, r0 + R) of a panel (row stride l floats) split into hi / lo
 // swizzled K-major tiles; rows past `nrows` are zero.  Eight 16-byte loads
 // per thread are in flight before the first split.
-template <int R>
-__device__ __forceinline__ void atc_split_rows(const float* panel, int64_t r0, int64_t nrows, int l, uint8_t* hi,
+__device__ __forceinline__ void atc_split_rows(const float* panel, int64_t r0, int64_t nrows, int R, int l, uint8_t* hi,
                                                uint8_t* lo, int atom_bytes, int ptid) {
   constexpr int NT = 32 * kAtcProd, B = 8;
   const int l4 = l >> 2;
@@ -2066,7 +2066,7 @@ __device__ __forceinline__ void atc_split_rows(const float* panel, int64_t r0, i
 }
 
 template <typename TW, typename TP>
-__global__ void __launch_bounds__(kAtcThreads, 1) k_apply_tc(const __grid_constant__ LApplyArgs a, int nmat,
+__global__ void __launch_bounds__(kAtcThreads, 1) k_apply_tc(const __grid_constant__ LApplyArgs a, int nmat, int nt,
                                                               int natoms, int* flags) {
   extern __shared__ uint8_t atc_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(atc_raw) + 1023) & ~uintptr_t(1023));
@@ -2082,15 +2082,15 @@ __global__ void __launch_bounds__(kAtcThreads, 1) k_apply_tc(const __grid_consta
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int64_t rt = (a.rows + kAtcRows - 1) / kAtcRows, ct = (a.cols + kAtcCols - 1) / kAtcCols;
+  const int64_t rt = (a.rows + nt - 1) / nt, ct = (a.cols + kAtcCols - 1) / kAtcCols;
   const int64_t per_mat = rt * ct;
   const int64_t units = per_mat * nmat;
   const int64_t u0 = units * blockIdx.x / gridDim.x, u1 = units * (blockIdx.x + 1) / gridDim.x;
-  // column tiles fastest: consecutive units of a CTA share the 256-row Lm tile
+  // column tiles fastest: consecutive units of a CTA share the Lm tile
   auto unit_of = [&](int64_t u, int& b, int64_t& i0, int64_t& j0) {
     b = static_cast<int>(u / per_mat);
     const int64_t rem = u - b * per_mat;
-    i0 = (rem / ct) * kAtcRows;
+    i0 = (rem / ct) * nt;
     j0 = (rem % ct) * kAtcCols;
   };
   if (threadIdx.x == 0) {
@@ -2110,8 +2110,9 @@ __global__ void __launch_bounds__(kAtcThreads, 1) k_apply_tc(const __grid_consta
   }
   // K columns past l up to the next multiple of 8 enter the last MMA K step
   // and are never written below: zero the operand tiles once
-  for (int i = threadIdx.x; i < natoms * 2 * (kAtcAtomA + kAtcAtomB) / 16; i += blockDim.x)
-    reinterpret_cast<float4*>(smem)[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+  if (a.l % 8 != 0)
+    for (int i = threadIdx.x; i < natoms * 2 * (kAtcAtomA + kAtcAtomB) / 16; i += blockDim.x)
+      reinterpret_cast<float4*>(smem)[i] = make_float4(0.f, 0.f, 0.f, 0.f);
   asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   __syncthreads();
   tc::fence_after();
@@ -2133,11 +2134,11 @@ __global__ void __launch_bounds__(kAtcThreads, 1) k_apply_tc(const __grid_consta
       if (!ok) break;
       // the warps of this role finish the previous unit's writes before any
       // of them overwrites a tile: the MMAs that read them are done (opfree)
-      const int64_t key = static_cast<int64_t>(b) * rt + i0 / kAtcRows;
+      const int64_t key = static_cast<int64_t>(b) * rt + i0 / nt;
       if (key != b_key)
-        atc_split_rows<kAtcRows>(a.lm + b * a.lm_bs, i0, a.rows, l, b_hi, b_lo, kAtcAtomB, ptid);
+        atc_split_rows(a.lm + b * a.lm_bs, i0, a.rows, nt, l, b_hi, b_lo, kAtcAtomB, ptid);
       b_key = key;
-      atc_split_rows<kAtcCols>(a.rm + b * a.rm_bs, j0, a.cols, l, a_hi, a_lo, kAtcAtomA, ptid);
+      atc_split_rows(a.rm + b * a.rm_bs, j0, a.cols, kAtcCols, l, a_hi, a_lo, kAtcAtomA, ptid);
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
       __syncwarp();
       if (lane == 0) tc::mbar_arrive(opfull);
@@ -2145,7 +2146,7 @@ __global__ void __launch_bounds__(kAtcThreads, 1) k_apply_tc(const __grid_consta
     if (!ok && lane == 0) { *abort_flag = 1; raise_flag(flags, kFlagTimeout); }
   } else if (warp == kAtcProd) {
     // ---------------- MMA issuer ----------------
-    const uint32_t idesc = tc::idesc_tf32(kAtcCols, kAtcRows, 0, 0);
+    const uint32_t idesc = tc::idesc_tf32(kAtcCols, nt, 0, 0);
     bool ok = true;
     uint32_t it = 0;
     for (int64_t u = u0; u < u1 && ok; ++u, ++it) {
@@ -2175,17 +2176,19 @@ __global__ void __launch_bounds__(kAtcThreads, 1) k_apply_tc(const __grid_consta
     if (!ok && lane == 0) { *abort_flag = 1; raise_flag(flags, kFlagTimeout); }
   } else {
     // ---------------- epilogue: W <- (1 - lr wd) W - lr s (Psi + D) ----------------
-    // A stream of 16-row chunks (8 per unit: W rows 128 h .. 128 h + 127 of
-    // the tile, W columns 32 q + lane): the Psi and W loads of a chunk do not
+    // A stream of 16-row chunks (nt / 32 per unit: the nt / 2 W rows from
+    // h nt / 2 of the tile on, W columns 32 q + lane): the Psi and W loads of a chunk do not
     // depend on the accumulator, so they are issued kAtcSlots - 1 chunks ahead
     // into a register ring and stay in flight while earlier chunks wait for
     // their MMAs and are combined.
     const int e = warp - kAtcProd - 1;
     const int q = warp & 3;          // TMEM lane quarter = W columns 32 q .. 32 q + 31 of the tile
-    const int h = e >> 2;            // W rows 128 h .. 128 h + 127 of the tile
+    const int h = e >> 2;            // half of the tile's W rows
+    const int hrow = h * (nt >> 1);
     const double mn = static_cast<double>(a.rows) * static_cast<double>(a.cols);
     const float cw = 1.f - a.lr * a.wd;
-    constexpr int CH = kAtcChunk, NCH = 128 / kAtcChunk, S = kAtcSlots;
+    constexpr int CH = kAtcChunk, S = kAtcSlots;
+    const int NCH = nt / (2 * kAtcChunk);
     const int64_t nck = (u1 - u0) * NCH;
     // issue cursor: the unit (matrix b, row tile i0, column tile j0) and chunk
     int ib;
@@ -2202,7 +2205,7 @@ __global__ void __launch_bounds__(kAtcThreads, 1) k_apply_tc(const __grid_consta
     auto issue = [&](int64_t k, TP* P, TW* Wv, TW*& wptr, int& nrows, float& ct) {
       if (k < nck) {
         const int64_t j = ij0 + 32 * q + lane;
-        const int64_t r0 = ii0 + 128 * h + CH * icc;
+        const int64_t r0 = ii0 + hrow + CH * icc;
         if (ib != cur_b) {
           // fp64 throughput is low on this part: one lane per warp forms the
           // scale of a new matrix and broadcasts it
@@ -2236,7 +2239,7 @@ __global__ void __launch_bounds__(kAtcThreads, 1) k_apply_tc(const __grid_consta
           ij0 += kAtcCols;
           if (ij0 >= a.cols) {
             ij0 = 0;
-            ii0 += kAtcRows;
+            ii0 += nt;
             if (ii0 >= a.rows) { ii0 = 0; ++ib; }
           }
         }
@@ -2245,27 +2248,29 @@ __global__ void __launch_bounds__(kAtcThreads, 1) k_apply_tc(const __grid_consta
 #pragma unroll
     for (int sl = 0; sl < S; ++sl) issue(sl, pv[sl], wv[sl], wp[sl], nr[sl], ctt[sl]);
     bool ok = true;
+    int c = 0;                       // chunk of the unit
+    uint32_t un = 0;                 // unit, counted from u0
     for (int64_t k0 = 0; k0 < nck && ok; k0 += S) {
 #pragma unroll
       for (int sl = 0; sl < S; ++sl) {
         const int64_t k = k0 + sl;
         if (k >= nck) break;
-        const int64_t it = k / NCH;            // unit of this chunk, counted from u0
-        const int c = static_cast<int>(k - it * NCH);
-        const int acc = static_cast<int>(it & 1);
+        const int acc = static_cast<int>(un & 1);
         if (c == 0) {
-          ok = __all_sync(0xffffffffu, tc::mbar_wait(&tfull[acc], static_cast<uint32_t>((it >> 1) & 1), abort_flag));
+          ok = __all_sync(0xffffffffu, tc::mbar_wait(&tfull[acc], (un >> 1) & 1, abort_flag));
           if (!ok) break;
           tc::fence_after();
         }
         uint32_t v[CH];
-        tc::tmem_ld16(tmem_base + (static_cast<uint32_t>(32 * q) << 16) + static_cast<uint32_t>(256 * acc + 128 * h + CH * c), v);
+        tc::tmem_ld16(tmem_base + (static_cast<uint32_t>(32 * q) << 16) + static_cast<uint32_t>(256 * acc + hrow + CH * c), v);
         tc::tmem_ld_wait();
-        if (c == NCH - 1) {
-          // the accumulator is read: the MMAs of unit it + 2 may overwrite it
+        if (++c == NCH) {
+          // the accumulator is read: the MMAs of unit un + 2 may overwrite it
           tc::fence_before();
           __syncwarp();
           if (lane == 0) tc::mbar_arrive(&tempty[acc]);
+          c = 0;
+          ++un;
         }
         TW* W = wp[sl];
         if (nr[sl] == CH) {
@@ -2417,6 +2422,8 @@ cudaError_t sketch_group_alloc(SketchGroup& g, int rank, int oversample, std::ve
     cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kCqMaxSmem));
   contract_attrs<false>();
   contract_attrs<true>();
+  for (auto fn : {k_apply_tc<float, float>, k_apply_tc<float, bf16>, k_apply_tc<bf16, float>, k_apply_tc<bf16, bf16>})
+    cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(atc_smem(2)));
   // tensor-core contractions: Psi as a 3-D tensor {cols, rows, batch}; the
   // l-wide operands need 16-byte rows and matrix strides (checked per launch)
   {
@@ -2757,20 +2764,15 @@ cudaError_t run_sketch_group(SketchGroup& g, const SketchParams& p, const int* m
       // the two-atom size for every l: one CTA per SM, so the 512 TMEM
       // columns of a CTA never wait for another's
       const size_t smem = atc_smem(2);
-      static bool attr_set[4] = {false, false, false, false};
+      int nt = kAtcRows;
+      while (nt > 64 && cdiv(g.rows, nt) * cdiv(g.cols, kAtcCols) * nb < device_sm_count()) nt /= 2;
       const int kind = 2 * (g.w_dtype != 0) + (g.psi_bf16 ? 1 : 0);
       auto go = [&](auto* tw, auto* tp) -> cudaError_t {
         using TWT = std::remove_pointer_t<decltype(tw)>;
         using TPT = std::remove_pointer_t<decltype(tp)>;
-        if (!attr_set[kind]) {
-          const cudaError_t ea = cudaFuncSetAttribute(k_apply_tc<TWT, TPT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                      static_cast<int>(smem));
-          if (ea != cudaSuccess) return ea;
-          attr_set[kind] = true;
-        }
-        const int64_t units = cdiv(g.rows, kAtcRows) * cdiv(g.cols, kAtcCols) * nb;
+        const int64_t units = cdiv(g.rows, nt) * cdiv(g.cols, kAtcCols) * nb;
         const unsigned ctas = static_cast<unsigned>(std::min<int64_t>(units, device_sm_count()));
-        k_apply_tc<TWT, TPT><<<ctas, kAtcThreads, smem, s>>>(la, nb, natoms, flags);
+        k_apply_tc<TWT, TPT><<<ctas, kAtcThreads, smem, s>>>(la, nb, nt, natoms, flags);
         return cudaGetLastError();
       };
       switch (kind) {
