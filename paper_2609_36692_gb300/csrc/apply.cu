@@ -13,6 +13,8 @@ namespace normpre {
 
 template <typename TW, typename TT, bool VEC>
 __global__ void __launch_bounds__(256) k_apply_g(const __grid_constant__ ApplyLaunch a) {
+  pdl_wait();
+  pdl_trigger();
   __shared__ double red[32];
   __shared__ float scale_s;
   const int b = blockIdx.y;
@@ -40,7 +42,7 @@ __global__ void __launch_bounds__(256) k_apply_g(const __grid_constant__ ApplyLa
       const uint32_t r = v / cpr, c = (v - r * cpr) * 8;
       float w[8], t[8];
       load8(W + static_cast<int64_t>(r) * a.cols + c, w);
-      load8(T + static_cast<int64_t>(r) * a.t_ld + c, t);
+      load8_cg(T + static_cast<int64_t>(r) * a.t_ld + c, t);
 #pragma unroll
       for (int e = 0; e < 8; ++e) w[e] = fmaf(cw, w[e], ct * t[e]);
       store8(W + static_cast<int64_t>(r) * a.cols + c, w);
@@ -86,8 +88,8 @@ cudaError_t launch_apply_g(const ApplyLaunch& a, cudaStream_t s) {
   auto go = [&](auto* tw, auto* tt) {
     using TW = std::remove_pointer_t<decltype(tw)>;
     using TT = std::remove_pointer_t<decltype(tt)>;
-    if (vec) k_apply_g<TW, TT, true><<<grid, 256, 0, s>>>(a);
-    else k_apply_g<TW, TT, false><<<grid, 256, 0, s>>>(a);
+    if (vec) launch_pdl(true, k_apply_g<TW, TT, true>, grid, dim3(256), 0, s, a);
+    else launch_pdl(true, k_apply_g<TW, TT, false>, grid, dim3(256), 0, s, a);
     return cudaGetLastError();
   };
   if (a.w_dtype == 0 && a.t_dtype == 0) return go((float*)0, (float*)0);

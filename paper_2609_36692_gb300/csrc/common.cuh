@@ -11,6 +11,16 @@ __device__ __forceinline__ void raise_flag(int* flags, int bit) {
   if (flags) atomicOr(flags, bit);
 }
 
+// Programmatic dependent launch: a kernel launched by launch_pdl may start while
+// the kernel before it on the stream is still running.  Every such kernel calls
+// pdl_wait() in all threads before it touches global memory (it returns once
+// the kernel before has completed and its writes are visible), and may call
+// pdl_trigger() from when its successor may be brought onto the GPU.  Data
+// written by the kernel before is not read through ld.global.nc, which the
+// compiler may move above the wait.
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
 typedef __nv_bfloat16 bf16;
 
 __device__ __forceinline__ float to_f32(float v) { return v; }

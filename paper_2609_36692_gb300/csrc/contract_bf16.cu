@@ -39,6 +39,8 @@ struct VSplitArgs {
 static_assert(sizeof(VSplitArgs) + 64 <= 4096, "kernel arguments beyond 4 KB");
 constexpr int kVsRows = 256;
 __global__ void __launch_bounds__(256) k_vsplit_bf(const __grid_constant__ VSplitArgs a) {
+  pdl_wait();
+  pdl_trigger();
   __shared__ float tile[64][64 + 1];
   const int b = blockIdx.y, tid = threadIdx.x;
   const int l = a.l;   // <= 64
@@ -52,7 +54,7 @@ __global__ void __launch_bounds__(256) k_vsplit_bf(const __grid_constant__ VSpli
     if ((l & 3) == 0 && (reinterpret_cast<uintptr_t>(v) & 15) == 0) {
       for (int i4 = tid; i4 < 16 * l; i4 += 256) {          // 64 l / 4 float4s
         const int i = 4 * i4;
-        const float4 x = i < nvalid ? __ldg(reinterpret_cast<const float4*>(v) + i4) : make_float4(0.f, 0.f, 0.f, 0.f);
+        const float4 x = i < nvalid ? __ldcg(reinterpret_cast<const float4*>(v) + i4) : make_float4(0.f, 0.f, 0.f, 0.f);
         const int k = i / l, n = i - k * l;                   // l % 4 == 0: the 4 values share row k
         tile[k][n] = x.x; tile[k][n + 1] = x.y; tile[k][n + 2] = x.z; tile[k][n + 3] = x.w;
       }
@@ -161,6 +163,7 @@ __global__ void __launch_bounds__(kCbThreads, 1) k_contract_bf(const __grid_cons
   __syncthreads();
   tc::fence_after();
   const uint32_t tmem_base = *tmem_slot;
+  pdl_wait();
   const uint32_t vbytes = static_cast<uint32_t>(2 * a.np * 128);
 
   if (warp == 0) {
@@ -191,6 +194,7 @@ __global__ void __launch_bounds__(kCbThreads, 1) k_contract_bf(const __grid_cons
         __syncwarp();
       }
     }
+    pdl_trigger();   // this CTA's last copies are on their way
     if (!ok && lane == 0) { *abort_flag = 1; raise_flag(a.flags, kFlagTimeout); }
   } else if (warp == 1) {
     // ---------------- MMA issuer ----------------
@@ -317,7 +321,7 @@ cudaError_t launch_contract_bf16(const ContractBf16Launch& c, cudaStream_t s) {
   VSplitArgs vs;
   vs.v = c.v; vs.v_bs = c.v_bs; vs.K = c.K; vs.l = c.l; vs.np = np;
   vs.vb = static_cast<bf16*>(c.vb); vs.vb_bs = c.vb_bs; vs.kpad = kpad;
-  k_vsplit_bf<<<dim3(static_cast<unsigned>(cdiv(kpad, kVsRows)), static_cast<unsigned>(c.batch)), 256, 0, s>>>(vs);
+  launch_pdl(c.overlap, k_vsplit_bf, dim3(static_cast<unsigned>(cdiv(kpad, kVsRows)), static_cast<unsigned>(c.batch)), dim3(256), 0, s, vs);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   ContractBfArgs a;
@@ -335,8 +339,8 @@ cudaError_t launch_contract_bf16(const ContractBf16Launch& c, cudaStream_t s) {
   a.stall_first_copy = c.stall_first_copy;
   const int64_t units = cdiv(c.P, 128) * c.ksplit * c.batch;
   const unsigned grid = static_cast<unsigned>(std::min<int64_t>(units, device_sm_count()));
-  if (c.trans) k_contract_bf<true><<<grid, kCbThreads, kCbSmem, s>>>(a);
-  else k_contract_bf<false><<<grid, kCbThreads, kCbSmem, s>>>(a);
+  if (c.trans) launch_pdl(c.overlap, k_contract_bf<true>, dim3(grid), dim3(kCbThreads), kCbSmem, s, a);
+  else launch_pdl(c.overlap, k_contract_bf<false>, dim3(grid), dim3(kCbThreads), kCbSmem, s, a);
   return cudaGetLastError();
 }
 

@@ -84,6 +84,27 @@ class ProfileHook {
 };
 inline int64_t cdiv(int64_t x, int64_t m) { return (x + m - 1) / m; }
 
+// Launches a kernel that begins with pdl_wait() so that it may start before the
+// kernel ahead of it on the stream has ended (overlap: otherwise an ordinary
+// launch, for the first kernel behind a copy, a memset or an event wait).  A
+// dependent launch costs 3 to 5 us of launch latency, barrier and TMEM setup
+// on these short kernels; all of it but the wait itself then overlaps.
+template <typename... P, typename... A>
+inline cudaError_t launch_pdl(bool overlap, void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
+                              A... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = overlap ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+
 // ----------------------------------------------------------------------------
 // K1: momentum + relaxed tangent + diagonal-Gram normalization (normalize.cu)
 // ----------------------------------------------------------------------------
@@ -106,6 +127,8 @@ struct NormLaunch {
   // column-active scratch (see normalize_cols_scratch_bytes) and rows per
   // block of the column sums, fixed for a group so that its slices sum alike
   int col_rb = kColStatsRB;
+  bool overlap = false;           // launch_pdl: the first kernel, behind another one of the step
+  bool overlap_next = true;       // the others
   double* col_part = nullptr;
   float2* col_coef = nullptr;
 };
@@ -242,6 +265,7 @@ class NSPlan {
 // ----------------------------------------------------------------------------
 struct SketchGroup {
   int batch = 0;
+  bool alone = false;           // the handle's only group: its chain shares the GPU with no other
   int plan_batch = 0;           // batch the launch shapes are planned for (0: batch); a
                                 // slice keeps its group's, so its sums run in the same order
   int64_t rows = 0, cols = 0;   // stored shape
@@ -301,6 +325,7 @@ struct SketchParams {
   int64_t t = 0;
   int k = 0;                    // orientation of this step
   float lr = 0, wd = 0, target = 0.2f;
+  bool overlap = false;         // launch_pdl from the first kernel on (the stream's last work is a kernel)
   bool exact = false;           // NORMPRE_L_EXACT: exact eigenpairs instead of the sketch
   const int* mat_ids_host = nullptr;   // the group's (or slice's) matrix ids, host copy
   double* diag = nullptr;       // [n_mats][8] diagnostics (energies, alignment sums) or null
@@ -341,6 +366,7 @@ struct ContractBf16Launch {
   int ksplit, batch;
   int* flags;
   int stall_first_copy;
+  bool overlap;            // launch_pdl behind the kernel before
 };
 bool contract_bf16_map(CUtensorMap* map, const void* psi, int64_t rows, int64_t cols, int64_t ld, int batch,
                        int box_rows = 64);

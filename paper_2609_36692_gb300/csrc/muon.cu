@@ -16,6 +16,8 @@ namespace normpre {
 template <typename TG, typename TP, bool VEC>
 __global__ void __launch_bounds__(256) k_momentum_copy(const __grid_constant__ NormLaunch a, double* part, int nblk,
                                                        int stride) {
+  pdl_wait();
+  pdl_trigger();
   __shared__ double red[32];
   const int b = blockIdx.y, blk = blockIdx.x;
   const int64_t rows = a.rows, cols = a.cols;
@@ -63,6 +65,8 @@ __global__ void __launch_bounds__(256) k_momentum_copy(const __grid_constant__ N
 // (one thread walking 512 dependent fp64 loads took 40 us).
 __global__ void __launch_bounds__(32) k_muon_prescale(const double* part, int nblk, int stride, float* inscale,
                                                       float eps) {
+  pdl_wait();
+  pdl_trigger();
   const int b = blockIdx.x;
   double s = 0.0;
   for (int i = threadIdx.x; i < nblk; i += 32) s += part[static_cast<int64_t>(b) * stride + i];
@@ -77,8 +81,8 @@ cudaError_t launch_momentum_copy(const NormLaunch& a, double* part, int nblk, in
   auto go = [&](auto* tg, auto* tp) {
     using TG = std::remove_pointer_t<decltype(tg)>;
     using TP = std::remove_pointer_t<decltype(tp)>;
-    if (vec) k_momentum_copy<TG, TP, true><<<grid, 256, 0, s>>>(a, part, nblk, stride);
-    else k_momentum_copy<TG, TP, false><<<grid, 256, 0, s>>>(a, part, nblk, stride);
+    if (vec) launch_pdl(a.overlap, k_momentum_copy<TG, TP, true>, grid, dim3(256), 0, s, a, part, nblk, stride);
+    else launch_pdl(a.overlap, k_momentum_copy<TG, TP, false>, grid, dim3(256), 0, s, a, part, nblk, stride);
     return cudaGetLastError();
   };
   if (a.g_dtype == 0 && a.psi_dtype == 0) return go((float*)0, (float*)0);
@@ -89,7 +93,7 @@ cudaError_t launch_momentum_copy(const NormLaunch& a, double* part, int nblk, in
 
 cudaError_t launch_muon_prescale(const double* part, int nblk, int stride, int batch, float* inscale, float eps,
                                  cudaStream_t s) {
-  k_muon_prescale<<<batch, 32, 0, s>>>(part, nblk, stride, inscale, eps);
+  launch_pdl(true, k_muon_prescale, dim3(batch), dim3(32), 0, s, part, nblk, stride, inscale, eps);
   return cudaGetLastError();
 }
 

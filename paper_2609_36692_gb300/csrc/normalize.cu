@@ -99,6 +99,8 @@ __device__ __forceinline__ void row_store(T* p, int64_t j, int64_t cols, const f
 }
 template <typename TG, typename TW, typename TP, bool VEC>
 __global__ void __launch_bounds__(1024) k_norm_rows(const __grid_constant__ NormLaunch a) {
+  pdl_wait();
+  pdl_trigger();
   __shared__ float red[32];
   const int b = blockIdx.y;
   const int64_t row = blockIdx.x;
@@ -176,6 +178,8 @@ __global__ void __launch_bounds__(1024) k_norm_rows(const __grid_constant__ Norm
 // row-active, rows past 16 * 1024 columns: M is re-read by the thread that wrote it
 template <typename TG, typename TW, typename TP>
 __global__ void __launch_bounds__(256) k_norm_rows_scalar(const __grid_constant__ NormLaunch a) {
+  pdl_wait();
+  pdl_trigger();
   __shared__ float red[32];
   const int b = blockIdx.y;
   const int64_t row = blockIdx.x;
@@ -223,6 +227,8 @@ __global__ void __launch_bounds__(256) k_norm_rows_scalar(const __grid_constant_
 // ---------------------------------------------------------------------------
 template <typename TG, typename TW, bool VEC>
 __global__ void __launch_bounds__(kColThreads) k_norm_cols_stats(const __grid_constant__ NormLaunch a) {
+  pdl_wait();
+  pdl_trigger();
   __shared__ float part[8][3][256];
   const int b = blockIdx.z, rb = blockIdx.y;
   const int cc = threadIdx.x & 31, rl = threadIdx.x >> 5;
@@ -322,6 +328,8 @@ __global__ void __launch_bounds__(kColThreads) k_norm_cols_stats(const __grid_co
 // One warp per 32 columns: the few fp64 operations of a column spread over all
 // SMs.
 __global__ void __launch_bounds__(32) k_norm_cols_final(const __grid_constant__ NormLaunch a, int nrb, int stage) {
+  pdl_wait();
+  pdl_trigger();
   const int b = blockIdx.y;
   const int64_t cols = a.cols;
   const int64_t j = static_cast<int64_t>(blockIdx.x) * 32 + threadIdx.x;
@@ -368,6 +376,8 @@ __global__ void __launch_bounds__(32) k_norm_cols_final(const __grid_constant__ 
 // grid and thread layout as pass A.
 template <typename TW, bool VEC>
 __global__ void __launch_bounds__(kColThreads) k_norm_cols_xsq(const __grid_constant__ NormLaunch a) {
+  pdl_wait();
+  pdl_trigger();
   __shared__ float part[8][256];
   const int b = blockIdx.z, rb = blockIdx.y;
   const int cc = threadIdx.x & 31, rl = threadIdx.x >> 5;
@@ -388,7 +398,7 @@ __global__ void __launch_bounds__(kColThreads) k_norm_cols_xsq(const __grid_cons
       for (int e = 0; e < 8; ++e) ca[e] = coef[j0 + e].x;
       for (int64_t r = r0 + rl; r < r1; r += 8) {
         float mv[8], wv[8];
-        load8(M + r * cols + j0, mv);
+        load8_cg(M + r * cols + j0, mv);
         load8(w + r * cols + j0, wv);
 #pragma unroll
         for (int e = 0; e < 8; ++e) {
@@ -428,6 +438,8 @@ __global__ void __launch_bounds__(kColThreads) k_norm_cols_xsq(const __grid_cons
 // column-active pass B: Psi_ij = (m_ij - a_j w_ij) * inv_j
 template <typename TW, typename TP, bool VEC>
 __global__ void __launch_bounds__(kColThreads) k_norm_cols_apply(const __grid_constant__ NormLaunch a, int nrows) {
+  pdl_wait();
+  pdl_trigger();
   const int b = blockIdx.z, rb = blockIdx.y;
   const int cc = threadIdx.x & 31, rl = threadIdx.x >> 5;
   const int64_t rows = a.rows, cols = a.cols;
@@ -446,7 +458,7 @@ __global__ void __launch_bounds__(kColThreads) k_norm_cols_apply(const __grid_co
 #pragma unroll 2
     for (int64_t r = r0 + rl; r < r1; r += 8) {
       float mv[8], wv[8];
-      load8(M + r * cols + j0, mv);
+      load8_cg(M + r * cols + j0, mv);
       load8(w + r * cols + j0, wv);
 #pragma unroll
       for (int e = 0; e < 8; ++e) mv[e] = fmaf(-ca[e], wv[e], mv[e]) * ci[e];
@@ -486,6 +498,8 @@ __global__ void __launch_bounds__(kColThreads) k_norm_cols_apply(const __grid_co
 // ---------------------------------------------------------------------------
 template <typename TP>
 __global__ void __launch_bounds__(256) k_psi_colsq(const __grid_constant__ NormLaunch a) {
+  pdl_wait();
+  pdl_trigger();
   const int b = blockIdx.z, rb = blockIdx.y;
   const int64_t j = static_cast<int64_t>(blockIdx.x) * 256 + threadIdx.x;
   if (j >= a.cols) return;
@@ -500,6 +514,8 @@ __global__ void __launch_bounds__(256) k_psi_colsq(const __grid_constant__ NormL
 }
 
 __global__ void __launch_bounds__(256) k_psi_colfold(const __grid_constant__ NormLaunch a, int nrb) {
+  pdl_wait();
+  pdl_trigger();
   __shared__ float red[32];
   const int b = blockIdx.x;
   float nz = 0.f;
@@ -516,6 +532,8 @@ __global__ void __launch_bounds__(256) k_psi_colfold(const __grid_constant__ Nor
 
 template <typename TP>
 __global__ void __launch_bounds__(256) k_psi_colscale(const __grid_constant__ NormLaunch a) {
+  pdl_wait();
+  pdl_trigger();
   const int b = blockIdx.z;
   const int64_t j = static_cast<int64_t>(blockIdx.x) * 256 + threadIdx.x;
   if (j >= a.cols) return;
@@ -567,11 +585,11 @@ cudaError_t launch_normalize_rows(const NormLaunch& a, cudaStream_t s) {
     using TP = std::remove_pointer_t<decltype(tp)>;
     const int threads = static_cast<int>(round_up(cdiv(a.cols, 16), 32));
     if (vec) {
-      k_norm_rows<TG, TW, TP, true><<<grid, threads, 0, s>>>(a);
+      launch_pdl(a.overlap, k_norm_rows<TG, TW, TP, true>, dim3(grid), dim3(threads), 0, s, a);
     } else if (a.cols <= 16 * 1024) {
-      k_norm_rows<TG, TW, TP, false><<<grid, threads, 0, s>>>(a);
+      launch_pdl(a.overlap, k_norm_rows<TG, TW, TP, false>, dim3(grid), dim3(threads), 0, s, a);
     } else {
-      k_norm_rows_scalar<TG, TW, TP><<<grid, 256, 0, s>>>(a);
+      launch_pdl(a.overlap, k_norm_rows_scalar<TG, TW, TP>, dim3(grid), dim3(256), 0, s, a);
     }
     return cudaGetLastError();
   });
@@ -589,25 +607,25 @@ cudaError_t launch_normalize_cols(const NormLaunch& a, cudaStream_t s) {
     using TG = std::remove_pointer_t<decltype(tg)>;
     using TW = std::remove_pointer_t<decltype(tw)>;
     using TP = std::remove_pointer_t<decltype(tp)>;
-    if (vec) k_norm_cols_stats<TG, TW, true><<<grid, kColThreads, 0, s>>>(a);
-    else k_norm_cols_stats<TG, TW, false><<<grid, kColThreads, 0, s>>>(a);
+    if (vec) launch_pdl(a.overlap, k_norm_cols_stats<TG, TW, true>, dim3(grid), dim3(kColThreads), 0, s, a);
+    else launch_pdl(a.overlap, k_norm_cols_stats<TG, TW, false>, dim3(grid), dim3(kColThreads), 0, s, a);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     if (a.tangent == 2) {
       // strict: the coefficient first, then ||x_j||^2 summed from x itself
-      k_norm_cols_final<<<dim3(static_cast<unsigned>(cdiv(a.cols, 32)), a.n), 32, 0, s>>>(a, nrb, 1);
+      launch_pdl(a.overlap_next, k_norm_cols_final, dim3(static_cast<unsigned>(cdiv(a.cols, 32)), a.n), dim3(32), 0, s, a, nrb, 1);
       if ((e = cudaGetLastError()) != cudaSuccess) return e;
-      if (vec) k_norm_cols_xsq<TW, true><<<grid, kColThreads, 0, s>>>(a);
-      else k_norm_cols_xsq<TW, false><<<grid, kColThreads, 0, s>>>(a);
+      if (vec) launch_pdl(a.overlap_next, k_norm_cols_xsq<TW, true>, dim3(grid), dim3(kColThreads), 0, s, a);
+      else launch_pdl(a.overlap_next, k_norm_cols_xsq<TW, false>, dim3(grid), dim3(kColThreads), 0, s, a);
       if ((e = cudaGetLastError()) != cudaSuccess) return e;
-      k_norm_cols_final<<<dim3(static_cast<unsigned>(cdiv(a.cols, 32)), a.n), 32, 0, s>>>(a, nrb, 2);
+      launch_pdl(a.overlap_next, k_norm_cols_final, dim3(static_cast<unsigned>(cdiv(a.cols, 32)), a.n), dim3(32), 0, s, a, nrb, 2);
     } else {
-      k_norm_cols_final<<<dim3(static_cast<unsigned>(cdiv(a.cols, 32)), a.n), 32, 0, s>>>(a, nrb, 0);
+      launch_pdl(a.overlap_next, k_norm_cols_final, dim3(static_cast<unsigned>(cdiv(a.cols, 32)), a.n), dim3(32), 0, s, a, nrb, 0);
     }
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    if (vec) k_norm_cols_apply<TW, TP, true><<<grid_b, kColThreads, 0, s>>>(a, rb_b);
-    else k_norm_cols_apply<TW, TP, false><<<grid_b, kColThreads, 0, s>>>(a, rb_b);
+    if (vec) launch_pdl(a.overlap_next, k_norm_cols_apply<TW, TP, true>, dim3(grid_b), dim3(kColThreads), 0, s, a, rb_b);
+    else launch_pdl(a.overlap_next, k_norm_cols_apply<TW, TP, false>, dim3(grid_b), dim3(kColThreads), 0, s, a, rb_b);
     return cudaGetLastError();
   });
 }

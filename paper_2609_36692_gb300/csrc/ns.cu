@@ -288,6 +288,10 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_ns_gemm_tc(const __grid_const
   __syncthreads();
   tc::fence_after();
   const uint32_t tmem_base = *tmem_slot;
+  // everything above overlaps the end of the kernel before; the next one may
+  // come as SMs fall idle
+  pdl_wait();
+  pdl_trigger();
 
   if (warp == 0) {
     // ---------------- TMA producer (the warp waits, lane 0 issues) ----------------
@@ -420,7 +424,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_ns_gemm_tc(const __grid_const
       auto fetch_aux = [&](int c, uint4 (&dst)[4]) {
         if (auxp && c < c_hi && kind(c) != 2)
 #pragma unroll
-          for (int i = 0; i < 4; ++i) dst[i] = __ldg(reinterpret_cast<const uint4*>(auxp + i * aux8 + c));
+          for (int i = 0; i < 4; ++i) dst[i] = __ldcg(reinterpret_cast<const uint4*>(auxp + i * aux8 + c));
       };
       fetch_aux(c_lo, ax0);
       fetch_aux(c_lo + 32, ax1);
@@ -552,6 +556,8 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_ns_gemm_tc(const __grid_const
 // ---------------------------------------------------------------------------
 template <typename T>
 __global__ void __launch_bounds__(256) k_ns_gemm_simt(const __grid_constant__ GemmArgs args) {
+  pdl_wait();
+  pdl_trigger();
   __shared__ float As[16][64];
   __shared__ float Bs[16][64];
   __shared__ float red[8];
@@ -632,6 +638,8 @@ struct ScaleArgs {
   const int* count;
 };
 __global__ void k_scale_from_count(const ScaleArgs a) {
+  pdl_wait();
+  pdl_trigger();
   const int gi = blockIdx.x;
   for (int b = threadIdx.x; b < a.batch[gi]; b += blockDim.x) {
     const float m = static_cast<float>(a.count[a.mat_ids[gi][b]]);
@@ -660,6 +668,8 @@ struct NsCopyArgs {
 // One CTA per (matrix, row chunk).
 template <typename T, bool VEC>
 __global__ void __launch_bounds__(256) k_ns_load(const __grid_constant__ NsCopyArgs a) {
+  pdl_wait();
+  pdl_trigger();
   __shared__ double red[32];
   __shared__ float redf[32];
   constexpr int E = VEC ? 8 : 1;
@@ -717,6 +727,8 @@ __global__ void __launch_bounds__(256) k_ns_load(const __grid_constant__ NsCopyA
 // T's padded buffer -> the caller's [rows][cols]
 template <typename T, bool VEC>
 __global__ void __launch_bounds__(256) k_ns_store(const __grid_constant__ NsCopyArgs a) {
+  pdl_wait();
+  pdl_trigger();
   constexpr int E = VEC ? 8 : 1;
   const int b = blockIdx.x;
   const T* x = static_cast<const T*>(a.src) + static_cast<int64_t>(b) * a.rows_pad * a.cols_pad;
@@ -728,7 +740,7 @@ __global__ void __launch_bounds__(256) k_ns_store(const __grid_constant__ NsCopy
     const int r = r0 + i / cpr, c = (i % cpr) * E;
     if constexpr (VEC) {
       float v[8];
-      load8(x + static_cast<int64_t>(r) * a.cols_pad + c, v);
+      load8_cg(x + static_cast<int64_t>(r) * a.cols_pad + c, v);
       store8(y + static_cast<int64_t>(r) * a.cols + c, v);
     } else {
       y[static_cast<int64_t>(r) * a.cols + c] = x[static_cast<int64_t>(r) * a.cols_pad + c];
@@ -755,8 +767,10 @@ static void pair_config(cudaLaunchConfig_t* cfg, cudaLaunchAttribute* attr, int 
   attr[0].val.clusterDim.x = 2;
   attr[0].val.clusterDim.y = 1;
   attr[0].val.clusterDim.z = 1;
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[1].val.programmaticStreamSerializationAllowed = 1;
   cfg->attrs = attr;
-  cfg->numAttrs = 1;
+  cfg->numAttrs = 2;
 }
 
 // How many two-CTA clusters of the GEMM fit at once (a GPC with an odd number
@@ -772,7 +786,7 @@ static cudaError_t max_active_pairs(int* out, int num_sms) {
     return cudaSuccess;
   }
   cudaLaunchConfig_t cfg = {};
-  cudaLaunchAttribute attr[1];
+  cudaLaunchAttribute attr[2];
   pair_config(&cfg, attr, 2 * std::max(1, num_sms / 2), nullptr);
   e = cudaOccupancyMaxActiveClusters(out, k_ns_gemm_tc<true>, &cfg);
   if (e == cudaSuccess && dev >= 0 && dev < 64) known[dev].store(*out + 1);
@@ -1073,16 +1087,16 @@ cudaError_t NSPlan::run(int steps, const float coef[3], cudaStream_t s, int* fla
       if (bf16_) {
         if (L->mc[p] && units) {
           cudaLaunchConfig_t cfg = {};
-          cudaLaunchAttribute attr[1];
+          cudaLaunchAttribute attr[2];
           pair_config(&cfg, attr, 2 * std::min(ph[p]->total_tiles / 2, max_pairs_), s);
           cudaError_t le = cudaLaunchKernelEx(&cfg, k_ns_gemm_tc<true>, *ph[p]);
           if (le != cudaSuccess) return le;
         } else {
           const int grid = std::min(ph[p]->total_tiles, num_sms_);
-          k_ns_gemm_tc<false><<<grid, kTcThreads, kTcSmem, s>>>(*ph[p]);
+          launch_pdl(true, k_ns_gemm_tc<false>, dim3(grid), dim3(kTcThreads), kTcSmem, s, *ph[p]);
         }
       } else {
-        k_ns_gemm_simt<float><<<ph[p]->total_tiles, 256, 0, s>>>(*ph[p]);
+        launch_pdl(true, k_ns_gemm_simt<float>, dim3(ph[p]->total_tiles), dim3(256), 0, s, *ph[p]);
       }
       cudaError_t e = cudaGetLastError();
       if (e != cudaSuccess) return e;
@@ -1111,7 +1125,7 @@ cudaError_t NSPlan::scale_from_count(const int* count, const int* const* group_m
     a.batch[j] = (cnt == 1) ? m1 - m0 : groups_[g0 + j].spec.batch;
   }
   if (prof) prof->begin(kProfPrescale, s);
-  k_scale_from_count<<<a.n_groups, 128, 0, s>>>(a);
+  launch_pdl(true, k_scale_from_count, dim3(a.n_groups), dim3(128), 0, s, a);
   if (prof) prof->end(kProfPrescale, s, 1);
   return cudaGetLastError();
 }
@@ -1164,11 +1178,11 @@ cudaError_t NSPlan::store(void* T, int steps, cudaStream_t s) {
   const dim3 grid(g.spec.batch, n);
   const bool vec = g.spec.cols % 8 == 0;
   if (bf16_) {
-    if (vec) k_ns_store<normpre::bf16, true><<<grid, 256, 0, s>>>(a);
-    else k_ns_store<normpre::bf16, false><<<grid, 256, 0, s>>>(a);
+    if (vec) launch_pdl(true, k_ns_store<normpre::bf16, true>, grid, dim3(256), 0, s, a);
+    else launch_pdl(true, k_ns_store<normpre::bf16, false>, grid, dim3(256), 0, s, a);
   } else {
-    if (vec) k_ns_store<float, true><<<grid, 256, 0, s>>>(a);
-    else k_ns_store<float, false><<<grid, 256, 0, s>>>(a);
+    if (vec) launch_pdl(true, k_ns_store<float, true>, grid, dim3(256), 0, s, a);
+    else launch_pdl(true, k_ns_store<float, false>, grid, dim3(256), 0, s, a);
   }
   return cudaGetLastError();
 }

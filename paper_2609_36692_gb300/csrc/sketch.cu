@@ -85,6 +85,8 @@ struct OmegaArgs {
 };
 static_assert(sizeof(OmegaArgs) + 64 <= 4096, "kernel arguments beyond 4 KB");
 __global__ void k_omega(const __grid_constant__ OmegaArgs a) {
+  pdl_wait();
+  pdl_trigger();
   const int b = blockIdx.y;
   const int64_t n = a.n_a * a.l;
   const int64_t blk = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
@@ -493,6 +495,7 @@ __global__ void __launch_bounds__(kCtcThreads, 1) k_contract_tc(const __grid_con
   __syncthreads();
   tc::fence_after();
   const uint32_t tmem_base = *tmem_slot;
+  pdl_wait();
 
   if (warp == 0) {
     // ---------------- TMA producer ----------------
@@ -522,6 +525,7 @@ __global__ void __launch_bounds__(kCtcThreads, 1) k_contract_tc(const __grid_con
         __syncwarp();
       }
     }
+    pdl_trigger();   // this CTA's last copies are on their way
     if (!ok && lane == 0) { *abort_flag = 1; raise_flag(a.flags, kFlagTimeout); }
   } else if (warp == 1) {
     // ---------------- MMA issuer ----------------
@@ -700,6 +704,8 @@ struct SplitReduceArgs {
   int ksplit;
 };
 __global__ void k_split_reduce(const __grid_constant__ SplitReduceArgs a) {
+  pdl_wait();
+  pdl_trigger();
   const int b = blockIdx.y;
   const int64_t i = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
   if (i >= a.n) return;
@@ -746,6 +752,8 @@ static_assert(sizeof(GramArgs) + 64 <= 4096, "kernel arguments beyond 4 KB");
 // fill the CTA the rows are split into 2 or 4 groups whose sums are added in
 // a fixed order.
 __global__ void __launch_bounds__(256) k_gram_part(const __grid_constant__ GramArgs a) {
+  pdl_wait();
+  pdl_trigger();
   constexpr int LD = kLmax + 4;                  // 16-byte rows
   __shared__ __align__(16) float ys[kGramRows * LD];
   const int b = blockIdx.y, s = blockIdx.x, l = a.l, tid = threadIdx.x;
@@ -756,13 +764,13 @@ __global__ void __launch_bounds__(256) k_gram_part(const __grid_constant__ GramA
   if ((l & 3) == 0 && (reinterpret_cast<uintptr_t>(y) & 15) == 0) {
     for (int e4 = tid; e4 < kGramRows * l / 4; e4 += blockDim.x) {
       const int e = 4 * e4, i = e / l, j = e - i * l;   // l % 4 == 0: one row per float4
-      const float4 v = e < nval ? __ldg(reinterpret_cast<const float4*>(y) + e4) : make_float4(0.f, 0.f, 0.f, 0.f);
+      const float4 v = e < nval ? __ldcg(reinterpret_cast<const float4*>(y) + e4) : make_float4(0.f, 0.f, 0.f, 0.f);
       *reinterpret_cast<float4*>(ys + i * LD + j) = v;
     }
   } else {
     for (int e = tid; e < kGramRows * l; e += blockDim.x) {
       const int i = e / l, j = e - i * l;
-      ys[i * LD + j] = e < nval ? __ldg(y + e) : 0.f;
+      ys[i * LD + j] = e < nval ? __ldcg(y + e) : 0.f;
     }
   }
   for (int e = tid; e < kGramRows * (lp - l); e += blockDim.x) {
@@ -864,6 +872,8 @@ struct GramFoldArgs {
   int l;
 };
 __global__ void __launch_bounds__(256) k_gram_fold(const __grid_constant__ GramFoldArgs a) {
+  pdl_wait();
+  pdl_trigger();
   const int b = blockIdx.y;
   const int e = blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= a.l * a.l) return;
@@ -1363,6 +1373,7 @@ __device__ __forceinline__ bool cq_factor(const float* G, float* Rs, int l, floa
 
 template <int LP>
 __global__ void __launch_bounds__(kCqThreads, 1) k_cholqr_cluster(const __grid_constant__ CholClusterArgs a) {
+  pdl_wait();
   extern __shared__ float4 cq_smem4[];
   constexpr int LDX = LP + 4, L4 = LP / 4, TILES = cq_tiles(LP), GROUPS = cq_groups(LP);
   float* sums = reinterpret_cast<float*>(cq_smem4);          // [GROUPS][TILES][16]
@@ -1385,13 +1396,13 @@ __global__ void __launch_bounds__(kCqThreads, 1) k_cholqr_cluster(const __grid_c
 #pragma unroll 4
     for (int e = tid; e < nf / 4; e += kCqThreads) {
       const int r = e / l4, c = e - r * l4;
-      *reinterpret_cast<float4*>(X + r * LDX + 4 * c) = __ldg(reinterpret_cast<const float4*>(y) + e);
+      *reinterpret_cast<float4*>(X + r * LDX + 4 * c) = __ldcg(reinterpret_cast<const float4*>(y) + e);
     }
   } else {
 #pragma unroll 4
     for (int e = tid; e < nf; e += kCqThreads) {
       const int r = e / l;
-      X[r * LDX + e - r * l] = __ldg(y + e);
+      X[r * LDX + e - r * l] = __ldcg(y + e);
     }
   }
   if (l < LP)
@@ -1467,6 +1478,7 @@ __global__ void __launch_bounds__(kCqThreads, 1) k_cholqr_cluster(const __grid_c
       }
     }
     __syncthreads();
+    if (pass == 2) pdl_trigger();
     const bool zero = !(tr_s > 0.f);   // Y = 0 (a zero normalized update): Q = 0, nothing is selected downstream
     // R_ij = W_ij / R_ii strictly above the diagonal, and 1 / R_ii (0 for a
     // dropped column, and so a zero row of R)
@@ -1536,6 +1548,8 @@ struct RowMulArgs {
 // One thread per (row, 8 consecutive columns): the row's entries are
 // broadcast loads shared by its threads, S's rows 16-byte shared loads.
 __global__ void __launch_bounds__(256) k_rowmul(const __grid_constant__ RowMulArgs a) {
+  pdl_wait();
+  pdl_trigger();
   __shared__ __align__(16) float S[kLmax * (kLmax + 8)];
   const int b = blockIdx.y, l = a.l;
   const int lp = (l + 7) & ~7, ld = lp;          // S rows padded with zeros to 8 columns
@@ -1553,7 +1567,7 @@ __global__ void __launch_bounds__(256) k_rowmul(const __grid_constant__ RowMulAr
   const float* y = a.y + b * a.y_bs + i * l;
   float acc[8] = {};
   for (int k = 0; k < l; ++k) {
-    const float yk = __ldg(y + k);
+    const float yk = y[k];
     const float4 s0 = *reinterpret_cast<const float4*>(S + k * ld + j0);
     const float4 s1 = *reinterpret_cast<const float4*>(S + k * ld + j0 + 4);
     acc[0] = fmaf(yk, s0.x, acc[0]); acc[1] = fmaf(yk, s0.y, acc[1]);
@@ -1667,7 +1681,6 @@ __global__ void __launch_bounds__(1024) k_jacobi(const __grid_constant__ EigArgs
   auto vat = [&](int r, int c) -> float& { return r < npairs ? Vm[2 * (r * ldv + c)] : Vm[2 * ((r - npairs) * ldv + c) + 1]; };
   auto at = [&](uint32_t off) -> float& { return *reinterpret_cast<float*>(sm + off); };
   auto at2 = [&](uint32_t off) -> float2& { return *reinterpret_cast<float2*>(sm + off); };
-  fold_partials(a.part + b * a.part_bs, a.nsplit, l, A0, ld);
   for (int e = tid; e < n * n; e += nt) {
     const int i = e / n, j = e - (e / n) * n;
     if (i >= l || j >= l) A0[i * ld + j] = 0.f;
@@ -1683,6 +1696,8 @@ __global__ void __launch_bounds__(1024) k_jacobi(const __grid_constant__ EigArgs
     const uint32_t i = static_cast<uint32_t>(min(p, q)), j = static_cast<uint32_t>(max(p, q));
     table[e] = make_uint2(i * ld * 4 | (j * ld * 4) << 16, i * 4 | (j * 4) << 16);
   }
+  pdl_wait();
+  fold_partials(a.part + b * a.part_bs, a.nsplit, l, A0, ld);
   __syncthreads();
   // exact symmetry
   float s2 = 0.f;
@@ -1789,6 +1804,7 @@ __global__ void __launch_bounds__(1024) k_jacobi(const __grid_constant__ EigArgs
     // off-diagonal mass once it is tiny has reached that floor
     if (off <= 1e-12f * frob2 || (off <= 1e-9f * frob2 && off > 0.5f * prev)) { ++sweep; break; }
   }
+  pdl_trigger();
   const float* Af = A0;
   float* Zs = reinterpret_cast<float*>(sm + kJacCopy);   // Z, column c at [c * n]
   if (tid == 0 && sweep >= a.max_sweeps && off > 1e-8f * frob2) raise_flag(a.flags, kFlagNumeric);
@@ -2046,7 +2062,7 @@ __device__ __forceinline__ void atc_split_rows(const float* panel, int64_t r0, i
 #pragma unroll
     for (int k = 0; k < B; ++k) {
       const int idx = base + k * NT;
-      x[k] = (idx < n && idx < valid) ? __ldg(reinterpret_cast<const float4*>(src) + idx)
+      x[k] = (idx < n && idx < valid) ? __ldcg(reinterpret_cast<const float4*>(src) + idx)
                                       : make_float4(0.f, 0.f, 0.f, 0.f);
     }
 #pragma unroll
@@ -2117,6 +2133,7 @@ __global__ void __launch_bounds__(kAtcThreads, 1) k_apply_tc(const __grid_consta
   __syncthreads();
   tc::fence_after();
   const uint32_t tmem_base = *tmem_slot;
+  pdl_wait();
   const int l = a.l;
   const int ksteps = (l + 7) / 8;
 
@@ -2357,21 +2374,23 @@ static cudaError_t launch_cholqr(const CholQRArgs& c, float* rfac, int batch, in
 
 // CTAs per matrix of k_cholqr_cluster, or 0 where it does not apply (panels
 // wider than kCqLP, or too tall for the shared memory of eight CTAs): the
-// fewest with at most 512 rows each (one per thread of the solve).  More would
-// shorten the row work, but not the factorization, and take SMs from the other
-// groups' streams.
-static int cq_cluster_size(int64_t n, int lp) {
+// fewest with at most 512 rows each (one per thread of the solve), or, with
+// other groups' kernels on the other streams, that the shared memory admits
+// (GPT-2 Small L, 768 rows in one CTA instead of two: 2610 -> 2562 us a pass:
+// more CTAs hold SMs that those kernels want).
+static int cq_cluster_size(const SketchGroup& g, int64_t n, int lp) {
   if (lp > kCqLP) return 0;
+  auto fits = [&](int c) { return cdiv(n, c) <= 65536 && cq_smem(lp, static_cast<int>(cdiv(n, c))) <= kCqMaxSmem; };
   int c = 1;
-  while (c < kCqMaxCluster && cdiv(n, c) > 512) c *= 2;
-  const int64_t rows = cdiv(n, c);
-  return rows <= 65536 && cq_smem(lp, static_cast<int>(rows)) <= kCqMaxSmem ? c : 0;
+  while (c < kCqMaxCluster && (!fits(c) || (g.alone && cdiv(n, c) > 512))) c *= 2;
+  return fits(c) ? c : 0;
 }
 
-static cudaError_t launch_cholqr_cluster(CholClusterArgs c, int cluster, int batch, int lp, cudaStream_t s) {
+static cudaError_t launch_cholqr_cluster(CholClusterArgs c, int cluster, int batch, int lp, bool overlap,
+                                         cudaStream_t s) {
   c.rows_c = static_cast<int>(cdiv(c.n, cluster));
   cudaLaunchConfig_t cfg = {};
-  cudaLaunchAttribute attr[1];
+  cudaLaunchAttribute attr[2];
   cfg.gridDim = dim3(static_cast<unsigned>(cluster), static_cast<unsigned>(batch));
   cfg.blockDim = dim3(kCqThreads);
   cfg.dynamicSmemBytes = cq_smem(lp, c.rows_c);
@@ -2380,8 +2399,10 @@ static cudaError_t launch_cholqr_cluster(CholClusterArgs c, int cluster, int bat
   attr[0].val.clusterDim.x = static_cast<unsigned>(cluster);
   attr[0].val.clusterDim.y = 1;
   attr[0].val.clusterDim.z = 1;
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = overlap ? 2 : 1;
   switch (lp) {
 #define NP_CQC(N) case N: return cudaLaunchKernelEx(&cfg, k_cholqr_cluster<N>, c);
     NP_CQC(8) NP_CQC(16) NP_CQC(24) NP_CQC(32) NP_CQC(40) NP_CQC(48)
@@ -2513,6 +2534,12 @@ cudaError_t run_sketch_group(SketchGroup& g, const SketchParams& p, const int* m
   const int lp = static_cast<int>(round_up(l, 8));   // register width of the QR solves
   const int cpt = (l + 3) / 4;                         // columns per thread of the contractions
   const int64_t sq = static_cast<int64_t>(g.lmax) * g.lmax;
+  // Dependent launches (launch_pdl) on this chain: where the group is alone, or
+  // its contractions leave SMs idle.  With several groups on streams of their
+  // own, a full grid's CTAs that wait for their predecessor keep the SMs from
+  // the other groups' kernels (LLaMA 1B: 16822 us without, 17385 with).
+  const int64_t widest = cdiv(big, 128) * (g.plan_batch ? g.plan_batch : B);
+  const bool ov = g.alone || widest <= device_sm_count();
   cudaError_t e;
 #define NP_CHECK() do { e = cudaGetLastError(); if (e != cudaSuccess) return e; } while (0)
 
@@ -2525,7 +2552,7 @@ cudaError_t run_sketch_group(SketchGroup& g, const SketchParams& p, const int* m
     o.mat_id = mat_ids;
     const int64_t blocks = cdiv(n_a * l, 4);
     prof->begin(kProfOmega, s);
-    k_omega<<<dim3(static_cast<unsigned>(cdiv(blocks, 256)), B), 256, 0, s>>>(o);
+    launch_pdl(p.overlap, k_omega, dim3(static_cast<unsigned>(cdiv(blocks, 256)), B), dim3(256), 0, s, o);
     NP_CHECK();
     prof->end(kProfOmega, s, 1);
   }
@@ -2564,6 +2591,7 @@ cudaError_t run_sketch_group(SketchGroup& g, const SketchParams& p, const int* m
       cb.kchunk = round_up(cdiv(K, ks), 64);
       cb.ksplit = ks; cb.batch = B;
       cb.flags = flags;
+      cb.overlap = ov;
       cb.stall_first_copy = stall_pending ? 1 : 0;
       stall_pending = false;
       err = launch_contract_bf16(cb, s);
@@ -2589,8 +2617,8 @@ cudaError_t run_sketch_group(SketchGroup& g, const SketchParams& p, const int* m
       // persistent: one CTA per SM (shared memory and TMEM admit one)
       const int64_t units = cdiv(P, 128) * ks * B;
       const unsigned grid = static_cast<unsigned>(std::min<int64_t>(units, device_sm_count()));
-      if (trans) k_contract_tc<true><<<grid, kCtcThreads, kCtcSmem, s>>>(ct);
-      else k_contract_tc<false><<<grid, kCtcThreads, kCtcSmem, s>>>(ct);
+      if (trans) launch_pdl(ov, k_contract_tc<true>, dim3(grid), dim3(kCtcThreads), kCtcSmem, s, ct);
+      else launch_pdl(ov, k_contract_tc<false>, dim3(grid), dim3(kCtcThreads), kCtcSmem, s, ct);
       err = cudaGetLastError();
     } else {
       err = trans ? launch_contract<true>(c, B, cpt, s) : launch_contract<false>(c, B, cpt, s);
@@ -2602,7 +2630,7 @@ cudaError_t run_sketch_group(SketchGroup& g, const SketchParams& p, const int* m
       r.part = g.kpart; r.part_bs = vbs * kMaxKSplit;
       r.out = out; r.out_bs = vbs;
       r.n = P * l; r.ksplit = ks;
-      k_split_reduce<<<dim3(static_cast<unsigned>(cdiv(r.n, 256)), B), 256, 0, s>>>(r);
+      launch_pdl(ov, k_split_reduce, dim3(static_cast<unsigned>(cdiv(r.n, 256)), B), dim3(256), 0, s, r);
       err = cudaGetLastError();
       if (err) return err;
       ++n_l;
@@ -2623,12 +2651,12 @@ cudaError_t run_sketch_group(SketchGroup& g, const SketchParams& p, const int* m
     ga.part_bs = static_cast<int64_t>(g.max_part) * sq;
     ga.n = n; ga.l = l;
     ga.nsplit = static_cast<int>(cdiv(n, kGramRows));
-    k_gram_part<<<dim3(ga.nsplit, B), 256, 0, s>>>(ga);
+    launch_pdl(ov, k_gram_part, dim3(ga.nsplit, B), dim3(256), 0, s, ga);
     if (ga.nsplit == 1) return GramOut{g.part, ga.part_bs, 1};
     GramFoldArgs fa;
     fa.part = g.part; fa.part_bs = ga.part_bs; fa.nsplit = ga.nsplit;
     fa.gram = g.gram; fa.gram_bs = sq; fa.l = l;
-    k_gram_fold<<<dim3(static_cast<unsigned>(cdiv(static_cast<int64_t>(l) * l, 256)), B), 256, 0, s>>>(fa);
+    launch_pdl(ov, k_gram_fold, dim3(static_cast<unsigned>(cdiv(static_cast<int64_t>(l) * l, 256)), B), dim3(256), 0, s, fa);
     ++n_fold;
     return GramOut{g.gram, sq, 1};
   };
@@ -2654,13 +2682,13 @@ cudaError_t run_sketch_group(SketchGroup& g, const SketchParams& p, const int* m
     // columns): y -> q -> zt -> q
     prof->begin(kProfQR, s);
     int n_qr = 7;
-    if (const int cluster = cq_cluster_size(m_a, lp)) {
+    if (const int cluster = cq_cluster_size(g, m_a, lp)) {
       CholClusterArgs cq;
       cq.y = ycur; cq.q = g.q; cq.v_bs = vbs;
       cq.n = m_a; cq.l = l; cq.flags = flags;
       cq.vec = (l % 4 == 0) && (vbs % 4 == 0) && (reinterpret_cast<uintptr_t>(ycur) % 16 == 0) &&
                (reinterpret_cast<uintptr_t>(g.q) % 16 == 0);
-      if ((e = launch_cholqr_cluster(cq, cluster, B, lp, s))) return e;
+      if ((e = launch_cholqr_cluster(cq, cluster, B, lp, ov, s))) return e;
       n_qr = 1;
     } else {
       const float* src = ycur;
@@ -2672,7 +2700,7 @@ cudaError_t run_sketch_group(SketchGroup& g, const SketchParams& p, const int* m
       ga.part_bs = static_cast<int64_t>(g.max_part) * sq;
       ga.n = m_a; ga.l = l;
       ga.nsplit = static_cast<int>(cdiv(m_a, kGramRows));
-      k_gram_part<<<dim3(ga.nsplit, B), 256, 0, s>>>(ga);
+      launch_pdl(ov, k_gram_part, dim3(ga.nsplit, B), dim3(256), 0, s, ga);
       NP_CHECK();
       int nsplit = ga.nsplit;
       for (int pass = 0; pass < 3; ++pass) {
@@ -2710,8 +2738,8 @@ cudaError_t run_sketch_group(SketchGroup& g, const SketchParams& p, const int* m
       ea.m_a = m_a; ea.n_a = n_a;
       ea.max_sweeps = p.max_sweeps;
       ea.flags = flags;
-      if (l <= 64) k_jacobi<1><<<B, jacobi_threads(l), jacobi_smem(l), s>>>(ea);
-      else k_jacobi<2><<<B, jacobi_threads(l), jacobi_smem(l), s>>>(ea);
+      if (l <= 64) launch_pdl(ov, k_jacobi<1>, dim3(B), dim3(jacobi_threads(l)), jacobi_smem(l), s, ea);
+      else launch_pdl(ov, k_jacobi<2>, dim3(B), dim3(jacobi_threads(l)), jacobi_smem(l), s, ea);
       NP_CHECK();
     }
   }
@@ -2724,7 +2752,7 @@ cudaError_t run_sketch_group(SketchGroup& g, const SketchParams& p, const int* m
     RowMulArgs rm;
     rm.y = k_on_b ? g.bt : g.q; rm.y_bs = vbs; rm.s = g.kmat; rm.s_bs = sq;
     rm.out = g.qk; rm.out_bs = vbs; rm.n = k_on_b ? n_a : m_a; rm.l = l;
-    k_rowmul<<<dim3(static_cast<unsigned>(cdiv(rm.n * ((l + 7) / 8), 256)), B), 256, 0, s>>>(rm);
+    launch_pdl(ov, k_rowmul, dim3(static_cast<unsigned>(cdiv(rm.n * ((l + 7) / 8), 256)), B), dim3(256), 0, s, rm);
     NP_CHECK();
   }
   prof->end(kProfEig, s, (p.exact ? 1 : 3) + n_fold);
@@ -2772,7 +2800,7 @@ cudaError_t run_sketch_group(SketchGroup& g, const SketchParams& p, const int* m
         using TPT = std::remove_pointer_t<decltype(tp)>;
         const int64_t units = cdiv(g.rows, nt) * cdiv(g.cols, kAtcCols) * nb;
         const unsigned ctas = static_cast<unsigned>(std::min<int64_t>(units, device_sm_count()));
-        k_apply_tc<TWT, TPT><<<ctas, kAtcThreads, smem, s>>>(la, nb, nt, natoms, flags);
+        launch_pdl(ov, k_apply_tc<TWT, TPT>, dim3(ctas), dim3(kAtcThreads), smem, s, la, nb, nt, natoms, flags);
         return cudaGetLastError();
       };
       switch (kind) {
