@@ -198,7 +198,7 @@ struct NSGroupBuf {
   int64_t s = 0, big = 0;       // s = min(rows, cols), big = max(rows, cols)
   int64_t s_pad = 0, big_pad = 0;
   int64_t rows_pad = 0, cols_pad = 0;   // padded stored layout of X buffers
-  int bn_s = 256, bn_big = 256;         // N tile of the s x s GEMMs / of the update GEMM
+  int bn_gram = 64, bn_upd = 64;        // N tile of the s x s products / of the update
   void* X[3] = {};              // [batch][rows_pad][cols_pad]; X[0] receives Psi
   void* A = nullptr;            // [batch][s_pad][s_pad]
   void* B = nullptr;            // [batch][s_pad][s_pad]

@@ -122,12 +122,15 @@ static_assert(sizeof(GemmArgs) + 64 <= 4096, "kernel arguments beyond 4 KB");
 
 // Tiles of one matrix: the whole tiles_m x tiles_n grid, or for a symmetric
 // product only the tiles that reach the diagonal or lie above it
-// (tm <= (BN / 128)(tn + 1) - 1), enumerated column by column.
+// (128 tm < BN (tn + 1)), enumerated column by column.
+__host__ __device__ inline int sym_column(int tn, int tiles_m, int bn) {
+  const int n = ((tn + 1) * bn + 127) / 128;
+  return n < tiles_m ? n : tiles_m;
+}
 __host__ __device__ inline int tiles_per_matrix(int tiles_m, int tiles_n, int bn, int sym) {
   if (!sym) return tiles_m * tiles_n;
-  const int rr = bn / 128;
   int n = 0;
-  for (int tn = 0; tn < tiles_n; ++tn) n += (rr * (tn + 1) < tiles_m) ? rr * (tn + 1) : tiles_m;
+  for (int tn = 0; tn < tiles_n; ++tn) n += sym_column(tn, tiles_m, bn);
   return n;
 }
 
@@ -153,10 +156,9 @@ __device__ __forceinline__ int decode_tile(const GemmArgs& a, int t, int& b, int
     tn = r - tmu * g.tiles_n;
     tm = (tmu << pairs) + sub;
   } else {
-    const int rr = g.BN / 128;
     int c = 0;
     for (;; ++c) {
-      const int cnt = ((rr * (c + 1) < g.tiles_m) ? rr * (c + 1) : g.tiles_m) >> pairs;
+      const int cnt = sym_column(c, g.tiles_m, g.BN) >> pairs;
       if (r < cnt) break;
       r -= cnt;
     }
@@ -825,19 +827,51 @@ static NSGroupBuf ns_geometry(bool bf16, const NSGroupSpec& sp) {
   g.elem = bf16 ? 2 : 4;
   if (bf16) {
     g.s_pad = round_up(g.s, 128);
-    g.bn_s = (g.s_pad % 256 == 0) ? 256 : 128;
     // 256: the update of a tall matrix then has an even number of 128-row
     // tiles and can run on two-CTA clusters
     g.big_pad = round_up(g.big, 256);
-    g.bn_big = g.tall ? g.bn_s : 256;
   } else {
     g.s_pad = round_up(g.s, tile_m);
     g.big_pad = round_up(g.big, tile_m);
-    g.bn_s = g.bn_big = 64;
   }
   g.rows_pad = g.tall ? g.big_pad : g.s_pad;
   g.cols_pad = g.tall ? g.s_pad : g.big_pad;
   return g;
+}
+
+// N tiles of the products: 256 columns, or 128 or 64 while a product would
+// have fewer tiles than two thirds of the SMs (and 128 where 256 does not
+// divide N).  A tile's time is a fixed 8 us and its share of the MMAs and the
+// epilogue, so few wide tiles leave the chip idle: one 256 x 1024 matrix is
+// two tiles of 256 columns in the Gram product and 8 in the update, or 6 and
+// 32 of 64.
+static void ns_tiles(bool bf16, std::vector<NSGroupBuf>& groups, int num_sms) {
+  auto fit = [](int bn, int64_t n) { return bn > 128 && n % bn != 0 ? 128 : bn; };
+  auto gram = [&](const NSGroupBuf& g, int bn) { return fit(bn, g.s_pad); };
+  auto upd = [&](const NSGroupBuf& g, int bn) { return fit(bn, g.tall ? g.s_pad : g.big_pad); };
+  int bg = 256, bu = 256;
+  if (!bf16) bg = bu = 64;
+  for (; bg > 64; bg /= 2) {
+    int64_t n = 0;
+    for (const NSGroupBuf& g : groups) {
+      const int bn = gram(g, bg);
+      n += static_cast<int64_t>(g.spec.batch) *
+           tiles_per_matrix(static_cast<int>(g.s_pad / 128), static_cast<int>(g.s_pad / bn), bn, 1);
+    }
+    if (3 * n >= 2 * num_sms) break;
+  }
+  for (; bu > 64; bu /= 2) {
+    int64_t n = 0;
+    for (const NSGroupBuf& g : groups) {
+      const int64_t um = g.tall ? g.big_pad : g.s_pad, un = g.tall ? g.s_pad : g.big_pad;
+      n += static_cast<int64_t>(g.spec.batch) * (um / 128) * (un / upd(g, bu));
+    }
+    if (3 * n >= 2 * num_sms) break;
+  }
+  for (NSGroupBuf& g : groups) {
+    g.bn_gram = bf16 ? gram(g, bg) : 64;
+    g.bn_upd = bf16 ? upd(g, bu) : 64;
+  }
 }
 
 namespace {
@@ -864,8 +898,11 @@ cudaError_t NSPlan::init(bool bf16, const std::vector<NSGroupSpec>& specs, std::
     return cudaErrorInvalidValue;
   }
   const int64_t tile_m = bf16 ? 128 : 64;
-  for (const NSGroupSpec& sp : specs) {
-    NSGroupBuf g = ns_geometry(bf16, sp);
+  std::vector<NSGroupBuf> planned;
+  for (const NSGroupSpec& sp : specs) planned.push_back(ns_geometry(bf16, sp));
+  ns_tiles(bf16, planned, num_sms_);
+  for (NSGroupBuf& g : planned) {
+    const NSGroupSpec& sp = g.spec;
     if (ext) {
       // the caller's workspace, carved; nothing has to be zero in it (load()
       // writes the padding of X[0], the products write whole padded tiles)
@@ -884,8 +921,7 @@ cudaError_t NSPlan::init(bool bf16, const std::vector<NSGroupSpec>& specs, std::
     const size_t abytes = static_cast<size_t>(sp.batch) * g.s_pad * g.s_pad * g.elem;
     // tiles of the update GEMM (its epilogue emits the ||T||^2 partials)
     const int64_t um = g.tall ? g.big_pad : g.s_pad, un = g.tall ? g.s_pad : g.big_pad;
-    const int64_t ubn = g.tall ? g.bn_s : g.bn_big;
-    const int tiles = static_cast<int>((um / tile_m) * (un / (bf16 ? ubn : 64)));
+    const int tiles = static_cast<int>((um / tile_m) * (un / g.bn_upd));
     g.n_part = tiles * (bf16 ? kEpiWarps : 1);
     void* p;
     for (int i = 0; i < 3; ++i) {
@@ -931,7 +967,7 @@ cudaError_t NSPlan::init(bool bf16, const std::vector<NSGroupSpec>& specs, std::
         g.M = g.N = static_cast<int>(gb.s_pad);
         g.K = static_cast<int>(gb.big_pad);
         g.a_mn = g.b_mn = gb.tall ? 1 : 0;
-        g.BN = bf16 ? gb.bn_s : 64;
+        g.BN = gb.bn_gram;
         g.a_ld = g.b_ld = gb.cols_pad;
         g.a_bs = g.b_bs = xs;
         g.out_ld = gb.s_pad; g.out_bs = as;
@@ -939,7 +975,7 @@ cudaError_t NSPlan::init(bool bf16, const std::vector<NSGroupSpec>& specs, std::
       } else if (ph == 1) {    // B = b A + c A A   (A symmetric: A A = A A^T)
         g.M = g.N = g.K = static_cast<int>(gb.s_pad);
         g.a_mn = g.b_mn = 0;
-        g.BN = bf16 ? gb.bn_s : 64;
+        g.BN = gb.bn_gram;
         g.Abuf = g.Bbuf = gb.A;
         g.a_ld = g.b_ld = gb.s_pad;
         g.a_bs = g.b_bs = as;
@@ -950,13 +986,13 @@ cudaError_t NSPlan::init(bool bf16, const std::vector<NSGroupSpec>& specs, std::
         if (!gb.tall) {
           g.M = static_cast<int>(gb.s_pad); g.N = static_cast<int>(gb.big_pad);
           g.a_mn = 0; g.b_mn = 1;
-          g.BN = bf16 ? gb.bn_big : 64;
+          g.BN = gb.bn_upd;
           g.Abuf = gb.B; g.a_ld = gb.s_pad; g.a_bs = as;
           g.b_ld = gb.cols_pad; g.b_bs = xs;          // Bbuf = X_in (set per run)
         } else {
           g.M = static_cast<int>(gb.big_pad); g.N = static_cast<int>(gb.s_pad);
           g.a_mn = 0; g.b_mn = 0;
-          g.BN = bf16 ? gb.bn_s : 64;
+          g.BN = gb.bn_upd;
           g.a_ld = gb.cols_pad; g.a_bs = xs;          // Abuf = X_in (set per run)
           g.Bbuf = gb.B; g.b_ld = gb.s_pad; g.b_bs = as;
         }
@@ -990,7 +1026,8 @@ cudaError_t NSPlan::init(bool bf16, const std::vector<NSGroupSpec>& specs, std::
     a.total_tiles = tiles;
     bool cl = bf16;
     for (int gi = 0; gi < a.n_groups; ++gi)
-      if (a.g[gi].tiles_m % 2 != 0 || (a.g[gi].BN / 64) % 2 != 0) cl = false;
+      // pairs of vertically adjacent tiles: an even number of them per column
+      if (a.g[gi].tiles_m % 2 != 0 || a.g[gi].BN % 128 != 0 || (a.g[gi].sym && a.g[gi].BN != 256)) cl = false;
     L->mc[ph] = cl;
   }
   if (bf16) {
