@@ -1808,15 +1808,22 @@ __global__ void __launch_bounds__(1024) k_jacobi(const __grid_constant__ EigArgs
   const float* Af = A0;
   float* Zs = reinterpret_cast<float*>(sm + kJacCopy);   // Z, column c at [c * n]
   if (tid == 0 && sweep >= a.max_sweeps && off > 1e-8f * frob2) raise_flag(a.flags, kFlagNumeric);
-  // sort eigenvalues descending, ties by lower index (stable)
+  // sort eigenvalues descending, ties by lower index (stable).  Compared as
+  // integers of the same order, a total order also of NaN: `order` has to be a
+  // permutation whatever the values (a non-finite step is reported, not faulted)
+  auto key = [](float f) {
+    const int v = __float_as_int(f + 0.f);
+    return v ^ ((v >> 31) & 0x7fffffff);
+  };
   float* ritz = a.ritz + b * a.ritz_bs;
   for (int i = tid; i < l; i += nt) {
     const float li = Af[i * ld + i];
+    const int ki = key(li);
     int pos = 0;
 #pragma unroll 8
     for (int j = 0; j < l; ++j) {
-      const float lj = Af[j * ld + j];
-      if (lj > li || (lj == li && j < i)) ++pos;
+      const int kj = key(Af[j * ld + j]);
+      if (kj > ki || (kj == ki && j < i)) ++pos;
     }
     order[pos] = i;
     ritz[pos] = li;

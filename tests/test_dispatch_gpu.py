@@ -163,3 +163,33 @@ def test_sketch_basis_and_ritz_pairs(rows, cols, rank, oversample, t):
     opt.close()
 
 
+# ---------------------------------------------------------------------------
+# non-finite gradients: the step is reported, nothing faults, and the handle's
+# next step on finite inputs is that of a fresh one
+# ---------------------------------------------------------------------------
+@pytest.mark.parametrize("value", [float("nan"), float("inf")])
+@pytest.mark.parametrize("variant,precision,rank", [(1, 1, 32), (1, 0, 32), (1, 1, 64), (0, 0, 32), (2, 0, 32)])
+def test_nonfinite_gradient_is_reported(variant, precision, rank, value):
+    import torch
+    from paper_2609_36692_gb300 import normpre as C
+    from paper_2609_36692_gb300.optim import NormPre
+    gen = torch.Generator(device="cuda").manual_seed(3)
+    shapes = [(256, 320), (90, 200)]
+    draw = lambda f: [torch.randn(s, device="cuda", generator=gen) * f for s in shapes]  # noqa: E731
+    W0, G0, M0 = draw(0.02), draw(1.0), draw(1.0)
+    out = []
+    for poison in (True, False):
+        opt = NormPre(shapes, ["f32"] * 2, ["f32"] * 2, variant=variant, precision=precision, rank=rank)
+        for t in (0, 1):
+            if poison:
+                W, G, M = ([x.clone() for x in v] for v in (W0, G0, M0))
+                G[0][7, 11] = value
+                opt.step(t, 0.02, W, G, M)
+                assert opt.status(raise_on_error=False) != C.NORMPRE_OK
+            W, M = [x.clone() for x in W0], [x.clone() for x in M0]
+            opt.step(t, 0.02, W, G0, M)
+            assert opt.status() == C.NORMPRE_OK
+            out.append(W)
+        opt.close()
+    for a, b in zip(out[:2], out[2:]):
+        assert all(torch.equal(x, y) for x, y in zip(a, b))
