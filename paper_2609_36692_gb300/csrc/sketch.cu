@@ -1545,40 +1545,84 @@ struct RowMulArgs {
   int64_t n;
   int l;
 };
-// One thread per (row, 8 consecutive columns): the row's entries are
-// broadcast loads shared by its threads, S's rows 16-byte shared loads.
+// One thread per (R rows, 8 consecutive columns): two 16-byte shared loads of S
+// serve 8 FMAs of every row, and V4 (l % 4 == 0, 16-byte aligned rows) reads 16
+// entries of each row at a time.  Four rows per thread where that still fills
+// the SMs, bound by the shared loads (with one row and scalar loads of Y the
+// Qwen3 groups took 45 us); one row otherwise, where it is bound by the round
+// trips to L2.
+template <bool V4, int R>
 __global__ void __launch_bounds__(256) k_rowmul(const __grid_constant__ RowMulArgs a) {
+  __shared__ __align__(16) float S[kLmax * (kLmax + 8)];
   pdl_wait();
   pdl_trigger();
-  __shared__ __align__(16) float S[kLmax * (kLmax + 8)];
   const int b = blockIdx.y, l = a.l;
   const int lp = (l + 7) & ~7, ld = lp;          // S rows padded with zeros to 8 columns
   const float* s = a.s + b * a.s_bs;
-  for (int e = threadIdx.x; e < l * lp; e += blockDim.x) {
-    const int k = e / lp, j = e - k * lp;
-    S[k * ld + j] = j < l ? s[k * l + j] : 0.f;
+  if (V4 && lp == l) {
+    for (int e = threadIdx.x; e < l * l / 4; e += blockDim.x)
+      reinterpret_cast<float4*>(S)[e] = __ldcg(reinterpret_cast<const float4*>(s) + e);
+  } else {
+    for (int e = threadIdx.x; e < l * lp; e += blockDim.x) {
+      const int k = e / lp, j = e - k * lp;
+      S[k * ld + j] = j < l ? s[k * l + j] : 0.f;
+    }
   }
   __syncthreads();
   const int cg = lp >> 3;                        // column groups per row
   const int64_t t = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
-  if (t >= a.n * cg) return;
-  const int64_t i = t / cg;
-  const int j0 = 8 * static_cast<int>(t - i * cg);
-  const float* y = a.y + b * a.y_bs + i * l;
-  float acc[8] = {};
-  for (int k = 0; k < l; ++k) {
-    const float yk = y[k];
-    const float4 s0 = *reinterpret_cast<const float4*>(S + k * ld + j0);
-    const float4 s1 = *reinterpret_cast<const float4*>(S + k * ld + j0 + 4);
-    acc[0] = fmaf(yk, s0.x, acc[0]); acc[1] = fmaf(yk, s0.y, acc[1]);
-    acc[2] = fmaf(yk, s0.z, acc[2]); acc[3] = fmaf(yk, s0.w, acc[3]);
-    acc[4] = fmaf(yk, s1.x, acc[4]); acc[5] = fmaf(yk, s1.y, acc[5]);
-    acc[6] = fmaf(yk, s1.z, acc[6]); acc[7] = fmaf(yk, s1.w, acc[7]);
-  }
-  float* o = a.out + b * a.out_bs + i * l + j0;
+  const int64_t i0 = t / cg * R;
+  if (i0 >= a.n) return;
+  const int j0 = 8 * static_cast<int>(t % cg);
+  const int nr = static_cast<int>(min(static_cast<int64_t>(R), a.n - i0));
+  const float* y = a.y + b * a.y_bs + i0 * l;
+  float acc[R][8] = {};
+  constexpr int KS = V4 ? 16 : 4;
+  for (int k0 = 0; k0 < l; k0 += KS) {
+    float yk[R][KS];
 #pragma unroll
-  for (int c = 0; c < 8; ++c)
-    if (j0 + c < l) o[c] = acc[c];
+    for (int r = 0; r < R; ++r) {
+      const float* yr = y + (r < nr ? r : 0) * l + k0;
+      if constexpr (V4) {
+#pragma unroll
+        for (int q = 0; q < KS; q += 4) {
+          const float4 v = k0 + q < l ? __ldcg(reinterpret_cast<const float4*>(yr + q)) : make_float4(0.f, 0.f, 0.f, 0.f);
+          yk[r][q] = v.x; yk[r][q + 1] = v.y; yk[r][q + 2] = v.z; yk[r][q + 3] = v.w;
+        }
+      } else {
+#pragma unroll
+        for (int q = 0; q < KS; ++q) yk[r][q] = k0 + q < l ? __ldcg(yr + q) : 0.f;
+      }
+    }
+#pragma unroll
+    for (int q = 0; q < KS; ++q) {
+      if (k0 + q < l) {
+        const float4 s0 = *reinterpret_cast<const float4*>(S + (k0 + q) * ld + j0);
+        const float4 s1 = *reinterpret_cast<const float4*>(S + (k0 + q) * ld + j0 + 4);
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+          const float v = yk[r][q];
+          acc[r][0] = fmaf(v, s0.x, acc[r][0]); acc[r][1] = fmaf(v, s0.y, acc[r][1]);
+          acc[r][2] = fmaf(v, s0.z, acc[r][2]); acc[r][3] = fmaf(v, s0.w, acc[r][3]);
+          acc[r][4] = fmaf(v, s1.x, acc[r][4]); acc[r][5] = fmaf(v, s1.y, acc[r][5]);
+          acc[r][6] = fmaf(v, s1.z, acc[r][6]); acc[r][7] = fmaf(v, s1.w, acc[r][7]);
+        }
+      }
+    }
+  }
+#pragma unroll
+  for (int r = 0; r < R; ++r) {
+    if (r >= nr) continue;
+    float* o = a.out + b * a.out_bs + (i0 + r) * l + j0;
+    if (V4 && j0 + 8 <= l) {
+      *reinterpret_cast<float4*>(o) = make_float4(acc[r][0], acc[r][1], acc[r][2], acc[r][3]);
+      *reinterpret_cast<float4*>(o + 4) = make_float4(acc[r][4], acc[r][5], acc[r][6], acc[r][7]);
+    } else {
+#pragma unroll
+      for (int c = 0; c < 8; ++c)
+        if (j0 + c < l) o[c] = acc[r][c];
+    }
+  }
 }
 
 // ---------------------------------------------------------------------------
@@ -2759,7 +2803,17 @@ cudaError_t run_sketch_group(SketchGroup& g, const SketchParams& p, const int* m
     RowMulArgs rm;
     rm.y = k_on_b ? g.bt : g.q; rm.y_bs = vbs; rm.s = g.kmat; rm.s_bs = sq;
     rm.out = g.qk; rm.out_bs = vbs; rm.n = k_on_b ? n_a : m_a; rm.l = l;
-    launch_pdl(ov, k_rowmul, dim3(static_cast<unsigned>(cdiv(rm.n * ((l + 7) / 8), 256)), B), dim3(256), 0, s, rm);
+    const bool v4 = (l % 4 == 0) && (vbs % 4 == 0) && (sq % 4 == 0) &&
+                    ((reinterpret_cast<uintptr_t>(rm.y) | reinterpret_cast<uintptr_t>(rm.out) |
+                      reinterpret_cast<uintptr_t>(rm.s)) % 16 == 0);
+    const int cgs = (l + 7) / 8;
+    const int64_t planned = g.plan_batch ? g.plan_batch : B;
+    const bool four = cdiv(rm.n * cgs, 4 * 256) * planned >= device_sm_count();
+    const dim3 rgrid(static_cast<unsigned>(cdiv(cdiv(rm.n, four ? 4 : 1) * cgs, 256)), B);
+    if (v4 && four) launch_pdl(ov, k_rowmul<true, 4>, rgrid, dim3(256), 0, s, rm);
+    else if (v4) launch_pdl(ov, k_rowmul<true, 1>, rgrid, dim3(256), 0, s, rm);
+    else if (four) launch_pdl(ov, k_rowmul<false, 4>, rgrid, dim3(256), 0, s, rm);
+    else launch_pdl(ov, k_rowmul<false, 1>, rgrid, dim3(256), 0, s, rm);
     NP_CHECK();
   }
   prof->end(kProfEig, s, (p.exact ? 1 : 3) + n_fold);
