@@ -2083,15 +2083,21 @@ __global__ void __launch_bounds__(256) k_apply_l(const __grid_constant__ LApplyA
 // Persistent: CTA c takes a contiguous range of units (matrix, row tile of nt
 // rows, column tile), column tiles fastest, so the Lm tile is split once per
 // row tile.  nt is 256, or less where that leaves SMs idle: one 256 x 1024
-// matrix is 8 units of 256 rows or 32 of 64.  Warps 0-1 split the panel rows into the shared-memory operands
-// (K-major, 128-byte swizzle, 32-wide K atoms), warp 2 issues the MMAs into
-// one of two TMEM accumulators (256 columns each), warps 3-10 drain an
-// accumulator into the weight update while the next unit's operands and MMAs
-// proceed.
+// matrix is 8 units of 256 rows or 32 of 64.  Warps 0-2 split the panel rows
+// into the shared-memory operands (K-major, 128-byte swizzle, 32-wide K atoms),
+// warp 3 issues the MMAs into one of two TMEM accumulators (256 columns each),
+// warps 4-11 drain an accumulator into the weight update while the next unit's
+// operands and MMAs proceed.
+//
+// The operand split paces a bf16 unit: one operand buffer, so a unit takes at
+// least its split (a 128 x l tile, mostly L2 latency and address arithmetic)
+// and its MMAs.  With two warps, eight loads a round and a division per piece
+// that was about 17 thousand cycles a unit, in bf16 and fp32 alike, twice what
+// the bf16 stream needs.
 // ---------------------------------------------------------------------------
 constexpr int kAtcRows = 256;                         // most W rows per unit (MMA N = nt)
 constexpr int kAtcCols = 128;                         // W columns per unit (MMA M)
-constexpr int kAtcProd = 2, kAtcEpi = 8;
+constexpr int kAtcProd = 3, kAtcEpi = 8;
 constexpr int kAtcChunk = 16, kAtcSlots = 3;       // epilogue: rows per chunk, register ring slots
 constexpr int kAtcThreads = 32 * (kAtcProd + 1 + kAtcEpi);
 constexpr int kAtcAtomA = kAtcCols * 128;             // one 32-wide K atom of the A (Rm) tile
@@ -2099,32 +2105,33 @@ constexpr int kAtcAtomB = kAtcRows * 128;             // one 32-wide K atom of t
 static size_t atc_smem(int natoms) { return 1024 + static_cast<size_t>(natoms) * 2 * (kAtcAtomA + kAtcAtomB) + 256; }
 
 // rows [r0, r0 + R) of a panel (row stride l floats) split into hi / lo
-// swizzled K-major tiles; rows past `nrows` are zero.  Eight 16-byte loads
-// per thread are in flight before the first split.
-__device__ __forceinline__ void atc_split_rows(const float* panel, int64_t r0, int64_t nrows, int R, int l, uint8_t* hi,
-                                               uint8_t* lo, int atom_bytes, int ptid) {
-  constexpr int NT = 32 * kAtcProd, B = 8;
+// swizzled K-major tiles; rows past `nrows` are zero.  Fourteen 16-byte loads per
+// thread are in flight before the first split (128 rows at l = 40: one round
+// trip).  inv = ceil(2^16 / (l / 4)): idx * inv >> 16 is idx / (l / 4) for
+// idx < 4096 = 256 rows of 64 columns.
+__device__ __forceinline__ void atc_split_rows(const float* panel, int64_t r0, int64_t nrows, int R, int l, uint32_t inv,
+                                               uint8_t* hi, uint8_t* lo, int atom_bytes, int ptid) {
+  constexpr int NT = 32 * kAtcProd, B = 14;
   const int l4 = l >> 2;
   const int n = R * l4;
   const float* src = panel + r0 * l;
-  const int64_t valid = (nrows - r0) * l4;   // float4s of rows below nrows
+  const int64_t left = (nrows - r0) * l4;    // float4s of rows below nrows
+  const int valid = static_cast<int>(left < n ? left : n);
   for (int base = ptid; base < n; base += B * NT) {
     float4 x[B];
 #pragma unroll
     for (int k = 0; k < B; ++k) {
       const int idx = base + k * NT;
-      x[k] = (idx < n && idx < valid) ? __ldcg(reinterpret_cast<const float4*>(src) + idx)
-                                      : make_float4(0.f, 0.f, 0.f, 0.f);
+      x[k] = idx < valid ? __ldcg(reinterpret_cast<const float4*>(src) + idx) : make_float4(0.f, 0.f, 0.f, 0.f);
     }
 #pragma unroll
     for (int k = 0; k < B; ++k) {
       const int idx = base + k * NT;
       if (idx < n) {
-        const int r = idx / l4, c4 = idx - r * l4;
+        const int r = static_cast<int>((static_cast<uint32_t>(idx) * inv) >> 16), c4 = idx - r * l4;
         float4 h, lw;
         split4(x[k], h, lw);
-        const int kk = 4 * c4;
-        const uint32_t off = static_cast<uint32_t>((kk >> 5) * atom_bytes) + sw128(r, (kk & 31) >> 2);
+        const uint32_t off = static_cast<uint32_t>((c4 >> 3) * atom_bytes) + sw128(r, c4 & 7);
         *reinterpret_cast<float4*>(hi + off) = h;
         *reinterpret_cast<float4*>(lo + off) = lw;
       }
@@ -2191,6 +2198,7 @@ __global__ void __launch_bounds__(kAtcThreads, 1) k_apply_tc(const __grid_consta
   if (warp < kAtcProd) {
     // ---------------- operand split ----------------
     const int ptid = threadIdx.x;
+    const uint32_t inv = static_cast<uint32_t>(65536 + (l >> 2) - 1) / static_cast<uint32_t>(l >> 2);
     bool ok = true;
     int64_t b_key = -1;
     uint32_t it = 0;
@@ -2204,9 +2212,9 @@ __global__ void __launch_bounds__(kAtcThreads, 1) k_apply_tc(const __grid_consta
       // of them overwrites a tile: the MMAs that read them are done (opfree)
       const int64_t key = static_cast<int64_t>(b) * rt + i0 / nt;
       if (key != b_key)
-        atc_split_rows(a.lm + b * a.lm_bs, i0, a.rows, nt, l, b_hi, b_lo, kAtcAtomB, ptid);
+        atc_split_rows(a.lm + b * a.lm_bs, i0, a.rows, nt, l, inv, b_hi, b_lo, kAtcAtomB, ptid);
       b_key = key;
-      atc_split_rows(a.rm + b * a.rm_bs, j0, a.cols, kAtcCols, l, a_hi, a_lo, kAtcAtomA, ptid);
+      atc_split_rows(a.rm + b * a.rm_bs, j0, a.cols, kAtcCols, l, inv, a_hi, a_lo, kAtcAtomA, ptid);
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
       __syncwarp();
       if (lane == 0) tc::mbar_arrive(opfull);
