@@ -1548,9 +1548,9 @@ struct RowMulArgs {
 // One thread per (R rows, 8 consecutive columns): two 16-byte shared loads of S
 // serve 8 FMAs of every row, and V4 (l % 4 == 0, 16-byte aligned rows) reads 16
 // entries of each row at a time.  Four rows per thread where that still fills
-// the SMs, bound by the shared loads (with one row and scalar loads of Y the
-// Qwen3 groups took 45 us); one row otherwise, where it is bound by the round
-// trips to L2.
+// the SMs, bound by the shared loads (a Qwen3 group: 20 us; with one row and
+// scalar loads of Y 45 us); one row otherwise, where it is bound by the round
+// trips to L2 (a GPT-2 group: 10 us, 12 before).
 template <bool V4, int R>
 __global__ void __launch_bounds__(256) k_rowmul(const __grid_constant__ RowMulArgs a) {
   __shared__ __align__(16) float S[kLmax * (kLmax + 8)];
@@ -2089,11 +2089,12 @@ __global__ void __launch_bounds__(256) k_apply_l(const __grid_constant__ LApplyA
 // warps 4-11 drain an accumulator into the weight update while the next unit's
 // operands and MMAs proceed.
 //
-// The operand split paces a bf16 unit: one operand buffer, so a unit takes at
-// least its split (a 128 x l tile, mostly L2 latency and address arithmetic)
-// and its MMAs.  With two warps, eight loads a round and a division per piece
-// that was about 17 thousand cycles a unit, in bf16 and fp32 alike, twice what
-// the bf16 stream needs.
+// The split and the MMAs of a unit are in series on one operand buffer.  With
+// three splitting warps, a tile's loads in one round trip and no division per
+// piece, against two warps, eight loads a round and a division: 341 against
+// 356 us a Qwen3 launch (bf16), 54 against 59 us a GPT-2 launch (fp32).  fp32
+// launches as large as LLaMA 1B's reach 5.5 TB/s; what paces bf16 (3.5 TB/s, 24
+// instructions an element in the drain, its warps waiting for loads) is open.
 // ---------------------------------------------------------------------------
 constexpr int kAtcRows = 256;                         // most W rows per unit (MMA N = nt)
 constexpr int kAtcCols = 128;                         // W columns per unit (MMA M)
