@@ -2089,15 +2089,23 @@ __global__ void __launch_bounds__(256) k_apply_l(const __grid_constant__ LApplyA
 // warps 4-11 drain an accumulator into the weight update while the next unit's
 // operands and MMAs proceed.
 //
+// PAIR (bf16 W and Psi, rows of even width): a lane holds two adjacent columns.
+// The unit is 256 columns by nt <= 128 rows, its even and odd columns two M = 128
+// tiles whose accumulators lie side by side in TMEM, so that a warp reads rows of
+// 128 bytes in one word a lane, as fp32 does; row tiles are fastest, so the
+// larger operand, now Rm's, is the one that is split once per column tile.  One
+// column a lane left 64-byte rows and half as many bytes in flight for the same
+// registers: 341 us a Qwen3 launch (201 M elements, 3.5 TB/s), 258 now (4.7).
+//
 // The split and the MMAs of a unit are in series on one operand buffer.  With
 // three splitting warps, a tile's loads in one round trip and no division per
-// piece, against two warps, eight loads a round and a division: 341 against
-// 356 us a Qwen3 launch (bf16), 54 against 59 us a GPT-2 launch (fp32).  fp32
-// launches as large as LLaMA 1B's reach 5.5 TB/s; what paces bf16 (3.5 TB/s, 24
-// instructions an element in the drain, its warps waiting for loads) is open.
+// piece, against two warps, eight loads a round and a division: 54 against 59 us
+// a GPT-2 launch (fp32).  What bounds it is HBM: fp32 launches as large as LLaMA
+// 1B's reach 5.5 TB/s, the rest of the peak goes to the ramps of the units' loads.
 // ---------------------------------------------------------------------------
 constexpr int kAtcRows = 256;                         // most W rows per unit (MMA N = nt)
 constexpr int kAtcCols = 128;                         // W columns per unit (MMA M)
+constexpr int kAtcPairCol = 128;                      // PAIR: TMEM columns of one parity (nt <= 128)
 constexpr int kAtcProd = 3, kAtcEpi = 8;
 constexpr int kAtcChunk = 16, kAtcSlots = 3;       // epilogue: rows per chunk, register ring slots
 constexpr int kAtcThreads = 32 * (kAtcProd + 1 + kAtcEpi);
@@ -2110,6 +2118,8 @@ static size_t atc_smem(int natoms) { return 1024 + static_cast<size_t>(natoms) *
 // thread are in flight before the first split (128 rows at l = 40: one round
 // trip).  inv = ceil(2^16 / (l / 4)): idx * inv >> 16 is idx / (l / 4) for
 // idx < 4096 = 256 rows of 64 columns.
+// PAIR: even rows go to the first half of the tile, odd rows to the second.
+template <bool PAIR>
 __device__ __forceinline__ void atc_split_rows(const float* panel, int64_t r0, int64_t nrows, int R, int l, uint32_t inv,
                                                uint8_t* hi, uint8_t* lo, int atom_bytes, int ptid) {
   constexpr int NT = 32 * kAtcProd, B = 14;
@@ -2132,7 +2142,8 @@ __device__ __forceinline__ void atc_split_rows(const float* panel, int64_t r0, i
         const int r = static_cast<int>((static_cast<uint32_t>(idx) * inv) >> 16), c4 = idx - r * l4;
         float4 h, lw;
         split4(x[k], h, lw);
-        const uint32_t off = static_cast<uint32_t>((c4 >> 3) * atom_bytes) + sw128(r, c4 & 7);
+        const int tr = PAIR ? (r & 1) * (R >> 1) + (r >> 1) : r;
+        const uint32_t off = static_cast<uint32_t>((c4 >> 3) * atom_bytes) + sw128(tr, c4 & 7);
         *reinterpret_cast<float4*>(hi + off) = h;
         *reinterpret_cast<float4*>(lo + off) = lw;
       }
@@ -2140,16 +2151,18 @@ __device__ __forceinline__ void atc_split_rows(const float* panel, int64_t r0, i
   }
 }
 
-template <typename TW, typename TP>
+template <typename TW, typename TP, bool PAIR>
 __global__ void __launch_bounds__(kAtcThreads, 1) k_apply_tc(const __grid_constant__ LApplyArgs a, int nmat, int nt,
                                                               int natoms, int* flags) {
   extern __shared__ uint8_t atc_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(atc_raw) + 1023) & ~uintptr_t(1023));
+  constexpr int UC = PAIR ? 2 * kAtcCols : kAtcCols;                 // W columns per unit
+  constexpr int AtomA = PAIR ? kAtcAtomB : kAtcAtomA, AtomB = PAIR ? kAtcAtomA : kAtcAtomB;
   uint8_t* a_hi = smem;
-  uint8_t* a_lo = a_hi + natoms * kAtcAtomA;
-  uint8_t* b_hi = a_lo + natoms * kAtcAtomA;
-  uint8_t* b_lo = b_hi + natoms * kAtcAtomB;
-  uint64_t* opfull = reinterpret_cast<uint64_t*>(b_lo + natoms * kAtcAtomB);   // operands written
+  uint8_t* a_lo = a_hi + natoms * AtomA;
+  uint8_t* b_hi = a_lo + natoms * AtomA;
+  uint8_t* b_lo = b_hi + natoms * AtomB;
+  uint64_t* opfull = reinterpret_cast<uint64_t*>(b_lo + natoms * AtomB);       // operands written
   uint64_t* opfree = opfull + 1;                                               // MMAs done with them
   uint64_t* tfull = opfree + 1;                                                // [2] accumulator ready
   uint64_t* tempty = tfull + 2;                                                // [2] accumulator drained
@@ -2157,16 +2170,17 @@ __global__ void __launch_bounds__(kAtcThreads, 1) k_apply_tc(const __grid_consta
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int64_t rt = (a.rows + nt - 1) / nt, ct = (a.cols + kAtcCols - 1) / kAtcCols;
+  const int64_t rt = (a.rows + nt - 1) / nt, ct = (a.cols + UC - 1) / UC;
   const int64_t per_mat = rt * ct;
   const int64_t units = per_mat * nmat;
   const int64_t u0 = units * blockIdx.x / gridDim.x, u1 = units * (blockIdx.x + 1) / gridDim.x;
-  // column tiles fastest: consecutive units of a CTA share the Lm tile
+  // column tiles fastest: consecutive units of a CTA share the Lm tile (PAIR:
+  // row tiles, the Rm tile, each time the larger operand)
   auto unit_of = [&](int64_t u, int& b, int64_t& i0, int64_t& j0) {
     b = static_cast<int>(u / per_mat);
     const int64_t rem = u - b * per_mat;
-    i0 = (rem / ct) * nt;
-    j0 = (rem % ct) * kAtcCols;
+    i0 = (PAIR ? rem % rt : rem / ct) * nt;
+    j0 = (PAIR ? rem / rt : rem % ct) * UC;
   };
   if (threadIdx.x == 0) {
     tc::mbar_init(opfull, kAtcProd);
@@ -2201,7 +2215,7 @@ __global__ void __launch_bounds__(kAtcThreads, 1) k_apply_tc(const __grid_consta
     const int ptid = threadIdx.x;
     const uint32_t inv = static_cast<uint32_t>(65536 + (l >> 2) - 1) / static_cast<uint32_t>(l >> 2);
     bool ok = true;
-    int64_t b_key = -1;
+    int64_t held = -1;
     uint32_t it = 0;
     for (int64_t u = u0; u < u1 && ok; ++u, ++it) {
       int b;
@@ -2211,11 +2225,12 @@ __global__ void __launch_bounds__(kAtcThreads, 1) k_apply_tc(const __grid_consta
       if (!ok) break;
       // the warps of this role finish the previous unit's writes before any
       // of them overwrites a tile: the MMAs that read them are done (opfree)
-      const int64_t key = static_cast<int64_t>(b) * rt + i0 / nt;
-      if (key != b_key)
-        atc_split_rows(a.lm + b * a.lm_bs, i0, a.rows, nt, l, inv, b_hi, b_lo, kAtcAtomB, ptid);
-      b_key = key;
-      atc_split_rows(a.rm + b * a.rm_bs, j0, a.cols, kAtcCols, l, inv, a_hi, a_lo, kAtcAtomA, ptid);
+      const int64_t key = PAIR ? b * ct + j0 / UC : b * rt + i0 / nt;
+      if (PAIR || key != held)
+        atc_split_rows<false>(a.lm + b * a.lm_bs, i0, a.rows, nt, l, inv, b_hi, b_lo, AtomB, ptid);
+      if (!PAIR || key != held)
+        atc_split_rows<PAIR>(a.rm + b * a.rm_bs, j0, a.cols, UC, l, inv, a_hi, a_lo, AtomA, ptid);
+      held = key;
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
       __syncwarp();
       if (lane == 0) tc::mbar_arrive(opfull);
@@ -2237,13 +2252,17 @@ __global__ void __launch_bounds__(kAtcThreads, 1) k_apply_tc(const __grid_consta
         const uint32_t d = tmem_base + static_cast<uint32_t>(256 * acc);
         for (int kk = 0; kk < ksteps; ++kk) {
           const uint32_t off = static_cast<uint32_t>(kk & 3) * 32u;
-          const uint32_t aa = static_cast<uint32_t>(kk >> 2) * kAtcAtomA + off;
-          const uint32_t bb = static_cast<uint32_t>(kk >> 2) * kAtcAtomB + off;
-          const uint64_t dah = tc::sdesc(tc::su32(a_hi) + aa, 16, 1024), dal = tc::sdesc(tc::su32(a_lo) + aa, 16, 1024);
+          const uint32_t bb = static_cast<uint32_t>(kk >> 2) * AtomB + off;
           const uint64_t dbh = tc::sdesc(tc::su32(b_hi) + bb, 16, 1024), dbl = tc::sdesc(tc::su32(b_lo) + bb, 16, 1024);
-          tc::mma_tf32(d, dah, dbh, idesc, kk > 0 ? 1u : 0u);
-          tc::mma_tf32(d, dah, dbl, idesc, 1u);
-          tc::mma_tf32(d, dal, dbh, idesc, 1u);
+#pragma unroll
+          for (int p = 0; p < UC / kAtcCols; ++p) {     // PAIR: even, then odd W columns
+            const uint32_t aa = static_cast<uint32_t>(kk >> 2) * AtomA + p * kAtcAtomA + off;
+            const uint64_t dah = tc::sdesc(tc::su32(a_hi) + aa, 16, 1024), dal = tc::sdesc(tc::su32(a_lo) + aa, 16, 1024);
+            const uint32_t dp = d + kAtcPairCol * p;
+            tc::mma_tf32(dp, dah, dbh, idesc, kk > 0 ? 1u : 0u);
+            tc::mma_tf32(dp, dah, dbl, idesc, 1u);
+            tc::mma_tf32(dp, dal, dbh, idesc, 1u);
+          }
         }
         tc::mma_commit(opfree);
         tc::mma_commit(&tfull[acc]);
@@ -2274,14 +2293,17 @@ __global__ void __launch_bounds__(kAtcThreads, 1) k_apply_tc(const __grid_consta
     int icc = 0;
     int cur_b = -1;
     float cur_ct = 0.f;
-    TP pv[S][CH];
-    TW wv[S][CH];
+    // what a lane reads of a row of Psi and of W: one entry, or (PAIR) two
+    using PT = std::conditional_t<PAIR, uint32_t, TP>;
+    using WT = std::conditional_t<PAIR, uint32_t, TW>;
+    PT pv[S][CH];
+    WT wv[S][CH];
     TW* wp[S];
     int nr[S];
     float ctt[S];
-    auto issue = [&](int64_t k, TP* P, TW* Wv, TW*& wptr, int& nrows, float& ct) {
+    auto issue = [&](int64_t k, PT* P, WT* Wv, TW*& wptr, int& nrows, float& cts) {
       if (k < nck) {
-        const int64_t j = ij0 + 32 * q + lane;
+        const int64_t j = ij0 + (UC / 4) * q + (UC / kAtcCols) * lane;
         const int64_t r0 = ii0 + hrow + CH * icc;
         if (ib != cur_b) {
           // fp64 throughput is low on this part: one lane per warp forms the
@@ -2294,30 +2316,39 @@ __global__ void __launch_bounds__(kAtcThreads, 1) k_apply_tc(const __grid_consta
           cur_ct = -a.lr * __shfl_sync(0xffffffffu, scale, 0);
           cur_b = ib;
         }
-        ct = cur_ct;
+        cts = cur_ct;
         const TP* pptr = static_cast<const TP*>(a.psi) + ib * a.psi_bs + r0 * a.psi_ld + j;
         wptr = static_cast<TW*>(a.W[ib]) + r0 * a.cols + j;
         nrows = (r0 < a.rows && j < a.cols) ? static_cast<int>(a.rows - r0 < CH ? a.rows - r0 : CH) : 0;
         if (nrows == CH) {
 #pragma unroll
           for (int rr = 0; rr < CH; ++rr) {
-            P[rr] = __ldcs(pptr + rr * a.psi_ld);
-            Wv[rr] = wptr[rr * a.cols];
+            P[rr] = __ldcs(reinterpret_cast<const PT*>(pptr + rr * a.psi_ld));
+            Wv[rr] = *reinterpret_cast<const WT*>(wptr + rr * a.cols);
           }
         } else {
 #pragma unroll
           for (int rr = 0; rr < CH; ++rr) {
-            P[rr] = rr < nrows ? pptr[rr * a.psi_ld] : from_f32<TP>(0.f);
-            Wv[rr] = rr < nrows ? wptr[rr * a.cols] : from_f32<TW>(0.f);
+            P[rr] = rr < nrows ? *reinterpret_cast<const PT*>(pptr + rr * a.psi_ld) : PT(0.f);
+            Wv[rr] = rr < nrows ? *reinterpret_cast<const WT*>(wptr + rr * a.cols) : WT(0.f);
           }
         }
         if (++icc == NCH) {
           icc = 0;
-          ij0 += kAtcCols;
-          if (ij0 >= a.cols) {
-            ij0 = 0;
+          if constexpr (PAIR) {
             ii0 += nt;
-            if (ii0 >= a.rows) { ii0 = 0; ++ib; }
+            if (ii0 >= a.rows) {
+              ii0 = 0;
+              ij0 += UC;
+              if (ij0 >= a.cols) { ij0 = 0; ++ib; }
+            }
+          } else {
+            ij0 += UC;
+            if (ij0 >= a.cols) {
+              ij0 = 0;
+              ii0 += nt;
+              if (ii0 >= a.rows) { ii0 = 0; ++ib; }
+            }
           }
         }
       }
@@ -2338,8 +2369,10 @@ __global__ void __launch_bounds__(kAtcThreads, 1) k_apply_tc(const __grid_consta
           if (!ok) break;
           tc::fence_after();
         }
-        uint32_t v[CH];
-        tc::tmem_ld16(tmem_base + (static_cast<uint32_t>(32 * q) << 16) + static_cast<uint32_t>(256 * acc + hrow + CH * c), v);
+        uint32_t v[CH], vo[CH];
+        const uint32_t dcol = tmem_base + (static_cast<uint32_t>(32 * q) << 16) + static_cast<uint32_t>(256 * acc + hrow + CH * c);
+        tc::tmem_ld16(dcol, v);
+        if constexpr (PAIR) tc::tmem_ld16(dcol + kAtcPairCol, vo);
         tc::tmem_ld_wait();
         if (++c == NCH) {
           // the accumulator is read: the MMAs of unit un + 2 may overwrite it
@@ -2350,15 +2383,23 @@ __global__ void __launch_bounds__(kAtcThreads, 1) k_apply_tc(const __grid_consta
           ++un;
         }
         TW* W = wp[sl];
+        auto step = [&](float w, float p, uint32_t d) { return fmaf(cw, w, ctt[sl] * (p + __uint_as_float(d))); };
+        auto put = [&](int rr) {
+          if constexpr (PAIR) {
+            const uint32_t w2 = wv[sl][rr], p2 = pv[sl][rr];
+            *reinterpret_cast<uint32_t*>(W + rr * a.cols) =
+                pack_bf16x2(step(bf16lo(w2), bf16lo(p2), v[rr]), step(bf16hi(w2), bf16hi(p2), vo[rr]));
+          } else {
+            W[rr * a.cols] = from_f32<TW>(step(to_f32(wv[sl][rr]), to_f32(pv[sl][rr]), v[rr]));
+          }
+        };
         if (nr[sl] == CH) {
 #pragma unroll
-          for (int rr = 0; rr < CH; ++rr)
-            W[rr * a.cols] = from_f32<TW>(fmaf(cw, to_f32(wv[sl][rr]), ctt[sl] * (to_f32(pv[sl][rr]) + __uint_as_float(v[rr]))));
+          for (int rr = 0; rr < CH; ++rr) put(rr);
         } else {
 #pragma unroll
           for (int rr = 0; rr < CH; ++rr)
-            if (rr < nr[sl])
-              W[rr * a.cols] = from_f32<TW>(fmaf(cw, to_f32(wv[sl][rr]), ctt[sl] * (to_f32(pv[sl][rr]) + __uint_as_float(v[rr]))));
+            if (rr < nr[sl]) put(rr);
         }
         issue(k + S, pv[sl], wv[sl], wp[sl], nr[sl], ctt[sl]);
       }
@@ -2503,7 +2544,8 @@ cudaError_t sketch_group_alloc(SketchGroup& g, int rank, int oversample, std::ve
     cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kCqMaxSmem));
   contract_attrs<false>();
   contract_attrs<true>();
-  for (auto fn : {k_apply_tc<float, float>, k_apply_tc<float, bf16>, k_apply_tc<bf16, float>, k_apply_tc<bf16, bf16>})
+  for (auto fn : {k_apply_tc<float, float, false>, k_apply_tc<float, bf16, false>, k_apply_tc<bf16, float, false>,
+                  k_apply_tc<bf16, bf16, false>, k_apply_tc<bf16, bf16, true>})
     cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(atc_smem(2)));
   // tensor-core contractions: Psi as a 3-D tensor {cols, rows, batch}; the
   // l-wide operands need 16-byte rows and matrix strides (checked per launch)
@@ -2864,20 +2906,30 @@ cudaError_t run_sketch_group(SketchGroup& g, const SketchParams& p, const int* m
       const size_t smem = atc_smem(2);
       int nt = kAtcRows;
       while (nt > 64 && cdiv(g.rows, nt) * cdiv(g.cols, kAtcCols) * nb < device_sm_count()) nt /= 2;
+      // two columns a lane where its units, wider than they are tall, fill the
+      // SMs; below that a step of 8 x 512 x 1024 (17.4 us narrow, 18.0 wide), 4 x
+      // 512 x 512 (11.3, 13.3) or 2048 x 2048 (17.3, 16.3) gains nothing by it
+      const bool pair = g.w_dtype != 0 && g.psi_bf16 && g.cols % 2 == 0 && g.ld % 2 == 0 &&
+                        cdiv(g.rows, kAtcPairCol) * cdiv(g.cols, 2 * kAtcCols) * nb >= device_sm_count();
+      if (pair) nt = kAtcPairCol;
       const int kind = 2 * (g.w_dtype != 0) + (g.psi_bf16 ? 1 : 0);
-      auto go = [&](auto* tw, auto* tp) -> cudaError_t {
+      auto go = [&](auto* tw, auto* tp, auto two) -> cudaError_t {
         using TWT = std::remove_pointer_t<decltype(tw)>;
         using TPT = std::remove_pointer_t<decltype(tp)>;
-        const int64_t units = cdiv(g.rows, nt) * cdiv(g.cols, kAtcCols) * nb;
+        constexpr bool P = decltype(two)::value;
+        const int64_t units = cdiv(g.rows, nt) * cdiv(g.cols, P ? 2 * kAtcCols : kAtcCols) * nb;
         const unsigned ctas = static_cast<unsigned>(std::min<int64_t>(units, device_sm_count()));
-        launch_pdl(ov, k_apply_tc<TWT, TPT>, dim3(ctas), dim3(kAtcThreads), smem, s, la, nb, nt, natoms, flags);
+        launch_pdl(ov, k_apply_tc<TWT, TPT, P>, dim3(ctas), dim3(kAtcThreads), smem, s, la, nb, nt, natoms, flags);
         return cudaGetLastError();
       };
       switch (kind) {
-        case 0: e = go((float*)nullptr, (float*)nullptr); break;
-        case 1: e = go((float*)nullptr, (bf16*)nullptr); break;
-        case 2: e = go((bf16*)nullptr, (float*)nullptr); break;
-        default: e = go((bf16*)nullptr, (bf16*)nullptr); break;
+        case 0: e = go((float*)nullptr, (float*)nullptr, std::false_type{}); break;
+        case 1: e = go((float*)nullptr, (bf16*)nullptr, std::false_type{}); break;
+        case 2: e = go((bf16*)nullptr, (float*)nullptr, std::false_type{}); break;
+        default:
+          e = pair ? go((bf16*)nullptr, (bf16*)nullptr, std::true_type{})
+                   : go((bf16*)nullptr, (bf16*)nullptr, std::false_type{});
+          break;
       }
       if (e != cudaSuccess) return e;
       NP_CHECK();

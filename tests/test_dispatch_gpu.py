@@ -164,6 +164,48 @@ def test_sketch_basis_and_ritz_pairs(rows, cols, rank, oversample, t):
 
 
 # ---------------------------------------------------------------------------
+# NormPre-L apply, bf16 W and Psi: two W columns a lane where the launch has
+# enough units and its rows have an even width, one column a lane elsewhere
+# ---------------------------------------------------------------------------
+@pytest.mark.parametrize("t", [0, 1])
+@pytest.mark.parametrize("rows,cols,n,rank", [(130, 520, 30, 40), (1000, 510, 12, 16), (513, 1030, 8, 36),
+                                              (37, 1300, 30, 32), (641, 2, 31, 16), (256, 770, 33, 64),
+                                              (1, 1290, 30, 4)])
+def test_apply_two_columns_a_lane(rows, cols, n, rank, t):
+    """W_new against cw W + ct (Psi + Q K Q^T Psi) formed in fp64 from the step's
+    own Psi, Q and Ritz pairs, cw and ct fitted.  W_new is rounded to bf16, 2^-9 of
+    it; Q, the Ritz pairs and the panels are fp32, 2e-5 each of the largest entry
+    (as the basis test above), and the panels' largest singular value may be some
+    tens of an entry's size: 1e-3 of the largest."""
+    import torch
+    from paper_2609_36692_gb300 import normpre as C
+    from paper_2609_36692_gb300.optim import NormPre
+    gen = torch.Generator(device="cuda").manual_seed(rows + cols)
+    G = [torch.randn(rows, cols, device="cuda", generator=gen).bfloat16() for _ in range(n)]
+    M = [torch.randn(rows, cols, device="cuda", generator=gen) for _ in range(n)]
+    W0 = [(torch.randn(rows, cols, device="cuda", generator=gen) * 0.02).bfloat16() for _ in range(n)]
+    W = [x.clone() for x in W0]
+    opt = NormPre([(rows, cols)] * n, ["bf16"] * n, ["bf16"] * n, variant=C.NORMPRE_L, precision=0, rank=rank,
+                  oversample=0)
+    opt.step(t, 0.5, W, G, M)
+    assert opt.status() == C.NORMPRE_OK
+    for i in range(n):
+        psi = opt.read(i, C.NORMPRE_BUF_PSI).astype(np.float64)
+        pa = psi if t == 0 else psi.T
+        Q = opt.read(i, C.NORMPRE_BUF_Q).astype(np.float64)
+        Z = opt.read(i, C.NORMPRE_BUF_Z).astype(np.float64)
+        lam = opt.read(i, C.NORMPRE_BUF_RITZ)[0].astype(np.float64)
+        gain = 1.0 / np.sqrt(np.maximum(lam, 1.0)) - 1.0     # of the values above one
+        T = pa + Q @ ((Z * gain) @ (Z.T @ (Q.T @ pa)))
+        T = T if t == 0 else T.T
+        w0, w1 = (x[i].double().cpu().numpy() for x in (W0, W))
+        X = np.stack([w0.ravel(), T.ravel()], 1)
+        fit = (X @ np.linalg.lstsq(X, w1.ravel(), rcond=None)[0]).reshape(rows, cols)
+        assert np.all(np.abs(w1 - fit) <= 2.0 ** -8 * np.abs(w1) + 1e-3 * np.abs(w1).max()), (i, np.abs(w1 - fit).max())
+    opt.close()
+
+
+# ---------------------------------------------------------------------------
 # non-finite gradients: the step is reported, nothing faults, and the handle's
 # next step on finite inputs is that of a fresh one
 # ---------------------------------------------------------------------------
