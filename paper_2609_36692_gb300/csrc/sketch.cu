@@ -2089,13 +2089,15 @@ __global__ void __launch_bounds__(256) k_apply_l(const __grid_constant__ LApplyA
 // warps 4-11 drain an accumulator into the weight update while the next unit's
 // operands and MMAs proceed.
 //
-// PAIR (bf16 W and Psi, rows of even width): a lane holds two adjacent columns.
+// PAIR (W or Psi bf16, or both, rows of even width): a lane holds two adjacent columns.
 // The unit is 256 columns by nt <= 128 rows, its even and odd columns two M = 128
 // tiles whose accumulators lie side by side in TMEM, so that a warp reads rows of
-// 128 bytes in one word a lane, as fp32 does; row tiles are fastest, so the
+// 128 bytes (256 of an fp32 operand), as fp32 does with one; row tiles are fastest, so the
 // larger operand, now Rm's, is the one that is split once per column tile.  One
 // column a lane left 64-byte rows and half as many bytes in flight for the same
 // registers: 341 us a Qwen3 launch (201 M elements, 3.5 TB/s), 258 now (4.7).
+// With one of the two in fp32 (two ring slots, the same registers) GPT-2's
+// launches take 51 us instead of 66 (fp32 W) and 49 instead of 62 (fp32 Psi).
 //
 // The split and the MMAs of a unit are in series on one operand buffer.  With
 // three splitting warps, a tile's loads in one round trip and no division per
@@ -2112,6 +2114,21 @@ constexpr int kAtcThreads = 32 * (kAtcProd + 1 + kAtcEpi);
 constexpr int kAtcAtomA = kAtcCols * 128;             // one 32-wide K atom of the A (Rm) tile
 constexpr int kAtcAtomB = kAtcRows * 128;             // one 32-wide K atom of the B (Lm) tile
 static size_t atc_smem(int natoms) { return 1024 + static_cast<size_t>(natoms) * 2 * (kAtcAtomA + kAtcAtomB) + 256; }
+
+// two adjacent entries of a row
+template <typename T> struct AtcTwo;
+template <> struct AtcTwo<bf16> {
+  using type = uint32_t;
+  static __device__ __forceinline__ float lo(uint32_t v) { return bf16lo(v); }
+  static __device__ __forceinline__ float hi(uint32_t v) { return bf16hi(v); }
+  static __device__ __forceinline__ uint32_t of(float a, float b) { return pack_bf16x2(a, b); }
+};
+template <> struct AtcTwo<float> {
+  using type = float2;
+  static __device__ __forceinline__ float lo(float2 v) { return v.x; }
+  static __device__ __forceinline__ float hi(float2 v) { return v.y; }
+  static __device__ __forceinline__ float2 of(float a, float b) { return make_float2(a, b); }
+};
 
 // rows [r0, r0 + R) of a panel (row stride l floats) split into hi / lo
 // swizzled K-major tiles; rows past `nrows` are zero.  Fourteen 16-byte loads per
@@ -2283,7 +2300,7 @@ __global__ void __launch_bounds__(kAtcThreads, 1) k_apply_tc(const __grid_consta
     const int hrow = h * (nt >> 1);
     const double mn = static_cast<double>(a.rows) * static_cast<double>(a.cols);
     const float cw = 1.f - a.lr * a.wd;
-    constexpr int CH = kAtcChunk, S = kAtcSlots;
+    constexpr int CH = kAtcChunk, S = PAIR && sizeof(TW) + sizeof(TP) > 4 ? 2 : kAtcSlots;
     const int NCH = nt / (2 * kAtcChunk);
     const int64_t nck = (u1 - u0) * NCH;
     // issue cursor: the unit (matrix b, row tile i0, column tile j0) and chunk
@@ -2294,8 +2311,8 @@ __global__ void __launch_bounds__(kAtcThreads, 1) k_apply_tc(const __grid_consta
     int cur_b = -1;
     float cur_ct = 0.f;
     // what a lane reads of a row of Psi and of W: one entry, or (PAIR) two
-    using PT = std::conditional_t<PAIR, uint32_t, TP>;
-    using WT = std::conditional_t<PAIR, uint32_t, TW>;
+    using PT = std::conditional_t<PAIR, typename AtcTwo<TP>::type, TP>;
+    using WT = std::conditional_t<PAIR, typename AtcTwo<TW>::type, TW>;
     PT pv[S][CH];
     WT wv[S][CH];
     TW* wp[S];
@@ -2329,8 +2346,8 @@ __global__ void __launch_bounds__(kAtcThreads, 1) k_apply_tc(const __grid_consta
         } else {
 #pragma unroll
           for (int rr = 0; rr < CH; ++rr) {
-            P[rr] = rr < nrows ? *reinterpret_cast<const PT*>(pptr + rr * a.psi_ld) : PT(0.f);
-            Wv[rr] = rr < nrows ? *reinterpret_cast<const WT*>(wptr + rr * a.cols) : WT(0.f);
+            P[rr] = rr < nrows ? *reinterpret_cast<const PT*>(pptr + rr * a.psi_ld) : PT{};
+            Wv[rr] = rr < nrows ? *reinterpret_cast<const WT*>(wptr + rr * a.cols) : WT{};
           }
         }
         if (++icc == NCH) {
@@ -2386,9 +2403,12 @@ __global__ void __launch_bounds__(kAtcThreads, 1) k_apply_tc(const __grid_consta
         auto step = [&](float w, float p, uint32_t d) { return fmaf(cw, w, ctt[sl] * (p + __uint_as_float(d))); };
         auto put = [&](int rr) {
           if constexpr (PAIR) {
-            const uint32_t w2 = wv[sl][rr], p2 = pv[sl][rr];
-            *reinterpret_cast<uint32_t*>(W + rr * a.cols) =
-                pack_bf16x2(step(bf16lo(w2), bf16lo(p2), v[rr]), step(bf16hi(w2), bf16hi(p2), vo[rr]));
+            using W2 = AtcTwo<TW>;
+            using P2 = AtcTwo<TP>;
+            const WT w2 = wv[sl][rr];
+            const PT p2 = pv[sl][rr];
+            *reinterpret_cast<WT*>(W + rr * a.cols) =
+                W2::of(step(W2::lo(w2), P2::lo(p2), v[rr]), step(W2::hi(w2), P2::hi(p2), vo[rr]));
           } else {
             W[rr * a.cols] = from_f32<TW>(step(to_f32(wv[sl][rr]), to_f32(pv[sl][rr]), v[rr]));
           }
@@ -2545,7 +2565,8 @@ cudaError_t sketch_group_alloc(SketchGroup& g, int rank, int oversample, std::ve
   contract_attrs<false>();
   contract_attrs<true>();
   for (auto fn : {k_apply_tc<float, float, false>, k_apply_tc<float, bf16, false>, k_apply_tc<bf16, float, false>,
-                  k_apply_tc<bf16, bf16, false>, k_apply_tc<bf16, bf16, true>})
+                  k_apply_tc<bf16, bf16, false>, k_apply_tc<float, bf16, true>, k_apply_tc<bf16, float, true>,
+                  k_apply_tc<bf16, bf16, true>})
     cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(atc_smem(2)));
   // tensor-core contractions: Psi as a 3-D tensor {cols, rows, batch}; the
   // l-wide operands need 16-byte rows and matrix strides (checked per launch)
@@ -2909,7 +2930,7 @@ cudaError_t run_sketch_group(SketchGroup& g, const SketchParams& p, const int* m
       // two columns a lane where its units, wider than they are tall, fill the
       // SMs; below that a step of 8 x 512 x 1024 (17.4 us narrow, 18.0 wide), 4 x
       // 512 x 512 (11.3, 13.3) or 2048 x 2048 (17.3, 16.3) gains nothing by it
-      const bool pair = g.w_dtype != 0 && g.psi_bf16 && g.cols % 2 == 0 && g.ld % 2 == 0 &&
+      const bool pair = (g.w_dtype != 0 || g.psi_bf16) && g.cols % 2 == 0 && g.ld % 2 == 0 &&
                         cdiv(g.rows, kAtcPairCol) * cdiv(g.cols, 2 * kAtcCols) * nb >= device_sm_count();
       if (pair) nt = kAtcPairCol;
       const int kind = 2 * (g.w_dtype != 0) + (g.psi_bf16 ? 1 : 0);
@@ -2924,8 +2945,14 @@ cudaError_t run_sketch_group(SketchGroup& g, const SketchParams& p, const int* m
       };
       switch (kind) {
         case 0: e = go((float*)nullptr, (float*)nullptr, std::false_type{}); break;
-        case 1: e = go((float*)nullptr, (bf16*)nullptr, std::false_type{}); break;
-        case 2: e = go((bf16*)nullptr, (float*)nullptr, std::false_type{}); break;
+        case 1:
+          e = pair ? go((float*)nullptr, (bf16*)nullptr, std::true_type{})
+                   : go((float*)nullptr, (bf16*)nullptr, std::false_type{});
+          break;
+        case 2:
+          e = pair ? go((bf16*)nullptr, (float*)nullptr, std::true_type{})
+                   : go((bf16*)nullptr, (float*)nullptr, std::false_type{});
+          break;
         default:
           e = pair ? go((bf16*)nullptr, (bf16*)nullptr, std::true_type{})
                    : go((bf16*)nullptr, (bf16*)nullptr, std::false_type{});

@@ -164,14 +164,15 @@ def test_sketch_basis_and_ritz_pairs(rows, cols, rank, oversample, t):
 
 
 # ---------------------------------------------------------------------------
-# NormPre-L apply, bf16 W and Psi: two W columns a lane where the launch has
+# NormPre-L apply, bf16 W or Psi: two W columns a lane where the launch has
 # enough units and its rows have an even width, one column a lane elsewhere
 # ---------------------------------------------------------------------------
+@pytest.mark.parametrize("w_dtype,precision", [("bf16", 0), ("f32", 0), ("bf16", 1)])
 @pytest.mark.parametrize("t", [0, 1])
 @pytest.mark.parametrize("rows,cols,n,rank", [(130, 520, 30, 40), (1000, 510, 12, 16), (513, 1030, 8, 36),
                                               (37, 1300, 30, 32), (641, 2, 31, 16), (256, 770, 33, 64),
                                               (1, 1290, 30, 4)])
-def test_apply_two_columns_a_lane(rows, cols, n, rank, t):
+def test_apply_two_columns_a_lane(rows, cols, n, rank, t, w_dtype, precision):
     """W_new against cw W + ct (Psi + Q K Q^T Psi) formed in fp64 from the step's
     own Psi, Q and Ritz pairs, cw and ct fitted.  W_new is rounded to bf16, 2^-9 of
     it; Q, the Ritz pairs and the panels are fp32, 2e-5 each of the largest entry
@@ -181,11 +182,12 @@ def test_apply_two_columns_a_lane(rows, cols, n, rank, t):
     from paper_2609_36692_gb300 import normpre as C
     from paper_2609_36692_gb300.optim import NormPre
     gen = torch.Generator(device="cuda").manual_seed(rows + cols)
+    td = torch.bfloat16 if w_dtype == "bf16" else torch.float32
     G = [torch.randn(rows, cols, device="cuda", generator=gen).bfloat16() for _ in range(n)]
     M = [torch.randn(rows, cols, device="cuda", generator=gen) for _ in range(n)]
-    W0 = [(torch.randn(rows, cols, device="cuda", generator=gen) * 0.02).bfloat16() for _ in range(n)]
+    W0 = [(torch.randn(rows, cols, device="cuda", generator=gen) * 0.02).to(td) for _ in range(n)]
     W = [x.clone() for x in W0]
-    opt = NormPre([(rows, cols)] * n, ["bf16"] * n, ["bf16"] * n, variant=C.NORMPRE_L, precision=0, rank=rank,
+    opt = NormPre([(rows, cols)] * n, [w_dtype] * n, ["bf16"] * n, variant=C.NORMPRE_L, precision=precision, rank=rank,
                   oversample=0)
     opt.step(t, 0.5, W, G, M)
     assert opt.status() == C.NORMPRE_OK
