@@ -158,6 +158,7 @@ struct ContractArgs {
   int l;
   int ksplit;
   int64_t kchunk;                  // K range of one split (multiple of 32)
+  int v16;                         // every matrix's V begins on 16 bytes and l % 4 == 0: 16-byte copies of V
 };
 static_assert(sizeof(ContractArgs) + 64 <= 4096, "kernel arguments beyond 4 KB");
 constexpr int kCtP = 256, kCtK = 32, kCtThreads = 128;
@@ -185,7 +186,7 @@ __global__ void __launch_bounds__(kCtThreads) k_contract(const __grid_constant__
   const float* v = a.v + b * a.v_bs;
   const int l = a.l;
   const int64_t ld = a.psi_ld;
-  const bool v16 = (l % 4) == 0;
+  const bool v16 = a.v16 != 0;
 
   auto load_stage = [&](int st, int64_t k0) {
     float* S = smem + st * kCtStageFloats;
@@ -2698,6 +2699,9 @@ cudaError_t run_sketch_group(SketchGroup& g, const SketchParams& p, const int* m
     c.rows = g.rows; c.cols = g.cols; c.l = l;
     c.ksplit = ks;
     c.kchunk = round_up(cdiv(K, ks), kCtK);
+    // (with a narrower l on the other axis the matrix stride need not be a
+    // multiple of four: 4 x 5 matrices at r + o >= 5 have l = 4 and a stride of 25)
+    c.v16 = (l % 4 == 0) && (vbs % 4 == 0) && (reinterpret_cast<uintptr_t>(v) % 16 == 0);
     if (ks == 1) {
       c.out = out; c.out_bs = vbs;
     } else {

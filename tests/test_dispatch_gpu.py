@@ -128,7 +128,9 @@ def test_update_g_any_width(rows, cols, w_dtype):
                                                        (1025, 130, 9, 4), (2049, 70, 16, 0), (4097, 96, 24, 8),
                                                        (130, 600, 33, 0), (520, 1030, 39, 8), (700, 600, 40, 8),
                                                        (260, 700, 49, 0), (300, 400, 64, 1), (300, 310, 64, 8),
-                                                       (9000, 72, 8, 8), (400, 9, 16, 8)])
+                                                       (9000, 72, 8, 8), (400, 9, 16, 8),
+                                                       # l % 4 == 0 with panels whose matrix stride is odd
+                                                       (4, 5, 8, 8), (12, 39, 32, 8), (67, 16, 64, 8)])
 def test_sketch_basis_and_ritz_pairs(rows, cols, rank, oversample, t):
     """Q orthonormal on its kept columns, the Ritz pairs those of (Psi_a^T Q)'s
     Gram matrix in fp64: residuals and orthonormality at 2e-5 of the largest
