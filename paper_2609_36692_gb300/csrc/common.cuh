@@ -88,8 +88,10 @@ __device__ __forceinline__ float warp_max(float v) {
   return v;
 }
 
-// Sum of fp32 values kept as s + e by error-free additions (TwoSum), about
-// 2^-46 relative: what fp64 sums give here at 1/64 of its cost on this part.
+// Sum of fp32 values kept as s + e: the rounding errors of the additions to s
+// are exact (TwoSum), their sum e is rounded, about 2^-46 relative in all, at
+// 1/64 of what fp64 sums cost on this part.  The range is that of fp32: an
+// addition that overflows leaves NaN in e.
 struct PairSum {
   float s = 0.f, e = 0.f;
   __device__ __forceinline__ void add(float x) {

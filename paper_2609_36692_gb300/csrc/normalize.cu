@@ -10,7 +10,7 @@
 // Column-active steps (k = 1): the reduction runs down the columns of the
 // row-major layout.  Pass A streams G, M_{t-1}, W once, writes M_t and per-
 // (row block, column) partial sums of ||m||^2, <m, w> and ||w||^2; a small
-// pass folds the partials (error-free, fixed order, no atomics on floats) into
+// pass folds the partials (fp32 pairs, fixed order, no atomics on floats) into
 // a_j = <m_j, w_j> and 1/||x_j|| with ||x||^2 = ||m||^2 - a^2 (2 - ||w||^2);
 // pass B re-reads M_t and W and writes Psi.
 //
@@ -37,7 +37,20 @@ namespace normpre {
 constexpr int kColApplyRB = 64;   // rows per block of pass B (16 where that leaves SMs idle)
 constexpr int kColThreads = 256;  // 32 column chunks of 8 x 8 row lanes
 
+// The column sums are fp32 pairs (PairSum): folded in fp64 instead, every listed
+// size of both variants gives the same results bit for bit, 1.6 % later on LLaMA
+// 1B and 2.1 % on Qwen3 (24 additions and conversions per column of a block keep
+// the fp64 pipe busy for 3 us).  The fold has the range of fp64 all the same: a
+// block's sums whose pairs overflow (a column of entries of 1e18 has a squared
+// norm of 1e36 times its rows, though its row lanes stay finite) are kept at
+// 2^-4 of their size, marked by the sign bit of a sum that is never negative,
+// and a column with a marked or overflowing sum is folded in fp64.
 __device__ __forceinline__ float2* col_pairs(const NormLaunch& a) { return reinterpret_cast<float2*>(a.col_part); }
+__device__ __forceinline__ float2 mark_wide(const PairSum& p) { return make_float2(copysignf(p.s, -1.f), p.e); }
+__device__ __forceinline__ bool is_wide(float2 v) { return __float_as_int(v.x) < 0; }
+__device__ __forceinline__ double wide_value(float s, float e, bool wide) {
+  return (wide ? 16.0 : 1.0) * (static_cast<double>(s) + static_cast<double>(e));
+}
 
 // c_i of the tangent step for mode 0 relaxed, 1 none, 2 strict (mw = <m_i, w_i>,
 // ww = ||w_i||^2).
@@ -223,7 +236,7 @@ __global__ void __launch_bounds__(256) k_norm_rows_scalar(const __grid_constant_
 // ---------------------------------------------------------------------------
 // column-active pass A: momentum + column partial sums (three pairs s + e per
 // row block and column, 8 bytes each)
-// grid (ceil(cols / 256), nrb, n); thread = (column chunk cc = tid % 32, row lane rl = tid / 32)
+// grid (ceil(cols / 256), nrb, n); thread = (column chunk cc = tid % 32, row lane rl = tid / 32).
 // ---------------------------------------------------------------------------
 template <typename TG, typename TW, bool VEC>
 __global__ void __launch_bounds__(kColThreads) k_norm_cols_stats(const __grid_constant__ NormLaunch a) {
@@ -244,8 +257,13 @@ __global__ void __launch_bounds__(kColThreads) k_norm_cols_stats(const __grid_co
   if (VEC) {
     const int64_t j0 = static_cast<int64_t>(blockIdx.x) * 256 + cc * 8;
     if (j0 < cols) {
+      // a 32-bit counter takes the form with bf16 G and W from 82 registers (two
+      // CTAs per SM) to 60: a Qwen3 NormPre-L pass of two steps 16660 and 16190 us;
+      // with fp32 W it is slower (LLaMA 1B 16990 us, 16650 with 64 bits)
+      using row_t = std::conditional_t<sizeof(TG) + sizeof(TW) == 4, int, int64_t>;
+      const row_t end = static_cast<row_t>(r1);
 #pragma unroll 4
-      for (int64_t r = r0 + rl; r < r1; r += 8) {
+      for (row_t r = static_cast<row_t>(r0) + rl; r < end; r += 8) {
         float gv[8], mp[8], wv[8];
         load8(g + r * cols + j0, gv);
         load8_cg(M + r * cols + j0, mp);
@@ -312,22 +330,28 @@ __global__ void __launch_bounds__(kColThreads) k_norm_cols_stats(const __grid_co
     }
   }
   __syncthreads();
-  // fold the 8 row lanes (error-free, fixed order) and write this block's
-  // partials: 24 fp64 additions and conversions per column kept the fp64 pipe
-  // busy for 3 us a block
+  // fold the 8 row lanes (fixed order) and write this block's partials
   const int col = threadIdx.x;   // 0..255
   const int64_t j = static_cast<int64_t>(blockIdx.x) * 256 + col;
   if (j < cols) {
     PairSum s0, s1, s2;
+    bool wide = false;
+#pragma unroll 1
+    for (float f = 1.f;; f = 0.0625f) {
+      s0 = s1 = s2 = PairSum();
 #pragma unroll
-    for (int l = 0; l < 8; ++l) {
-      s0.add(part[l][0][col]);
-      s1.add(part[l][1][col]);
-      s2.add(part[l][2][col]);
+      for (int l = 0; l < 8; ++l) {
+        s0.add(f * part[l][0][col]);
+        s1.add(f * part[l][1][col]);
+        s2.add(f * part[l][2][col]);
+      }
+      wide = f != 1.f;
+      if (wide || isfinite(s0.e + s1.e + s2.e)) break;   // an addition that overflows leaves NaN in e
     }
     const int64_t nrb = gridDim.y;
     float2* p = col_pairs(a) + ((static_cast<int64_t>(b) * nrb + rb) * cols + j) * 3;
-    p[0] = make_float2(s0.s, s0.e); p[1] = make_float2(s1.s, s1.e); p[2] = make_float2(s2.s, s2.e);
+    p[0] = make_float2(s0.s, s0.e); p[1] = make_float2(s1.s, s1.e);
+    p[2] = wide ? mark_wide(s2) : make_float2(s2.s, s2.e);
   }
 }
 
@@ -348,13 +372,30 @@ __global__ void __launch_bounds__(32) k_norm_cols_final(const __grid_constant__ 
   if (j < cols) {
     PairSum p0, p1, p2;
     const float2* p = col_pairs(a) + (static_cast<int64_t>(b) * nrb * cols + j) * 3;
+    bool wide = false;
 #pragma unroll 8
     for (int rb = 0; rb < nrb; ++rb) {
       const float2 v0 = p[0], v1 = p[1], v2 = p[2];
+      wide |= is_wide(v2) || (stage == 2 && is_wide(v1));
       p0.add(PairSum{v0.x, v0.y}); p1.add(PairSum{v1.x, v1.y}); p2.add(PairSum{v2.x, v2.y});
       p += cols * 3;
     }
-    const double s0 = p0.value(), s1 = p1.value(), s2 = p2.value();
+    double s0, s1, s2;
+    if (!wide && isfinite(p0.e + p1.e + p2.e)) {
+      s0 = p0.value(); s1 = p1.value(); s2 = p2.value();
+    } else {
+      // stage 2: slot 1 has a mark of its own (k_norm_cols_xsq)
+      s0 = s1 = s2 = 0;
+#pragma unroll 1
+      for (int rb = 0; rb < nrb; ++rb) {
+        p -= cols * 3;
+        const float2 v0 = p[0], v1 = p[1], v2 = p[2];
+        const bool w2 = is_wide(v2);
+        s0 += wide_value(v0.x, v0.y, w2);
+        s1 += stage == 2 ? wide_value(fabsf(v1.x), v1.y, is_wide(v1)) : wide_value(v1.x, v1.y, w2);
+        s2 += wide_value(fabsf(v2.x), v2.y, w2);
+      }
+    }
     float2* out = a.col_coef + static_cast<int64_t>(b) * cols + j;
     if (stage == 1) {
       // strict: only the projection coefficient; the norm comes from the direct pass
@@ -440,9 +481,17 @@ __global__ void __launch_bounds__(kColThreads) k_norm_cols_xsq(const __grid_cons
   const int64_t j = static_cast<int64_t>(blockIdx.x) * 256 + col;
   if (j < cols) {
     PairSum s;
+    bool wide = false;
+#pragma unroll 1
+    for (float f = 1.f;; f = 0.0625f) {
+      s = PairSum();
 #pragma unroll
-    for (int l = 0; l < 8; ++l) s.add(part[l][col]);
-    col_pairs(a)[((static_cast<int64_t>(b) * gridDim.y + rb) * cols + j) * 3 + 1] = make_float2(s.s, s.e);
+      for (int l = 0; l < 8; ++l) s.add(f * part[l][col]);
+      wide = f != 1.f;
+      if (wide || isfinite(s.e)) break;
+    }
+    col_pairs(a)[((static_cast<int64_t>(b) * gridDim.y + rb) * cols + j) * 3 + 1] =
+        wide ? mark_wide(s) : make_float2(s.s, s.e);
   }
 }
 

@@ -96,6 +96,44 @@ def test_normalize_any_width(rows, cols, n, t, w_dtype):
     opt.close()
 
 
+@pytest.mark.parametrize("tangent", [0, 1, 2])
+@pytest.mark.parametrize("rows,cols,n", [(4096, 264, 1), (1000, 777, 2), (600, 256, 12),
+                                         (512, 20000, 4)])
+def test_normalize_columns_large_momentum(rows, cols, n, tangent):
+    """Entries of 1.5e18: the sum of a row lane stays in the range of fp32 (at most
+    32 rows), that of a column does not.  Psi per column against fp64 at 1e-5 (fp32
+    sums), through a step and through the allocation-free entry point."""
+    import torch
+    from paper_2609_36692_gb300 import normpre as C
+    from paper_2609_36692_gb300.optim import NormPre
+    gen = torch.Generator(device="cuda").manual_seed(rows + n)
+    draw = lambda f: [torch.randn(rows, cols, device="cuda", generator=gen) * f for _ in range(n)]  # noqa: E731
+    W, G, M0 = draw(0.02), [g.bfloat16() for g in draw(1.5e18)], draw(1e17)
+    M = [x.clone() for x in M0]
+    opt = NormPre([(rows, cols)] * n, ["f32"] * n, ["bf16"] * n, variant=C.NORMPRE_L, precision=1, rank=4,
+                  oversample=4, tangent=tangent)
+    x64 = []
+    for i in range(n):
+        m, w = M0[i].double() * f32(0.95) + G[i].double(), W[i].double()
+        assert m.square().sum(0).min() > torch.finfo(torch.float32).max
+        a = (m * w).sum(0)
+        a = a if tangent == 0 else a / w.square().sum(0) if tangent == 2 else 0 * a
+        x64.append(m - a * w)
+    if tangent == 0:      # the entry point without a handle; its W is not updated
+        m, psi = M0[0].clone(), torch.empty_like(M0[0])
+        C.normpre_normalize_cols_noalloc(rows, cols, 0.95, G[0].data_ptr(), C.NORMPRE_BF16, m.data_ptr(),
+                                         W[0].data_ptr(), C.NORMPRE_F32, psi.data_ptr(),
+                                         torch.cuda.current_stream().cuda_stream)
+        assert max_row_rel(to_host(psi).T, (x64[0] / x64[0].norm(dim=0)).T.cpu().numpy()) <= 1e-5
+    opt.step(1, 0.02, W, G, M)
+    assert opt.status() == C.NORMPRE_OK
+    for i in range(n):
+        psi = opt.read(i, C.NORMPRE_BUF_PSI).astype(np.float64)
+        assert max_row_rel(psi.T, (x64[i] / x64[i].norm(dim=0)).T.cpu().numpy()) <= 1e-5
+        assert int(opt.read(i, C.NORMPRE_BUF_STATS)[0][1]) == cols
+    opt.close()
+
+
 @pytest.mark.parametrize("w_dtype", ["f32", "bf16"])
 @pytest.mark.parametrize("rows,cols", [(1, 5), (37, 1), (9, 255), (50, 2049), (300, 257)])
 def test_update_g_any_width(rows, cols, w_dtype):
