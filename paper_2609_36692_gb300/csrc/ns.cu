@@ -841,33 +841,40 @@ static NSGroupBuf ns_geometry(bool bf16, const NSGroupSpec& sp) {
 
 // N tiles of the products: 256 columns, or 128 or 64 while a product would
 // have fewer tiles than two thirds of the SMs (and 128 where 256 does not
-// divide N).  A tile's time is a fixed 8 us and its share of the MMAs and the
-// epilogue, so few wide tiles leave the chip idle: one 256 x 1024 matrix is
-// two tiles of 256 columns in the Gram product and 8 in the update, or 6 and
-// 32 of 64.
+// divide N) and the narrower tiles still come to the SMs in one wave.  A tile's
+// time is a fixed 8 us and its share of the MMAs and the epilogue, so few wide
+// tiles leave the chip idle: one 256 x 1024 matrix is two tiles of 256 columns
+// in the Gram product and 8 in the update, or 6 and 32 of 64.  A second wave
+// undoes it, most of all where it doubles up long tiles: 24 matrices with 128
+// rows on the short side beside one of 1379 x 19636 are 90 Gram tiles of 128
+// columns or 180 of 64 (the step 1595 us and 1930), 90 of 128 x 4096 the same
+// (662 and 755).
 static void ns_tiles(bool bf16, std::vector<NSGroupBuf>& groups, int num_sms) {
   auto fit = [](int bn, int64_t n) { return bn > 128 && n % bn != 0 ? 128 : bn; };
   auto gram = [&](const NSGroupBuf& g, int bn) { return fit(bn, g.s_pad); };
   auto upd = [&](const NSGroupBuf& g, int bn) { return fit(bn, g.tall ? g.s_pad : g.big_pad); };
-  int bg = 256, bu = 256;
-  if (!bf16) bg = bu = 64;
-  for (; bg > 64; bg /= 2) {
+  auto gram_tiles = [&](int b) {
     int64_t n = 0;
     for (const NSGroupBuf& g : groups) {
-      const int bn = gram(g, bg);
+      const int bn = gram(g, b);
       n += static_cast<int64_t>(g.spec.batch) *
            tiles_per_matrix(static_cast<int>(g.s_pad / 128), static_cast<int>(g.s_pad / bn), bn, 1);
     }
-    if (3 * n >= 2 * num_sms) break;
-  }
-  for (; bu > 64; bu /= 2) {
+    return n;
+  };
+  auto upd_tiles = [&](int b) {
     int64_t n = 0;
     for (const NSGroupBuf& g : groups) {
       const int64_t um = g.tall ? g.big_pad : g.s_pad, un = g.tall ? g.s_pad : g.big_pad;
-      n += static_cast<int64_t>(g.spec.batch) * (um / 128) * (un / upd(g, bu));
+      n += static_cast<int64_t>(g.spec.batch) * (um / 128) * (un / upd(g, b));
     }
-    if (3 * n >= 2 * num_sms) break;
-  }
+    return n;
+  };
+  auto narrow = [&](int bn, auto& tiles) {
+    while (bn > 64 && 3 * tiles(bn) < 2 * num_sms && tiles(bn / 2) <= num_sms) bn /= 2;
+    return bn;
+  };
+  const int bg = bf16 ? narrow(256, gram_tiles) : 64, bu = bf16 ? narrow(256, upd_tiles) : 64;
   for (NSGroupBuf& g : groups) {
     g.bn_gram = bf16 ? gram(g, bg) : 64;
     g.bn_upd = bf16 ? upd(g, bu) : 64;

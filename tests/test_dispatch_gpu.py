@@ -16,11 +16,13 @@ pytestmark = pytest.mark.gpu
 # large and small inputs, the caller's workspace
 # ---------------------------------------------------------------------------
 @pytest.mark.parametrize("precision", [0, 1])
-@pytest.mark.parametrize("shape", [(2, 256, 512), (1, 255, 513), (3, 40, 1000), (1, 512, 256), (2, 128, 131)])
+@pytest.mark.parametrize("shape", [(2, 256, 512), (1, 255, 513), (3, 40, 1000), (1, 512, 256), (2, 128, 131),
+                                   (2, 3, 5)])
 def test_newton_schulz_input_scale(shape, precision):
     """The prescale through the copying and the direct path, below 1e-15 (where
-    the norm is summed in fp64) and far above one, and with the result over the
-    input: with eps = 0 the iteration only sees X / ||X||, and a power of two
+    the norm is summed in fp64) and far above one (3 x 5: past 1e18, in fp64 too;
+    the Gram matrix of larger ones would leave the range of fp32 there), and with
+    the result over the input: with eps = 0 the iteration only sees X / ||X||, and a power of two
     changes no rounding, so the results are equal bit for bit; and the norm
     itself through one step of X <- 1 X (T = X / ||X|| to one rounding)."""
     import torch
@@ -30,7 +32,7 @@ def test_newton_schulz_input_scale(shape, precision):
     x = torch.from_numpy(rng.standard_normal(shape).astype(np.float32)).cuda()
     x = x.to(torch.bfloat16) if precision == 0 else x
     T = newton_schulz(x, precision=precision, ns_eps=0.0)
-    for scale in (2.0 ** -53, 2.0 ** 53):
+    for scale in (2.0 ** -53, 2.0 ** 53 if shape[2] > 5 else 2.0 ** 60):
         assert torch.equal(newton_schulz(x * scale, precision=precision, ns_eps=0.0), T)
     # T over X
     y = x.clone()
@@ -42,6 +44,33 @@ def test_newton_schulz_input_scale(shape, precision):
     X = to_host(x).astype(np.float64)
     ref = X / np.sqrt((X * X).sum(axis=(1, 2), keepdims=True))
     assert np.all(np.abs(u - ref) <= (2.0 ** -8 if precision == 0 else 2.0 ** -22) * np.abs(ref))
+
+
+# Widths of the tiles of the Gram product and of the update at 152 SMs: 128 and 256;
+# 64 and 128 (the update on two-CTA clusters); 64 and 256 (80 tiles, which narrower
+# ones would bring to two waves); 128 and 256, the tall ones 128 and 128; 64 and 64
+@pytest.mark.parametrize("shape", [(4, 1024, 4096), (4, 4096, 1024), (1, 1024, 2048), (1, 2048, 1024), (1, 1280, 2048),
+                                   (1, 2048, 1280), (90, 128, 256), (90, 256, 128), (1, 384, 640)])
+@pytest.mark.parametrize("coef,steps", [((0.0, 1.0, 0.0), 1), ((0.0, 0.0, 1.0), 1), ((3.4445, -4.7750, 2.0315), 5)])
+def test_newton_schulz_tile_widths(shape, coef, steps):
+    """Every product against fp64 at the tile widths that the small shapes and
+    the model sets do not take.  One step rounds to bf16 at most three times, a
+    2^-9 each; a lost or misplaced tile is some hundredths of the whole."""
+    import torch
+    from paper_2609_36692_gb300.optim import newton_schulz
+    gen = torch.Generator(device="cuda").manual_seed(sum(shape))
+    x = torch.randn(shape, device="cuda", generator=gen).bfloat16()
+    T = newton_schulz(x, ns_steps=steps, ns_coef=coef).double()
+    ref = x.double()
+    ref = ref.mT if shape[1] > shape[2] else ref
+    ref = ref / (ref.flatten(1).norm(dim=1)[:, None, None] + f32(1e-7))
+    a, b, c = (f32(v) for v in coef)
+    for _ in range(steps):
+        gram = ref @ ref.mT
+        ref = a * ref + (b * gram + c * (gram @ gram)) @ ref
+    ref = ref.mT if shape[1] > shape[2] else ref
+    err = (T - ref).flatten(1).norm(dim=1) / ref.flatten(1).norm(dim=1)
+    assert err.max() <= (3 * 2.0 ** -9 if steps == 1 else 2e-2), err
 
 
 def test_newton_schulz_workspace():
