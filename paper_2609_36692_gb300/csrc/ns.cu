@@ -116,6 +116,7 @@ struct GemmArgs {
   GemmGroup g[kMaxGroups];
   int n_groups;
   int total_tiles;
+  int trigger_early;      // fp32: see simt_overlap
   int* flags;
 };
 static_assert(sizeof(GemmArgs) + 64 <= 4096, "kernel arguments beyond 4 KB");
@@ -559,7 +560,6 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_ns_gemm_tc(const __grid_const
 template <typename T>
 __global__ void __launch_bounds__(256) k_ns_gemm_simt(const __grid_constant__ GemmArgs args) {
   pdl_wait();
-  pdl_trigger();
   __shared__ float As[16][64];
   __shared__ float Bs[16][64];
   __shared__ float red[8];
@@ -568,6 +568,7 @@ __global__ void __launch_bounds__(256) k_ns_gemm_simt(const __grid_constant__ Ge
   const int tid = threadIdx.x;
   const int ty = tid >> 4, tx = tid & 15;
   const int m0 = tm * 64, n0 = tn * 64;
+  if (args.trigger_early) pdl_trigger();
   const T* Ab = static_cast<const T*>(g.Abuf) + b * g.a_bs;
   const T* Bb = static_cast<const T*>(g.Bbuf) + b * g.b_bs;
   float acc[4][4] = {};
@@ -598,6 +599,7 @@ __global__ void __launch_bounds__(256) k_ns_gemm_simt(const __grid_constant__ Ge
     }
     __syncthreads();
   }
+  pdl_trigger();   // not before: simt_overlap
   float s = 1.f;
   if (g.scale_pow) {
     const float v = g.inscale[b];
@@ -1082,6 +1084,25 @@ static bool select_groups(GemmArgs& a, int g0, int cnt, int m0, int m1) {
   return (t0 & 1) == 0 && (t1 & 1) == 0;
 }
 
+// Whether an fp32 product is launched dependent on the kernel before it, one of
+// `prev` CTAs.  Dependent CTAs come to the SMs as room falls free, several to
+// one SM while others get none.  With the trigger at the kernel's head a step
+// of 8 x 300 x 1000 took 2350 us, 1770 with plain launches, 1745 with the trigger
+// behind the K loop; and there too a launch that does not fill the SMs, or a
+// smaller one behind a larger, loses by it when its tiles are long (4 x 100 x
+// 3000: 2470 us, 2410 plain).  Short tiles, and launches that find idle SMs, gain
+// the launch itself: 64 x 64 175 us, 205 plain.  Where every product of the step
+// is short (K <= 128) the trigger stays at the head: 8 x 128 x 128 328 us, 345
+// behind the loop, 368 plain.
+static int longest_k(const GemmArgs& a) {
+  int k = 0;
+  for (int gi = 0; gi < a.n_groups; ++gi) k = std::max(k, a.g[gi].K);
+  return k;
+}
+static bool simt_overlap(const GemmArgs& a, int prev, int num_sms) {
+  return longest_k(a) <= 256 || prev + a.total_tiles <= num_sms || (a.total_tiles >= num_sms && prev <= a.total_tiles);
+}
+
 cudaError_t NSPlan::run(int steps, const float coef[3], cudaStream_t s, int* flags, ProfileHook* prof, int g0,
                         int cnt, int m0, int m1) {
   ProfileHook none;
@@ -1095,6 +1116,8 @@ cudaError_t NSPlan::run(int steps, const float coef[3], cudaStream_t s, int* fla
   if (m1 < 0) m1 = batch0;
   if (m0 < 0 || m0 >= m1 || m1 > batch0 || (cnt > 1 && (m0 != 0 || m1 != batch0))) return cudaErrorInvalidValue;
   const float a = coef[0], b = coef[1], c = coef[2];
+  int before = 0;               // fp32: CTAs of the kernel before (the prescale's few at first)
+  bool early = false;
   for (int it = 0; it < steps; ++it) {
     const int in = (it == 0) ? 0 : ((it % 2 == 1) ? 1 : 2);
     const int out = (it % 2 == 0) ? 1 : 2;
@@ -1127,6 +1150,8 @@ cudaError_t NSPlan::run(int steps, const float coef[3], cudaStream_t s, int* fla
     const int cls[3] = {kProfNsGram, kProfNsPoly, kProfNsUpdate};
     for (int p = 0; p < 3; ++p) {
       const bool units = select_groups(*ph[p], g0, cnt, m0, m1);
+      if (p == 0) early = longest_k(*ph[p]) <= 128;   // the Gram product has the longest K
+      ph[p]->trigger_early = early;
       prof->begin(cls[p], s);
       if (bf16_) {
         if (L->mc[p] && units) {
@@ -1140,7 +1165,9 @@ cudaError_t NSPlan::run(int steps, const float coef[3], cudaStream_t s, int* fla
           launch_pdl(true, k_ns_gemm_tc<false>, dim3(grid), dim3(kTcThreads), kTcSmem, s, *ph[p]);
         }
       } else {
-        launch_pdl(true, k_ns_gemm_simt<float>, dim3(ph[p]->total_tiles), dim3(256), 0, s, *ph[p]);
+        launch_pdl(simt_overlap(*ph[p], before, num_sms_), k_ns_gemm_simt<float>, dim3(ph[p]->total_tiles), dim3(256),
+                   0, s, *ph[p]);
+        before = ph[p]->total_tiles;
       }
       cudaError_t e = cudaGetLastError();
       if (e != cudaSuccess) return e;
