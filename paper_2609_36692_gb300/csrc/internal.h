@@ -312,7 +312,6 @@ struct SketchGroup {
   // 64 x 64) against the bf16 hi / lo split of V in vb [batch][vb_bs]
   bool psi_bf16 = false;
   CUtensorMap psi_map_bf;       // box 64 x 64 (contractions)
-  CUtensorMap psi_map_apply;    // box 64 x 32 (apply)
   void* vb = nullptr;
   int64_t vb_bs = 0;
 };
@@ -368,8 +367,7 @@ struct ContractBf16Launch {
   int stall_first_copy;
   bool overlap;            // launch_pdl behind the kernel before
 };
-bool contract_bf16_map(CUtensorMap* map, const void* psi, int64_t rows, int64_t cols, int64_t ld, int batch,
-                       int box_rows = 64);
+bool contract_bf16_map(CUtensorMap* map, const void* psi, int64_t rows, int64_t cols, int64_t ld, int batch);
 cudaError_t launch_contract_bf16(const ContractBf16Launch& c, cudaStream_t s);
 
 // Records the message returned by normpre_last_error(NULL) on this thread.

@@ -2588,8 +2588,7 @@ cudaError_t sketch_group_alloc(SketchGroup& g, int rank, int oversample, std::ve
   // where the bf16 contraction applies (l <= 64, 16-byte Psi rows)
   if (g.psi_bf16) {
     g.vb_bs = 2 * round_up(g.lmax, 16) * round_up(big, 64);
-    g.psi_bf16 = g.lmax <= 64 && contract_bf16_map(&g.psi_map_bf, g.psi, g.rows, g.cols, g.ld, g.batch) &&
-                 contract_bf16_map(&g.psi_map_apply, g.psi, g.rows, g.cols, g.ld, g.batch, 32);
+    g.psi_bf16 = g.lmax <= 64 && contract_bf16_map(&g.psi_map_bf, g.psi, g.rows, g.cols, g.ld, g.batch);
     if (g.psi_bf16 && (e = alloc(&g.vb, static_cast<size_t>(g.batch) * g.vb_bs * sizeof(uint16_t)))) return e;
   }
   // the largest Jacobi footprint, so that groups of any width can share the kernel
@@ -2609,9 +2608,7 @@ cudaError_t sketch_group_slice(const SketchGroup& g, int b0, int b1, SketchGroup
                      : g.psi + b0 * g.rows * g.ld;
   if (g.psi_bf16) {
     s.vb = static_cast<uint16_t*>(g.vb) + b0 * g.vb_bs;
-    if (!contract_bf16_map(&s.psi_map_bf, s.psi, g.rows, g.cols, g.ld, s.batch) ||
-        !contract_bf16_map(&s.psi_map_apply, s.psi, g.rows, g.cols, g.ld, s.batch, 32))
-      return cudaErrorInvalidValue;
+    if (!contract_bf16_map(&s.psi_map_bf, s.psi, g.rows, g.cols, g.ld, s.batch)) return cudaErrorInvalidValue;
   }
   float** vbufs[] = {&s.omega, &s.y0, &s.zt, &s.y, &s.q, &s.bt, &s.qk};
   for (float** v : vbufs) *v += b0 * vbs;

@@ -54,8 +54,8 @@ def test_newton_schulz_input_scale(shape, precision):
 @pytest.mark.parametrize("coef,steps", [((0.0, 1.0, 0.0), 1), ((0.0, 0.0, 1.0), 1), ((3.4445, -4.7750, 2.0315), 5)])
 def test_newton_schulz_tile_widths(shape, coef, steps):
     """Every product against fp64 at the tile widths that the small shapes and
-    the model sets do not take.  One step rounds to bf16 at most three times, a
-    2^-9 each; a lost or misplaced tile is some hundredths of the whole."""
+    the model sets do not take.  One step rounds to bf16 at most three times, at
+    2^-9 each in the norm; a lost or misplaced tile is some hundredths of the whole."""
     import torch
     from paper_2609_36692_gb300.optim import newton_schulz
     gen = torch.Generator(device="cuda").manual_seed(sum(shape))
@@ -242,11 +242,12 @@ def test_sketch_basis_and_ritz_pairs(rows, cols, rank, oversample, t):
                                               (37, 1300, 30, 32), (641, 2, 31, 16), (256, 770, 33, 64),
                                               (1, 1290, 30, 4)])
 def test_apply_two_columns_a_lane(rows, cols, n, rank, t, w_dtype, precision):
-    """W_new against cw W + ct (Psi + Q K Q^T Psi) formed in fp64 from the step's
-    own Psi, Q and Ritz pairs, cw and ct fitted.  W_new is rounded to bf16, 2^-9 of
-    it; Q, the Ritz pairs and the panels are fp32, 2e-5 each of the largest entry
-    (as the basis test above), and the panels' largest singular value may be some
-    tens of an entry's size: 1e-3 of the largest."""
+    """W_new against cw W + ct (Psi + D), D = Q K Q^T Psi, formed in fp64 from the
+    step's own Psi, Q, Ritz pairs and ||T||^2.  D within 2^-14 of its largest entry:
+    the panels are fp32 (a bf16 Psi is contracted with a two-term split, 2^-16), the
+    product a three-product split, 2^-20; a split without one of its lo terms, cut
+    off at 2^-10, is out by 2^-11.  W_new is rounded to bf16, half a spacing (2^-8 of
+    it at most), or to fp32."""
     import torch
     from paper_2609_36692_gb300 import normpre as C
     from paper_2609_36692_gb300.optim import NormPre
@@ -266,13 +267,18 @@ def test_apply_two_columns_a_lane(rows, cols, n, rank, t, w_dtype, precision):
         Q = opt.read(i, C.NORMPRE_BUF_Q).astype(np.float64)
         Z = opt.read(i, C.NORMPRE_BUF_Z).astype(np.float64)
         lam = opt.read(i, C.NORMPRE_BUF_RITZ)[0].astype(np.float64)
+        nrm2 = float(opt.read(i, C.NORMPRE_BUF_STATS)[0][2])
         gain = 1.0 / np.sqrt(np.maximum(lam, 1.0)) - 1.0     # of the values above one
-        T = pa + Q @ ((Z * gain) @ (Z.T @ (Q.T @ pa)))
-        T = T if t == 0 else T.T
+        D = Q @ ((Z * gain) @ (Z.T @ (Q.T @ pa)))
+        D = D if t == 0 else D.T
         w0, w1 = (x[i].double().cpu().numpy() for x in (W0, W))
-        X = np.stack([w0.ravel(), T.ravel()], 1)
-        fit = (X @ np.linalg.lstsq(X, w1.ravel(), rcond=None)[0]).reshape(rows, cols)
-        assert np.all(np.abs(w1 - fit) <= 2.0 ** -8 * np.abs(w1) + 1e-3 * np.abs(w1).max()), (i, np.abs(w1 - fit).max())
+        ct = 0.5 * f32(0.2) * np.sqrt(rows * cols / nrm2)
+        ref = (1.0 - 0.5 * f32(0.1)) * w0 - ct * (psi + D)
+        size = np.abs(w0) + ct * (np.abs(psi) + np.abs(D))
+        tol = 2.0 ** -14 * ct * np.abs(D).max() + 2.0 ** -21 * size
+        if w_dtype == "bf16":
+            tol = tol + 2.0 ** -8 * (np.abs(ref) + tol)
+        assert np.all(np.abs(w1 - ref) <= tol), (i, (np.abs(w1 - ref) / tol).max())
     opt.close()
 
 
@@ -306,3 +312,34 @@ def test_nonfinite_gradient_is_reported(variant, precision, rank, value):
         opt.close()
     for a, b in zip(out[:2], out[2:]):
         assert all(torch.equal(x, y) for x, y in zip(a, b))
+
+
+# ---------------------------------------------------------------------------
+# stream capture: the dependent launches of a step as edges of a graph
+# ---------------------------------------------------------------------------
+@pytest.mark.parametrize("variant,precision", [(0, 0), (0, 1), (1, 1), (1, 0), (2, 0)])
+@pytest.mark.parametrize("shapes", [[(256, 512)], [(256, 512), (300, 77), (512, 256), (256, 512), (40, 1100)]])
+def test_captured_step_equals_eager(shapes, variant, precision):
+    """A captured pair of steps, replayed twice, updates W and M as the same four
+    steps launched one by one, bit for bit."""
+    import torch
+    from paper_2609_36692_gb300.optim import NormPre
+    gen = torch.Generator(device="cuda").manual_seed(9)
+    draw = lambda f: [torch.randn(s, device="cuda", generator=gen) * f for s in shapes]  # noqa: E731
+    W, G, M = draw(0.02), [g.bfloat16() for g in draw(1.0)], draw(1.0)
+    W2, M2 = [w.clone() for w in W], [m.clone() for m in M]
+    eager, captured = (NormPre.for_tensors(W, G, variant=variant, precision=precision, rank=16) for _ in range(2))
+    for t in (0, 1, 0, 1):
+        eager.step(t, 0.02, W, G, M)
+    graph = torch.cuda.CUDAGraph()
+    torch.cuda.synchronize()
+    with torch.cuda.graph(graph):
+        for t in (0, 1):
+            captured.step(t, 0.02, W2, G, M2)
+    graph.replay()
+    graph.replay()
+    torch.cuda.synchronize()
+    assert eager.status() == 0 and captured.status() == 0
+    assert all(torch.equal(a, b) for a, b in zip(W + M, W2 + M2))
+    eager.close()
+    captured.close()
