@@ -49,20 +49,6 @@ LR = 0.02
 FP32_FMA_TFLOPS = 152 * 128 * 2 * 2.07e9 / 1e12   # 80.5 TFLOP/s, for the fp32 exact-variant sweeps
 L2_BYTES = 129e6                                    # GB300 L2
 
-# Traffic of one launch of the dominant kernel class from an ncu capture
-# (dram__bytes_read.sum + dram__bytes_write.sum), per workload and variant;
-# absent until a capture of the current kernel exists (profiles/ keeps the
-# summaries).
-NCU_TRAFFIC_PER_LAUNCH = {
-    # dram__bytes_read.sum + dram__bytes_write.sum per launch of the roofline
-    # kernel class, from one ncu capture of the timed steps (profiles/launches_*.md)
-    ("gpt2_small_G", "G"): 207.8e6,      # mean of 45 launches: Gram, poly and update of five NS iterations, 3 steps
-    ("qwen3_1p7b", "G"): 4513e6,         # the same on the Qwen3 set
-    ("qwen3_1p7b", "L", "normalize"): 1.687e9,   # a row-active and a column-active step over their 28 launches
-    ("gpt2_small_L", "L", "contract"): 56.0e6,   # 78 launches: contractions and split-K reductions, 3 steps
-}
-
-
 # ---------------------------------------------------------------------------
 # helpers
 # ---------------------------------------------------------------------------
@@ -84,11 +70,22 @@ def ns_flops(cfg: S.ParamSetConfig, steps: int) -> float:
     return tot
 
 
+def ns_moved_bytes(cfg: S.ParamSetConfig) -> float:
+    """Bytes that the three products of an iteration read and write in bf16, each
+    operand once: X in, A out; A in, C out; C and X in, X out."""
+    tot = 0.0
+    for m in cfg.matrices:
+        s, n = min(m.rows, m.cols), m.rows * m.cols
+        tot += 2.0 * (3 * n + 4 * s * s)
+    return tot
+
+
 def ns_executed_flops(cfg: S.ParamSetConfig, steps: int) -> float:
     """Flops the tensor-core path executes in one step.  Dimensions are padded
     (the short side s to 128, the long side to 256), the Gram and polynomial
     products compute only the 128 x BN tiles that reach the diagonal (BN = 256
-    when the padded s is a multiple of 256, else 128) and mirror the rest."""
+    when the padded s is a multiple of 256, else 128; the narrower tiles of sets
+    too small to fill the SMs execute a little less) and mirror the rest."""
     def up(x, m):
         return (x + m - 1) // m * m
     tot = 0.0
@@ -303,7 +300,8 @@ def _roofline(cfg, variant, prof, steps, clocks, exact_sweeps=None):
                 "nominal_flops_per_launch": fl / ns_launches,
                 "achieved_nominal": fl / (ns_ms * 1e-3) / 1e12,
                 "frac_nominal": fl / (ns_ms * 1e-3) / 1e12 / peak,
-                "traffic": NCU_TRAFFIC_PER_LAUNCH.get((cfg.name, variant))}
+                "traffic": ns_moved_bytes(cfg) / 3,
+                "traffic_note": "counted from the launch's operands, each read or written once"}
     if variant == "L_exact":
         # the one-sided block Jacobi sweeps over Psi on the fp32 FMA pipes: per
         # sweep of a matrix, (nb - 1) rounds of nb / 2 column-block pairs, each
@@ -348,6 +346,9 @@ def _roofline(cfg, variant, prof, steps, clocks, exact_sweeps=None):
         # Psi and W read, W written
         "apply_l": (n_el * b_apply, "k_apply_tc (Psi + Lm Rm^T and the weight update, tcgen05 TF32 split)"),
     }
+    # what they move: a column-active step's second pass reads M and W again
+    moved = {name: nbytes for name, (nbytes, _) in classes.items()}
+    moved["normalize"] += n_el * (4 + (2 if cfg.w_dtype == "bf16" else 4)) / 2.0
     kern = {}
     for name, (nbytes, label) in classes.items():
         ms = prof[name][0] / steps
@@ -364,7 +365,8 @@ def _roofline(cfg, variant, prof, steps, clocks, exact_sweeps=None):
             "peak_source": "%s HBM copy bandwidth" % peak_src,
             "bytes_per_launch": d["bytes_per_launch"], "ms_per_launch": d["ms_per_launch"],
             "launches_per_step": d["launches_per_step"],
-            "traffic": NCU_TRAFFIC_PER_LAUNCH.get((cfg.name, variant, top)),
+            "traffic": moved[top] / d["launches_per_step"],
+            "traffic_note": "counted from what the launches read and write, steps of both orientations",
             "classes": {k: {kk: v for kk, v in x.items() if kk != "kernel"} for k, x in kern.items()}}
 
 

@@ -362,35 +362,59 @@ __global__ void __launch_bounds__(kColThreads) k_norm_cols_stats(const __grid_co
 // stage 1 (strict): a_j = <m_j, w_j> / ||w_j||^2 only.
 // stage 2 (strict): ||x_j||^2 from the direct sums of k_norm_cols_xsq (slot 1),
 // ||m_j||^2 from pass A (slot 0), a_j kept.
-// One warp per 32 columns: the few fp64 operations of a column spread over all
-// SMs.
-__global__ void __launch_bounds__(32) k_norm_cols_final(const __grid_constant__ NormLaunch a, int nrb, int stage) {
+// 32 columns per CTA (the few fp64 operations of a column spread over all SMs):
+// one warp, or past four row blocks eight that take every eighth, since a thread
+// walking a column's blocks alone waits for the loads.  65536 x 8, a step of
+// NormPre-L: 450 us with eight, 505 with one (1024 blocks); 2048 x 2048, two
+// matrices: 332 and 338 (64 blocks); 256 x 1024 228.6 and 229.7 (8)
+constexpr int kColFinalWarps = 8, kColFinalOne = 4;   // warps, past as many row blocks
+template <int NW>
+__global__ void __launch_bounds__(32 * NW) k_norm_cols_final(const __grid_constant__ NormLaunch a, int nrb, int stage) {
   pdl_wait();
   pdl_trigger();
-  const int b = blockIdx.y;
+  __shared__ float2 part[NW][3][32];
+  __shared__ bool part_wide[NW][32];
+  const int b = blockIdx.y, lane = threadIdx.x, y = threadIdx.y;
   const int64_t cols = a.cols;
-  const int64_t j = static_cast<int64_t>(blockIdx.x) * 32 + threadIdx.x;
-  float nz = 0.f;
+  const int64_t j = static_cast<int64_t>(blockIdx.x) * 32 + lane;
+  const float2* sums = col_pairs(a) + (static_cast<int64_t>(b) * nrb * cols + j) * 3;
+  PairSum p0, p1, p2;
+  bool wide = false;
   if (j < cols) {
-    PairSum p0, p1, p2;
-    const float2* p = col_pairs(a) + (static_cast<int64_t>(b) * nrb * cols + j) * 3;
-    bool wide = false;
+    const float2* p = sums + y * cols * 3;
 #pragma unroll 8
-    for (int rb = 0; rb < nrb; ++rb) {
+    for (int rb = y; rb < nrb; rb += NW) {
       const float2 v0 = p[0], v1 = p[1], v2 = p[2];
       wide |= is_wide(v2) || (stage == 2 && is_wide(v1));
       p0.add(PairSum{v0.x, v0.y}); p1.add(PairSum{v1.x, v1.y}); p2.add(PairSum{v2.x, v2.y});
-      p += cols * 3;
+      p += NW * cols * 3;
     }
+  }
+  if constexpr (NW > 1) {
+    part[y][0][lane] = make_float2(p0.s, p0.e);
+    part[y][1][lane] = make_float2(p1.s, p1.e);
+    part[y][2][lane] = make_float2(p2.s, p2.e);
+    part_wide[y][lane] = wide;
+    __syncthreads();
+    if (y > 0) return;
+#pragma unroll
+    for (int w = 1; w < NW; ++w) {
+      const float2 v0 = part[w][0][lane], v1 = part[w][1][lane], v2 = part[w][2][lane];
+      wide |= part_wide[w][lane];
+      p0.add(PairSum{v0.x, v0.y}); p1.add(PairSum{v1.x, v1.y}); p2.add(PairSum{v2.x, v2.y});
+    }
+  }
+  float nz = 0.f;
+  if (j < cols) {
     double s0, s1, s2;
     if (!wide && isfinite(p0.e + p1.e + p2.e)) {
       s0 = p0.value(); s1 = p1.value(); s2 = p2.value();
     } else {
       // stage 2: slot 1 has a mark of its own (k_norm_cols_xsq)
       s0 = s1 = s2 = 0;
+      const float2* p = sums;
 #pragma unroll 1
-      for (int rb = 0; rb < nrb; ++rb) {
-        p -= cols * 3;
+      for (int rb = 0; rb < nrb; ++rb, p += cols * 3) {
         const float2 v0 = p[0], v1 = p[1], v2 = p[2];
         const bool w2 = is_wide(v2);
         s0 += wide_value(v0.x, v0.y, w2);
@@ -421,7 +445,7 @@ __global__ void __launch_bounds__(32) k_norm_cols_final(const __grid_constant__ 
     }
   }
   nz = warp_sum(nz);
-  if (threadIdx.x == 0 && nz > 0.f) atomicAdd(&a.count[a.mat_id[b]], static_cast<int>(nz));
+  if (lane == 0 && nz > 0.f) atomicAdd(&a.count[a.mat_id[b]], static_cast<int>(nz));
 }
 
 // strict tangent, column-active: ||x_j||^2 of this block's rows summed from
@@ -663,6 +687,11 @@ cudaError_t launch_normalize_cols(const NormLaunch& a, cudaStream_t s) {
   const int nrb = static_cast<int>(cdiv(a.rows, a.col_rb));
   const dim3 grid(static_cast<unsigned>(cdiv(a.cols, 256)), static_cast<unsigned>(nrb),
                   static_cast<unsigned>(a.n));
+  auto fold = [&](bool overlap, int stage) {
+    const dim3 fgrid(static_cast<unsigned>(cdiv(a.cols, 32)), a.n);
+    if (nrb > kColFinalOne) launch_pdl(overlap, k_norm_cols_final<kColFinalWarps>, fgrid, dim3(32, kColFinalWarps), 0, s, a, nrb, stage);
+    else launch_pdl(overlap, k_norm_cols_final<1>, fgrid, dim3(32), 0, s, a, nrb, stage);
+  };
   const int rb_b = grid.x * cdiv(a.rows, kColApplyRB) * a.n < 4 * static_cast<int64_t>(device_sm_count()) ? 16 : kColApplyRB;
   const dim3 grid_b(grid.x, static_cast<unsigned>(cdiv(a.rows, rb_b)), static_cast<unsigned>(a.n));
   return dispatch3(a.g_dtype, a.w_dtype, a.psi_dtype, [&](auto* tg, auto* tw, auto* tp) {
@@ -675,14 +704,14 @@ cudaError_t launch_normalize_cols(const NormLaunch& a, cudaStream_t s) {
     if (e != cudaSuccess) return e;
     if (a.tangent == 2) {
       // strict: the coefficient first, then ||x_j||^2 summed from x itself
-      launch_pdl(a.overlap_next, k_norm_cols_final, dim3(static_cast<unsigned>(cdiv(a.cols, 32)), a.n), dim3(32), 0, s, a, nrb, 1);
+      fold(a.overlap_next, 1);
       if ((e = cudaGetLastError()) != cudaSuccess) return e;
       if (vec) launch_pdl(a.overlap_next, k_norm_cols_xsq<TW, true>, dim3(grid), dim3(kColThreads), 0, s, a);
       else launch_pdl(a.overlap_next, k_norm_cols_xsq<TW, false>, dim3(grid), dim3(kColThreads), 0, s, a);
       if ((e = cudaGetLastError()) != cudaSuccess) return e;
-      launch_pdl(a.overlap_next, k_norm_cols_final, dim3(static_cast<unsigned>(cdiv(a.cols, 32)), a.n), dim3(32), 0, s, a, nrb, 2);
+      fold(a.overlap_next, 2);
     } else {
-      launch_pdl(a.overlap_next, k_norm_cols_final, dim3(static_cast<unsigned>(cdiv(a.cols, 32)), a.n), dim3(32), 0, s, a, nrb, 0);
+      fold(a.overlap_next, 0);
     }
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
