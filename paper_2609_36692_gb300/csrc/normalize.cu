@@ -366,7 +366,8 @@ __global__ void __launch_bounds__(kColThreads) k_norm_cols_stats(const __grid_co
 // one warp, or past four row blocks eight that take every eighth, since a thread
 // walking a column's blocks alone waits for the loads.  65536 x 8, a step of
 // NormPre-L: 450 us with eight, 505 with one (1024 blocks); 2048 x 2048, two
-// matrices: 332 and 338 (64 blocks); 256 x 1024 228.6 and 229.7 (8)
+// matrices: 332 and 338 (64 blocks); 256 x 1024 228.6 and 229.7 (8).  Launches
+// of more than eight warps per SM fill them with one (Qwen3: 11.5 us, 13 with eight)
 constexpr int kColFinalWarps = 8, kColFinalOne = 4;   // warps, past as many row blocks
 template <int NW>
 __global__ void __launch_bounds__(32 * NW) k_norm_cols_final(const __grid_constant__ NormLaunch a, int nrb, int stage) {
@@ -689,8 +690,10 @@ cudaError_t launch_normalize_cols(const NormLaunch& a, cudaStream_t s) {
                   static_cast<unsigned>(a.n));
   auto fold = [&](bool overlap, int stage) {
     const dim3 fgrid(static_cast<unsigned>(cdiv(a.cols, 32)), a.n);
-    if (nrb > kColFinalOne) launch_pdl(overlap, k_norm_cols_final<kColFinalWarps>, fgrid, dim3(32, kColFinalWarps), 0, s, a, nrb, stage);
-    else launch_pdl(overlap, k_norm_cols_final<1>, fgrid, dim3(32), 0, s, a, nrb, stage);
+    if (nrb > kColFinalOne && static_cast<int64_t>(fgrid.x) * a.n < 8 * static_cast<int64_t>(device_sm_count()))
+      launch_pdl(overlap, k_norm_cols_final<kColFinalWarps>, fgrid, dim3(32, kColFinalWarps), 0, s, a, nrb, stage);
+    else
+      launch_pdl(overlap, k_norm_cols_final<1>, fgrid, dim3(32), 0, s, a, nrb, stage);
   };
   const int rb_b = grid.x * cdiv(a.rows, kColApplyRB) * a.n < 4 * static_cast<int64_t>(device_sm_count()) ? 16 : kColApplyRB;
   const dim3 grid_b(grid.x, static_cast<unsigned>(cdiv(a.rows, rb_b)), static_cast<unsigned>(a.n));
