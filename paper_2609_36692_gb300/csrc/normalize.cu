@@ -37,10 +37,10 @@ namespace normpre {
 constexpr int kColApplyRB = 64;   // rows per block of pass B (16 where that leaves SMs idle)
 constexpr int kColThreads = 256;  // 32 column chunks of 8 x 8 row lanes
 
-// The column sums are fp32 pairs (PairSum): folded in fp64 instead, every listed
-// size of both variants gives the same results bit for bit, 1.6 % later on LLaMA
-// 1B and 2.1 % on Qwen3 (24 additions and conversions per column of a block keep
-// the fp64 pipe busy for 3 us).  The fold has the range of fp64 all the same: a
+// The column sums are fp32 pairs (PairSum).  Folded in fp64 they gave the same
+// steps bit for bit on every set of perf/cases.py and were 1.6 % slower on LLaMA
+// 1B, 2.1 % on Qwen3 (24 additions and conversions per column of a block keep the
+// fp64 pipe busy for 3 us).  The fold has the range of fp64 all the same: a
 // block's sums whose pairs overflow (a column of entries of 1e18 has a squared
 // norm of 1e36 times its rows, though its row lanes stay finite) are kept at
 // 2^-4 of their size, marked by the sign bit of a sum that is never negative,
