@@ -110,12 +110,18 @@ __device__ __forceinline__ void row_store(T* p, int64_t j, int64_t cols, const f
     }
   }
 }
-template <typename TG, typename TW, typename TP, bool VEC>
+// TRIGGER: the next kernel may come early.  Not behind rows of up to 256 columns,
+// where at one CTA a row the trigger costs more than that gains (41 x 9728 rows of
+// 8, a NormPre-G step: 1000 us with it, 865 without, 924 with plain launches; 20 x
+// 2000 x 200 430 and 423; of 400 columns 393 and 398), and not in the element form,
+// where it makes no difference; wider rows do not notice it, and other groups'
+// kernels gain (13 layers of 384 to 2816 columns, two NormPre-L steps: 3110 us, 3125
+// without).  A template parameter, since a branch takes the kernel from 58 to 64
+// registers.
+template <typename TG, typename TW, typename TP, bool VEC, bool TRIGGER>
 __global__ void __launch_bounds__(1024) k_norm_rows(const __grid_constant__ NormLaunch a) {
   pdl_wait();
-  // (no trigger: at one CTA a row it costs more than the next kernel gains by
-  // coming early.  41 x 9728 rows of 8, a NormPre-G step: 1000 us with it, 865
-  // without, 924 with plain launches; from 768 columns on no difference)
+  if constexpr (TRIGGER) pdl_trigger();
   __shared__ float red[32];
   const int b = blockIdx.y;
   const int64_t row = blockIdx.x;
@@ -671,10 +677,12 @@ cudaError_t launch_normalize_rows(const NormLaunch& a, cudaStream_t s) {
     using TW = std::remove_pointer_t<decltype(tw)>;
     using TP = std::remove_pointer_t<decltype(tp)>;
     const int threads = static_cast<int>(round_up(cdiv(a.cols, 16), 32));
-    if (vec) {
-      launch_pdl(a.overlap, k_norm_rows<TG, TW, TP, true>, dim3(grid), dim3(threads), 0, s, a);
+    if (vec && a.cols > 256) {
+      launch_pdl(a.overlap, k_norm_rows<TG, TW, TP, true, true>, dim3(grid), dim3(threads), 0, s, a);
+    } else if (vec) {
+      launch_pdl(a.overlap, k_norm_rows<TG, TW, TP, true, false>, dim3(grid), dim3(threads), 0, s, a);
     } else if (a.cols <= 16 * 1024) {
-      launch_pdl(a.overlap, k_norm_rows<TG, TW, TP, false>, dim3(grid), dim3(threads), 0, s, a);
+      launch_pdl(a.overlap, k_norm_rows<TG, TW, TP, false, false>, dim3(grid), dim3(threads), 0, s, a);
     } else {
       launch_pdl(a.overlap, k_norm_rows_scalar<TG, TW, TP>, dim3(grid), dim3(256), 0, s, a);
     }
